@@ -100,8 +100,13 @@ typedef enum {
  * in use.  The fixed-point grid is 2^-100 of the a-priori bound
  * N max|m| max(0.385 / eps^2, 1 / eps) on every acceleration component and
  * potential; it is finer than FP64 rounding unless that bound exceeds the
- * smallest |a_i| by more than ~10^14.  DEFAULT takes SYMMETRIC for
- * 24576 <= N <= 2^24 and eps > 0 (FP32 and FP64 pairs), DIRECT otherwise.
+ * smallest |a_i| by more than ~10^14.  DEFAULT takes, for eps > 0, SYMMETRIC
+ * for 24576 <= N <= 2^24 (FP32 and FP64 pairs) and, FP32 pairs only, from
+ * N = 4800 unless a launch shape (nb_tune), NB_POS_ADAPTIVE or the
+ * test_unissued_stage hook asks for the direct kernel; DIRECT otherwise.
+ * Where every pair takes the same displacement form (forces below 32768 /
+ * 65536 particles), the totals have 174 instead of 100 bits: 224 B per
+ * particle of every single-system workspace up to 2^24.
  * For batches (B > 1, nb_forces_batched and
  * nb_step with offsets) DEFAULT and SYMMETRIC take the symmetric batched
  * path (warp-granular work items; workspace about 250 B per particle plus
@@ -181,7 +186,7 @@ const char *nb_last_error(void);
  * double patterns (splitmix64 from `seed`), and edge and n random
  * (value, exponent) pairs for the split, are compared with the C
  * conversions (round to nearest even), isfinite and v 2^F rounded half away
- * from zero;
+ * from zero, and sums in four-limb fixed point with 128-bit integers;
  * *mismatches receives the count (0 when they agree).  No device work.
  * NB_ERR_INVALID for a NULL pointer or n < 0.
  */

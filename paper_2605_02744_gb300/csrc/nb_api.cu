@@ -219,6 +219,13 @@ WsLayout ws_layout(int64_t N, int32_t B, const nb_opts *opts) {
     off = align256(off + 2 * (size_t)L.max_grid * (size_t)L.record_bytes_per_i);
     L.scratch = off;
     off = align256(off + kScratchBase + batched_scratch_bytes(B));
+    if (B == 1 && (N <= kSymMaxN ||
+                   (N <= kWsymMaxN && opts && opts->pairs == NB_PAIRS_SYMMETRIC))) {
+        L.wsym_head = off;
+        off = align256(off + 256);
+        L.wsym_fx = off;
+        off = align256(off + 8 * fx::kLimbs * kWsymComponents * (size_t)L.Np);
+    }
     if (sym_wanted(opts, N, B)) {
         const SymSizes z = sym_sizes(L.Np);
         L.sym_fx = off;
@@ -246,10 +253,22 @@ bool bsym_wanted(const nb_opts *o, int64_t N, int32_t B) {
     return o && B > 1 && o->precision != NB_PREC_FP64 && o->pairs != NB_PAIRS_DIRECT;
 }
 
+// A tune that names (part of) a direct-kernel launch shape.
+static bool shape_asked(const nb_opts *o) {
+    const nb_tune *t = o->tune;
+    return t && (t->threads || t->i_per_thread || t->tile_j || t->stages || t->ctas_per_sm);
+}
+
 bool sym_wanted(const nb_opts *o, int64_t N, int32_t B) {
     if (!o || B != 1) return false;
     if (o->pairs == NB_PAIRS_SYMMETRIC) return true;
-    return o->pairs == NB_PAIRS_DEFAULT && N >= kSymMinN && N <= kSymMaxN;
+    if (o->pairs != NB_PAIRS_DEFAULT || N > kSymMaxN) return false;
+    if (N >= kSymMinN) return true;
+    // below kSymMinN what asks for the direct kernel gets it: a launch shape,
+    // the adaptive displacement (its sorted symmetric form needs large
+    // systems), the ring's test hook
+    return o->precision != NB_PREC_FP64 && N >= kWsymMinN && !shape_asked(o) &&
+           o->positions != NB_POS_ADAPTIVE && o->test_unissued_stage == 0;
 }
 
 int check_ws(const void *ws, size_t ws_bytes, const WsLayout &L) {
@@ -487,6 +506,54 @@ int nb_check_fp_conversions(int64_t n, uint64_t seed, int64_t *mismatches) {
         const uint64_t e = (uint64_t)(1023 - F - 60 + (int)((r >> 56) % 170));
         check_split(fpconv::from_bits_d((r & 0x800fffffffffffffull) | ((e & 0x7ff) << 52)), F);
     }
+    // the four-limb form: single values come back exactly wherever nothing is
+    // below the grid, sums of values spread over three limbs as the 128-bit sum
+    // rounded to nearest even
+    auto add_limbs = [&](long long (&w)[fx::kLimbs], float v, int F) {
+        int q;
+        long long lo, hi;
+        if (!fx::split_limbs(v, F, q, lo, hi)) return false;
+        w[q] += lo;
+        if (hi) w[q + 1] += hi;
+        return true;
+    };
+    for (int64_t k = 0; k < n; ++k) {
+        const uint64_t r = next();
+        const float v = fpconv::from_bits_f((uint32_t)r);
+        const int F = (int)((r >> 32) % 331) - 30;
+        long long w[fx::kLimbs] = {};
+        int e = 0;
+        if (std::isfinite(v) && v != 0.f) frexpf(v, &e);  // |v| < 2^e, last bit >= 2^(e - 24)
+        const bool fits = std::isfinite(v) && e + F <= fx::kLimbs * fx::kLimbBits;
+        if (add_limbs(w, v, F) != (fits || v == 0.f)) {
+            ++bad;
+        } else if (fits) {
+            const double got = fx::limb_value(w, F), err = std::fabs(got - (double)v);
+            if (err > (e - 24 + F >= 0 || v == 0.f ? 0.0 : std::ldexp(0.5, -F))) ++bad;
+        }
+        // 16 values of up to 98 bits; half the time nearly cancelling
+        long long x[fx::kLimbs] = {};
+        __int128 sum = 0;
+        const int Fs = (int)(r >> 40) % 60;
+        for (int i = 0; i < 16; ++i) {
+            const uint64_t g = next();
+            const int sh = (int)((g >> 32) % 75);
+            long long m = (long long)(g & 0xffffffu);
+            if (g >> 63) m = -m;
+            if ((r & 1) && i == 15 && sum != 0) {  // the leading 24 bits of -sum
+                __int128 a = sum < 0 ? -sum : sum;
+                int up = 0;
+                while (a >> 24) a >>= 1, ++up;
+                const float c = std::ldexp((float)(long long)a, up - Fs) * (sum < 0 ? 1.f : -1.f);
+                if (!add_limbs(x, c, Fs)) ++bad;
+                sum += (sum < 0 ? a : -a) * ((__int128)1 << up);
+                continue;
+            }
+            if (!add_limbs(x, std::ldexp((float)m, sh - Fs), Fs)) ++bad;
+            sum += (__int128)m * ((__int128)1 << sh);
+        }
+        if (fx::limb_value(x, Fs) != std::ldexp((double)sum, -Fs)) ++bad;
+    }
     *mismatches = bad;
     return NB_OK;
 }
@@ -672,6 +739,10 @@ static int step_single_direct(nb_state *s, double dt, int64_t nsteps, const nb_o
     ForceJob j;
     NB_TRY(make_force_job(&j, s->pos, s->mass, s->N, s->eps, s->acc, s->pot, s->ws, s->ws_bytes, o));
     j.adaptive = positions_adaptive(o, s->N, nsteps > 0);
+    if (takes_wsym(j)) {
+        if (nsteps == 0 && s->acc_valid) return NB_OK;
+        return launch_step_wsym(j, s->vel, dt, nsteps, s->acc_valid != 0);
+    }
     int64_t sorted_at = -1;  // step index of the last full Hilbert sort
     // the potential is evaluated only where the caller can see it: a
     // forces-only call (nsteps = 0) or the last step of the loop

@@ -78,6 +78,18 @@ __device__ __forceinline__ void bulk_g2s(void *dst, const void *src, uint32_t by
         : "memory");
 }
 
+// Programmatic dependent launch (launch_pdl): grid_wait() holds a kernel that
+// was started early until the kernels before it on its stream are done and
+// their writes visible; every kernel launched that way calls it before its
+// first access to memory that another kernel touches, and reads such memory
+// with ordinary loads (the read-only path may hold lines from before the
+// wait).  grid_trigger() lets
+// the next kernel's blocks be placed as soon as there is room for them.
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void grid_trigger() {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 __device__ __forceinline__ void set_status(uint32_t *status, uint32_t bits) {
     atomicOr(status, bits);
 }

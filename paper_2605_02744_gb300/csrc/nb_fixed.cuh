@@ -129,19 +129,153 @@ __device__ __forceinline__ bool add_f32(unsigned long long *word_hi,
     return true;
 }
 
+// A magnitude m (nonzero) as sign 2^53-significand double m 2^(-shift),
+// rounded to nearest even in integer arithmetic (ldexp and the FP64
+// conversions are slow on this part); results below the smallest normal
+// double go through ldexp.
+__host__ __device__ inline double scaled(unsigned __int128 m, int shift, bool neg) {
+    const unsigned long long mh = (unsigned long long)(m >> 64), ml = (unsigned long long)m;
+#ifdef __CUDA_ARCH__
+    const int lz = mh ? __clzll((long long)mh) : 64 + __clzll((long long)ml);
+#else
+    const int lz = mh ? __builtin_clzll(mh) : 64 + __builtin_clzll(ml);
+#endif
+    const int top = 127 - lz;  // bit of the leading one
+    unsigned long long K;      // 53 significant bits
+    if (top <= 52) {
+        K = ml << (52 - top);
+    } else {
+        const int sh = top - 52;
+        K = (unsigned long long)(m >> sh);
+        const unsigned __int128 rest = m & (((unsigned __int128)1 << sh) - 1);
+        const unsigned __int128 half = (unsigned __int128)1 << (sh - 1);
+        if (rest > half || (rest == half && (K & 1ull))) ++K;  // 2^53: the exponent moves up
+    }
+    const int e = top + 1023 - shift;
+    double d;
+    if (e >= 1 && e < 2046) {
+        const unsigned long long b = ((unsigned long long)(e - 1) << 52) + K;
+        memcpy(&d, &b, 8);
+    } else {
+        d = ldexp((double)K, top - 52 - shift);
+    }
+    return neg ? -d : d;
+}
+
 // The accumulated value: (signed) hi 2^40 + lo, exactly as a 128-bit
 // integer, then rounded once to double and scaled by 2^-F.
-__device__ __forceinline__ double value(unsigned long long word_hi, unsigned long long word_lo,
+__host__ __device__ inline double value(unsigned long long word_hi, unsigned long long word_lo,
                                         int F) {
     const __int128 t = ((__int128)(long long)word_hi) * ((__int128)1 << kLoBits) +
                        (__int128)word_lo;
-    const bool neg = t < 0;
-    const unsigned __int128 m = neg ? (unsigned __int128)(-t) : (unsigned __int128)t;
-    const unsigned long long mh = (unsigned long long)(m >> 64);
-    const unsigned long long ml = (unsigned long long)m;
-    // mh < 2^40 converts exactly; one more rounding in the sum
-    const double d = mh ? ldexp((double)mh, 64) + (double)ml : (double)ml;
-    return ldexp(neg ? -d : d, -F);
+    if (!t) return 0.0;
+    return scaled(t < 0 ? (unsigned __int128)(-t) : (unsigned __int128)t, F, t < 0);
+}
+
+// ------------------------------------------------------------- four limbs
+// The same with four signed limbs of 44 bits, X = sum L_q 2^(44 q), for the
+// warp-granular kernels: their VJP and jerk bounds grow with eps^-3, and 100
+// bits below them would be coarser than the FP32 pair terms once eps is below
+// ~1e-6 of the system size; 174 bits are not before ~1e-13 of it, where FP32
+// displacements have long run out.  A 24-bit significand touches one limb, or
+// two where it straddles a boundary, whatever its sign.  19 bits of headroom:
+// 2^19 adds per accumulator.
+constexpr int kLimbs = 4, kLimbBits = 44;
+constexpr int kLimbMagBits = kLimbs * kLimbBits - 2;  // |X| < 2^174
+
+__host__ __device__ inline int limb_exponent_for(double bound) {
+    if (!(bound > 0.0)) return 0;
+    if (!isfinite(bound)) return -900;
+    int e = 0;
+    frexp(bound, &e);  // bound < 2^e
+    const int F = kLimbMagBits - e;
+    return F < -900 ? -900 : (F > 900 ? 900 : F);
+}
+
+// v 2^F rounded half away from zero: limb q gains lo, limb q + 1 hi (both with
+// v's sign; zeros need no add).  false (no increments) if v is not finite or
+// beyond the limbs.
+__host__ __device__ inline bool split_limbs(float v, int F, int &q, long long &lo, long long &hi) {
+    uint32_t b;
+    memcpy(&b, &v, 4);
+    const int be = (int)((b >> 23) & 0xffu);
+    q = 0;
+    lo = hi = 0;
+    if (be == 0xff) return false;  // inf or NaN
+    uint32_t m = b & 0x7fffffu;
+    if (be) m |= 0x800000u;
+    if (!m) return true;  // +-0
+    int s = (be ? be : 1) - 150 + F;  // X = m 2^s
+    unsigned long long M = m;
+    if (s < 0) {
+        if (s < -25) return true;  // below half a grid step
+        M = (M + (1ull << (-s - 1))) >> (-s);
+        s = 0;
+    }
+    q = s / kLimbBits;
+    const int r = s - q * kLimbBits;
+    const unsigned long long l = (M << r) & ((1ull << kLimbBits) - 1), h = M >> (kLimbBits - r);
+    if (q >= kLimbs || (q == kLimbs - 1 && h)) {
+        q = 0;
+        return false;
+    }
+    lo = (b >> 31) ? -(long long)l : (long long)l;
+    hi = (b >> 31) ? -(long long)h : (long long)h;
+    return true;
+}
+
+// The accumulated value of the limbs, rounded once to double.
+__host__ __device__ inline double limb_value(const long long (&w)[kLimbs], int F) {
+    long long t[kLimbs];
+    long long c = 0;  // carries: every limb but the top one into [0, 2^44)
+#pragma unroll
+    for (int k = 0; k < kLimbs; ++k) {
+        t[k] = w[k] + c;
+        if (k + 1 < kLimbs) {
+            c = t[k] >> kLimbBits;
+            t[k] -= c * (1ll << kLimbBits);
+        }
+    }
+    const bool neg = t[kLimbs - 1] < 0;
+    if (neg) {  // the magnitude's limbs
+        c = 0;
+#pragma unroll
+        for (int k = 0; k < kLimbs; ++k) {
+            t[k] = c - t[k];
+            if (k + 1 < kLimbs) {
+                c = t[k] >> kLimbBits;
+                t[k] -= c * (1ll << kLimbBits);
+            }
+        }
+    }
+    int shift = F;
+    if (t[3] == 0) {  // the leading three limbs that hold anything
+        t[3] = t[2];
+        t[2] = t[1];
+        t[1] = t[0];
+        t[0] = 0;
+        shift += kLimbBits;
+    }
+    if (t[3] == 0) {
+        t[3] = t[2];
+        t[2] = t[1];
+        t[1] = 0;
+        shift += kLimbBits;
+    }
+    if (t[3] == 0) {
+        t[3] = t[2];
+        t[2] = 0;
+        shift += kLimbBits;
+    }
+    // t3 2^132 + t2 2^88 + t1 2^44 + t0 with t3 != 0 unless all are zero: 128
+    // bits from 2^72 up (t3 < 2^63, so t3 2^60 fits), the rest as a sticky bit
+    // (they only decide ties)
+    const bool sticky = (t[1] & ((1ll << 28) - 1)) | t[0];
+    const unsigned __int128 m = ((unsigned __int128)t[3] << 60) |
+                                ((unsigned __int128)t[2] << 16) | ((unsigned __int128)t[1] >> 28) |
+                                (sticky ? 1 : 0);
+    if (!m) return 0.0;
+    return scaled(m, shift - 72, neg);
 }
 
 }  // namespace fx

@@ -497,7 +497,7 @@ int launch_force(const ForceJob &j) {
     if (j.precision == NB_PREC_FP64) {
         if (j.sym) {
             if (guard) return fail(NB_ERR_UNSUPPORTED, "symmetric pairs need eps > 0");
-            return launch_force_sym(j, false);
+            return launch_force_sym(j);
         }
         constexpr int NT = 128;
         const int64_t grid = cdiv(j.ni, NT);
@@ -517,6 +517,7 @@ int launch_force(const ForceJob &j) {
     const bool adaptive = j.adaptive && !guard;
     char *sb = j.ws + j.L.sortbuf;
     if (j.sym && guard) return fail(NB_ERR_UNSUPPORTED, "symmetric pairs need eps > 0");
+    if (takes_wsym(j)) return launch_force_wsym(j);
     if (adaptive) {
         // boxes per 64 j-slots and per warp of i-slots (direct kernel: 32 IR
         // slots; symmetric FP32 kernel: 256 slots)
@@ -531,7 +532,7 @@ int launch_force(const ForceJob &j) {
         int rc = launch_pack(j.pos, j.mass, j.N, j.L.Np, soa, j.stream);
         if (rc) return rc;
     }
-    if (j.sym) return launch_force_sym(j, adaptive);
+    if (j.sym && adaptive) return launch_force_sym(j);
     const Shape &sh = j.shape;
     ForceParams p;
     p.soa = soa;

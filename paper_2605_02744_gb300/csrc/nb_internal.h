@@ -63,6 +63,28 @@ void kernel_timer_end(cudaStream_t st);
 int occupancy(const void *kernel, int threads, size_t smem);
 int persistent_grid(int cps, int occ, int64_t total);
 
+// Launches `kernel` so that its blocks may be placed while the kernel before
+// it on the stream drains (programmatic dependent launch); the kernel itself
+// waits for that one with dev::grid_wait().  On a chain of short kernels this
+// hides most of the launch latency between them.
+template <class... P, class... A>
+int launch_pdl(void (*kernel)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t st,
+               A &&...args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at = {};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    NB_CUDA(cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...));
+    count_launch();
+    return NB_OK;
+}
+
 // --------------------------------------------------------- workspace
 // Byte offsets inside the caller's workspace.  Everything is 256-B aligned.
 struct WsLayout {
@@ -76,6 +98,8 @@ struct WsLayout {
     size_t scratch;   // O(N) reduction scratch (energy partials, batched queue)
     size_t sym_fx;    // symmetric-pair path: fixed-point totals, 64 B per slot
     size_t sym_cost;  // symmetric-pair path: exponent, item costs, their prefix, CTA ranges
+    size_t wsym_head; // warp-granular path: exponents (at 64), input maxima (at 128, zero between calls)
+    size_t wsym_fx;   // its fixed-point totals, 7 components x 4 limbs per slot (zero between calls)
     size_t bsym, bsym_bytes;  // batched symmetric-pair path (0 bytes: not provisioned)
     size_t sym_fx_bytes;      // 0 when the symmetric path is not provisioned
     size_t total;
@@ -198,14 +222,21 @@ int launch_force(const ForceJob &job);
 // ------------------------------------------------- symmetric-pair path
 // Row blocks of 2048 slots; items are the block pairs (I, J >= I).
 constexpr int64_t kSymBlock = 2048;
-// Default size range of the symmetric-pair path (its scratch is O(N): 64 B
-// per particle of fixed-point totals, 268 MB at N = 2^22, plus 12 B per
-// block pair of cost estimates, 25 MB at 2^22, 400 MB at 2^24).  Below the
-// lower end the direct kernel is faster (Kahan evaluation, direct /
-// symmetric: 0.185 / 0.232 ms at 16384, 0.386 / 0.365 at 24576, 0.673 /
-// 0.552 at 32768).
+// Default size range of the symmetric-pair paths.  From kSymMinN whatever the
+// options; up to kSymMaxN (scratch O(N): 64 B per particle of fixed-point
+// totals, 268 MB at N = 2^22, plus 12 B per block pair of the adaptive path's
+// cost estimates, 25 MB at 2^22, 400 MB at 2^24).  Below kSymMinN, from
+// kWsymMinN, what has no use for a direct-kernel option takes the
+// warp-granular path (F64ACC step, direct / warp-granular: 34.6 / 19.4 us at
+// 4095, 77.5 / 40.9 at 8192).
 constexpr int64_t kSymMinN = 24576;
 constexpr int64_t kSymMaxN = 1 << 24;
+constexpr int64_t kWsymMinN = 4800;
+constexpr int kWsymComponents = 7;  // sums per particle at most
+// Largest system of the warp-granular path (its accumulators take 2^19 adds,
+// one per block of 128 slots and range end); an explicit request for
+// symmetric pairs without the adaptive displacement goes direct above it.
+constexpr int64_t kWsymMaxN = 1 << 26;
 struct SymSizes {
     int64_t nb, T, U, ctas;  // row blocks, items, stream-K units, CTAs
     size_t fx_bytes, cost_bytes;
@@ -225,7 +256,14 @@ SymLayout sym_layout(char *ws, const WsLayout &L);
 // Whether the symmetric-pair path is provisioned / taken for N particles in
 // B clusters under opts (nb_pairs; FP32-pair policies, single systems).
 bool sym_wanted(const nb_opts *opts, int64_t N, int32_t B);
-int launch_force_sym(const ForceJob &job, bool adaptive);
+int launch_force_sym(const ForceJob &job);
+// The warp-granular symmetric path (nb_wsym.cu; no adaptive displacement):
+// one evaluation, and an nb_step loop's evaluations with its O(N) work fused.
+inline bool takes_wsym(const ForceJob &j) {
+    return j.sym && !j.adaptive && j.eps > 0.0 && j.precision != NB_PREC_FP64 && j.N <= kWsymMaxN;
+}
+int launch_force_wsym(const ForceJob &job);
+int launch_step_wsym(const ForceJob &job, double *vel, double dt, int64_t nsteps, bool acc_valid);
 
 struct VjpJob {
     const double *pos;

@@ -63,11 +63,11 @@
 // once (and zeroes them for the next call), applies G, scatters through the
 // Hilbert permutation and optionally kicks the velocity.
 //
-// Displacements: single floats, hi/lo pairs (x_j.hi - x_i.hi) +
-// (x_j.lo - x_i.lo), or adaptive: per (warp i-set, j-set) the hi/lo form
-// only when the bounding boxes are closer than gamma * max|x| (a 32-bit
-// mask per warp and item, from the Hilbert-sorted pack's boxes of 256 i-
-// and 64 j-slots).
+// Displacements are adaptive: per (warp i-set, j-set) the hi/lo form
+// (x_j.hi - x_i.hi) + (x_j.lo - x_i.lo) only when the bounding boxes are
+// closer than gamma * max|x| (a 32-bit mask per warp and item, from the
+// Hilbert-sorted pack's boxes of 256 i- and 64 j-slots), single floats
+// elsewhere.  Systems with one form for every pair go to nb_wsym.cu.
 //
 // FP64 pairs (force_sym64_kernel) keep the first form of this kernel: 16
 // warps of 128 slots (4 per lane, doubles), 32-slot j-sets of one particle
@@ -173,14 +173,12 @@ __device__ __forceinline__ void load_jp(const SymParams &p, int64_t s, float (&j
     symj::load_pair(p.soa, p.Np, s, j);
 }
 
-// MODE: 0 single-float displacement, 1 hi/lo, 2 adaptive.  POT: the
-// potential sums too (the caller wants phi).  The i-slots' lo parts stay in
-// registers for MODE 1 (every j-set is near) and come from shared memory
-// for MODE 2 (only near j-sets use them; 245 of 255 registers are taken).
-template <int POL, int MODE, bool POT>
+// POT: the potential sums too (the caller wants phi).  The i-slots' lo parts
+// come from shared memory: only near j-sets use them, and 245 of 255
+// registers are taken.
+template <int POL, bool POT>
 __global__ void __launch_bounds__(NT, CPS) force_sym_kernel(const SymParams p) {
     constexpr int NWJ = NW, IRJ = IRP, SNTJ = NT;
-    constexpr bool LOSM = MODE == 2;
     constexpr int HW = IRJ / 2;  // j-sets per warp i-set
     constexpr size_t kRedBytesJ = kRedBytes;
     extern __shared__ __align__(16) unsigned char smemj[];
@@ -188,7 +186,7 @@ __global__ void __launch_bounds__(NT, CPS) force_sym_kernel(const SymParams p) {
     Acc<POL> *tot = reinterpret_cast<Acc<POL> *>(smemj + kRedBytesJ);  // [IRJ * 4][SNTJ]
     constexpr bool MID = POL == NB_PREC_F64ACC;
     float *mid = reinterpret_cast<float *>(smemj + kRedBytesJ + 4 * IRJ * SNTJ * sizeof(Acc<POL>));
-    // LOSM: (-x.lo, -x.lo) pairs [3][IRJ][SNTJ] after the F64ACC middle sums
+    // (-x.lo, -x.lo) pairs [3][IRJ][SNTJ] after the F64ACC middle sums
     float2 *lo2 = reinterpret_cast<float2 *>(smemj + kRedBytesJ +
                                              4 * IRJ * SNTJ * sizeof(Acc<POL>) +
                                              (MID ? 4 * IRJ * SNTJ * sizeof(float) : 0)) +
@@ -225,17 +223,9 @@ __global__ void __launch_bounds__(NT, CPS) force_sym_kernel(const SymParams p) {
                 S.m[k] = f2(m, m);
                 const float xl = __ldg(p.soa + 4 * p.Np + sl), yl = __ldg(p.soa + 5 * p.Np + sl),
                             zl = __ldg(p.soa + 6 * p.Np + sl);
-                if (LOSM) {
-                    if (MODE != 0) {
-                        lo2[(0 * IRJ + k) * SNTJ] = f2(-xl, -xl);
-                        lo2[(1 * IRJ + k) * SNTJ] = f2(-yl, -yl);
-                        lo2[(2 * IRJ + k) * SNTJ] = f2(-zl, -zl);
-                    }
-                } else {
-                    S.nxl[k] = -xl;
-                    S.nyl[k] = -yl;
-                    S.nzl[k] = -zl;
-                }
+                lo2[(0 * IRJ + k) * SNTJ] = f2(-xl, -xl);
+                lo2[(1 * IRJ + k) * SNTJ] = f2(-yl, -yl);
+                lo2[(2 * IRJ + k) * SNTJ] = f2(-zl, -zl);
                 S.ax[k] = S.ay[k] = S.az[k] = S.ph[k] = f2(0.f, 0.f);
             }
 #pragma unroll
@@ -247,16 +237,13 @@ __global__ void __launch_bounds__(NT, CPS) force_sym_kernel(const SymParams p) {
         }
         const bool sym = J != I;
         const int64_t jb = J * BI;
-        unsigned near = 0u;
-        if (MODE == 2) {
-            float wb[7], tb[7];
+        float wb[7], tb[7];
 #pragma unroll
-            for (int a = 0; a < 7; ++a) {
-                wb[a] = __ldg(p.wbox + (ib / (32 * IRJ)) * 8 + a);
-                tb[a] = __ldg(p.jbox + (jb / JSP + l) * 8 + a);
-            }
-            near = __ballot_sync(0xffffffffu, boxes_near(wb, tb, p.gamma));
+        for (int a = 0; a < 7; ++a) {
+            wb[a] = __ldg(p.wbox + (ib / (32 * IRJ)) * 8 + a);
+            tb[a] = __ldg(p.jbox + (jb / JSP + l) * 8 + a);
         }
+        const unsigned near = __ballot_sync(0xffffffffu, boxes_near(wb, tb, p.gamma));
         float jn[14];
         load_jp(p, jb + qa * JSP + l, jn);
         for (int q = qa; q < qb; ++q) {
@@ -267,14 +254,14 @@ __global__ void __launch_bounds__(NT, CPS) force_sym_kernel(const SymParams p) {
             const bool nq = (near >> q) & 1u;
             float4 b0, b1;
             if (sym) {
-                run_setj<IRJ, MODE, true, POT, LOSM>(S, e2, jc, nq, b0, b1, -1, lo2, SNTJ);
+                run_setj<IRJ, true, POT>(S, e2, jc, nq, b0, b1, -1, lo2, SNTJ);
                 float4 *r = red + (((half * KBP + (q % KBP)) * 2) * NWJ + w) * 32 + l;
                 r[0] = b0;
                 r[NWJ * 32] = b1;
             } else {
                 // the warp's own slots are j-sets HW w .. HW w + HW - 1 of the block
-                run_setj<IRJ, MODE, false, POT, LOSM>(S, e2, jc, nq, b0, b1,
-                                                  q / HW == w ? q % HW : -1, lo2, SNTJ);
+                run_setj<IRJ, false, POT>(S, e2, jc, nq, b0, b1,
+                                          q / HW == w ? q % HW : -1, lo2, SNTJ);
             }
             if ((q + 1) % FLP == 0 || q + 1 == qb) {
 #pragma unroll
@@ -611,7 +598,7 @@ __device__ __forceinline__ void item_of(int64_t t, int64_t nb, int64_t &I, int64
 }
 
 // The adaptive FP32 kernel's unit costs of item t, one thread: the same
-// sums as sym_cost_kernel<2, NW, JSP> (which adds them up per item).
+// sums as sym_cost_kernel<true, NW, JSP> (which adds them up per item).
 __device__ void item_unit_costs(const SymParams &p, int64_t t, uint32_t (&uc)[US]) {
     int64_t I, J;
     item_of(t, p.nb, I, J);
@@ -636,10 +623,10 @@ __device__ void item_unit_costs(const SymParams &p, int64_t t, uint32_t (&uc)[US
 }
 
 // One warp per item: the near/far decisions the pair kernel will take.  For
-// the adaptive FP32 kernel lane l takes j-set l (unit l / 2): the unit's
-// cost is the maximum over the warps of its two j-sets' sum; other modes
-// give every unit the same cost.
-template <int MODE, int NWK, int JSET>
+// the FP32 kernel lane l takes j-set l (unit l / 2): the unit's cost is the
+// maximum over the warps of its two j-sets' sum; for FP64 pairs every unit
+// costs the same.
+template <bool NEARFAR, int NWK, int JSET>
 __global__ void __launch_bounds__(256) sym_cost_kernel(const SymParams p, uint32_t *cost) {
     constexpr int NJ = BI / JSET;  // j-sets per block
     constexpr int WS = BI / NWK;   // i-slots per warp
@@ -652,9 +639,8 @@ __global__ void __launch_bounds__(256) sym_cost_kernel(const SymParams p, uint32
     const uint32_t cn = sym ? kCostSymNear : kCostDiagNear;
     const uint32_t cf = sym ? kCostSymFar : kCostDiagFar;
     uint32_t c = 0;
-    if constexpr (MODE != 2) {
-        // every unit of the item alike (every j-set near for MODE 1)
-        c = (l & 1) ? 0u : 2 * (MODE == 1 ? cn : cf) + kCostSymUnit;
+    if constexpr (!NEARFAR) {
+        c = (l & 1) ? 0u : 2 * cf + kCostSymUnit;
     } else {
         static_assert(NJ == 32 && KBP == 2 && NWK == NW, "lane l: j-set l, unit l / 2");
         float tb[7];
@@ -708,7 +694,7 @@ __global__ void __launch_bounds__(1024) sym_scan_kernel(const uint32_t *cost, in
 // (the nearest unit boundary, from the item's unit costs for the adaptive
 // kernel, linearly inside an item otherwise); lo[0] = 0, lo[ctas] = U,
 // non-decreasing.
-template <int MODE>
+template <bool NEARFAR>
 __global__ void sym_ranges_kernel(const SymParams p, const uint32_t *cost,
                                   const unsigned long long *prefix, int64_t T, int64_t ctas,
                                   int64_t *lo) {
@@ -729,7 +715,7 @@ __global__ void sym_ranges_kernel(const SymParams p, const uint32_t *cost,
         }
         const unsigned long long r = target - prefix[a];
         int64_t off;
-        if (MODE == 2) {
+        if (NEARFAR) {
             uint32_t uc[US];
             item_unit_costs(p, a, uc);
             unsigned long long run = 0;
@@ -744,12 +730,12 @@ __global__ void sym_ranges_kernel(const SymParams p, const uint32_t *cost,
     }
 }
 
-template <int POL, int MODE, bool POT>
+template <int POL, bool POT>
 int launch_pair(const SymParams &p, cudaStream_t st) {
-    auto kern = force_sym_kernel<POL, MODE, POT>;
+    auto kern = force_sym_kernel<POL, POT>;
     const size_t smem = kRedBytes + 4 * BI * sizeof(Acc<POL>) +
                         (POL == NB_PREC_F64ACC ? 4 * BI * sizeof(float) : 0) +
-                        (MODE == 2 ? 3 * BI * sizeof(float2) : 0);
+                        3 * BI * sizeof(float2);
     const int rc = smem_optin(reinterpret_cast<const void *>(kern), smem);
     if (rc != NB_OK) return rc;
     kernel_timer_begin(st);
@@ -760,16 +746,16 @@ int launch_pair(const SymParams &p, cudaStream_t st) {
     return NB_OK;
 }
 
-// FP64: the cost estimate per (16 warps x 32-slot j-sets), else per
-// (8 warps x 64-slot j-sets).
-template <int MODE, bool FP64 = false>
+// FP64: units of equal cost; FP32: the near/far estimate per (8 warps x
+// 64-slot j-sets).
+template <bool FP64>
 int launch_split(const SymParams &p, const ForceJob &j, const SymLayout &y) {
     if constexpr (FP64)
-        sym_cost_kernel<0, SW, JS><<<(unsigned)cdiv(p.T * 32, 256), 256, 0, j.stream>>>(p, y.cost);
+        sym_cost_kernel<false, SW, JS><<<(unsigned)cdiv(p.T * 32, 256), 256, 0, j.stream>>>(p, y.cost);
     else
-        sym_cost_kernel<MODE, NW, JSP><<<(unsigned)cdiv(p.T * 32, 256), 256, 0, j.stream>>>(p, y.cost);
+        sym_cost_kernel<true, NW, JSP><<<(unsigned)cdiv(p.T * 32, 256), 256, 0, j.stream>>>(p, y.cost);
     sym_scan_kernel<<<1, 1024, 0, j.stream>>>(y.cost, p.T, y.prefix);
-    sym_ranges_kernel<FP64 ? 0 : MODE><<<(unsigned)cdiv(p.ctas + 1, 256), 256, 0, j.stream>>>(
+    sym_ranges_kernel<!FP64><<<(unsigned)cdiv(p.ctas + 1, 256), 256, 0, j.stream>>>(
         p, y.cost, y.prefix, p.T, p.ctas, y.lo);
     sym_exponent_kernel<<<(unsigned)std::min<int64_t>(cdiv(j.N, 4 * 256), 1024), 256, 0,
                           j.stream>>>(j.mass, j.N, j.eps, y.fx_exp, y.mmax_bits, y.arrivals);
@@ -787,11 +773,10 @@ int launch_fold(const SymParams &p, const ForceJob &j, const int *perm) {
     return NB_OK;
 }
 
-template <int POL, int MODE>
-int launch_sym_mode(const SymParams &p, const ForceJob &j, const SymLayout &y, const int *perm) {
-    NB_TRY_SYM(launch_split<MODE>(p, j, y));
-    NB_TRY_SYM(j.pot ? launch_pair<POL, MODE, true>(p, j.stream)
-                     : launch_pair<POL, MODE, false>(p, j.stream));
+template <int POL>
+int launch_sym_pol(const SymParams &p, const ForceJob &j, const SymLayout &y, const int *perm) {
+    NB_TRY_SYM(launch_split<false>(p, j, y));
+    NB_TRY_SYM(j.pot ? launch_pair<POL, true>(p, j.stream) : launch_pair<POL, false>(p, j.stream));
     return launch_fold(p, j, perm);
 }
 
@@ -807,19 +792,9 @@ int launch_pair64(const SymParams64 &p, cudaStream_t st) {
 }
 
 int launch_sym64(const SymParams64 &p, const ForceJob &j, const SymLayout &y) {
-    NB_TRY_SYM(launch_split<0, true>(p, j, y));
+    NB_TRY_SYM(launch_split<true>(p, j, y));
     NB_TRY_SYM(j.pot ? launch_pair64<true>(p, j.stream) : launch_pair64<false>(p, j.stream));
     return launch_fold(p, j, nullptr);
-}
-
-template <int POL>
-int launch_sym_pol(const SymParams &p, const ForceJob &j, const SymLayout &y, int mode,
-                   const int *perm) {
-    switch (mode) {
-        case 0: return launch_sym_mode<POL, 0>(p, j, y, perm);
-        case 1: return launch_sym_mode<POL, 1>(p, j, y, perm);
-        default: return launch_sym_mode<POL, 2>(p, j, y, perm);
-    }
 }
 
 }  // namespace
@@ -851,7 +826,7 @@ SymLayout sym_layout(char *ws, const WsLayout &L) {
     return y;
 }
 
-int launch_force_sym(const ForceJob &j, bool adaptive) {
+int launch_force_sym(const ForceJob &j) {
     if (j.eps <= 0.0) return fail(NB_ERR_UNSUPPORTED, "symmetric pairs need eps > 0");
     if (j.L.sym_fx_bytes == 0)
         return fail(NB_ERR_WORKSPACE, "workspace has no symmetric-pair buffers");
@@ -868,14 +843,13 @@ int launch_force_sym(const ForceJob &j, bool adaptive) {
     const float ef = (float)j.eps;
     p.eps2 = ef * ef;
     p.gamma = j.gamma;
-    p.jbox = adaptive ? sort_tile_boxes(sb, j.L) : nullptr;
-    p.wbox = adaptive ? sort_block_boxes(sb, j.L) : nullptr;
+    p.jbox = sort_tile_boxes(sb, j.L);
+    p.wbox = sort_block_boxes(sb, j.L);
     p.acc_fx = y.acc_fx;
     p.fx_exp = y.fx_exp;
     p.lo = y.lo;
-    const int *perm = adaptive ? sort_perm(sb, j.L) : nullptr;
+    const int *perm = sort_perm(sb, j.L);
     p.status = reinterpret_cast<uint32_t *>(j.ws + j.L.status);
-    const int mode = adaptive ? 2 : (j.split ? 1 : 0);
     if (j.precision == NB_PREC_FP64) {
         SymParams64 p64;
         static_cast<SymParams &>(p64) = p;
@@ -886,9 +860,9 @@ int launch_force_sym(const ForceJob &j, bool adaptive) {
         return launch_sym64(p64, j, y);
     }
     switch (j.precision) {
-        case NB_PREC_FP32: return launch_sym_pol<NB_PREC_FP32>(p, j, y, mode, perm);
-        case NB_PREC_KAHAN: return launch_sym_pol<NB_PREC_KAHAN>(p, j, y, mode, perm);
-        case NB_PREC_F64ACC: return launch_sym_pol<NB_PREC_F64ACC>(p, j, y, mode, perm);
+        case NB_PREC_FP32: return launch_sym_pol<NB_PREC_FP32>(p, j, y, perm);
+        case NB_PREC_KAHAN: return launch_sym_pol<NB_PREC_KAHAN>(p, j, y, perm);
+        case NB_PREC_F64ACC: return launch_sym_pol<NB_PREC_F64ACC>(p, j, y, perm);
     }
     return fail(NB_ERR_INVALID, "unknown precision %d", j.precision);
 }
