@@ -271,6 +271,14 @@ bool sym_wanted(const nb_opts *o, int64_t N, int32_t B) {
            o->positions != NB_POS_ADAPTIVE && o->test_unissued_stage == 0;
 }
 
+// Whether the acceleration + jerk of N particles takes the
+// warp-granular symmetric path (from min_n particles).  Direct pairs, a launch
+// shape or the ring's test hook ask for the direct kernel; eps = 0 needs it.
+static bool wsym_wanted(const nb_opts *o, int64_t N, double eps, int64_t min_n) {
+    return o->precision != NB_PREC_FP64 && o->pairs != NB_PAIRS_DIRECT && eps > 0.0 && N >= min_n &&
+           N <= kSymMaxN && !shape_asked(o) && o->test_unissued_stage == 0;
+}
+
 int check_ws(const void *ws, size_t ws_bytes, const WsLayout &L) {
     if (!ws) return fail(NB_ERR_INVALID, "workspace pointer is NULL");
     if (((uintptr_t)ws & 255) != 0) return fail(NB_ERR_INVALID, "workspace must be 256-byte aligned");
@@ -1025,6 +1033,7 @@ static int make_jerk_job(JerkJob *j, double *pos, double *vel, const double *mas
     j->jerk = jerk;
     j->pot = pot;
     j->precision = o->precision;
+    j->sym = wsym_wanted(o, N, eps, kWsymJerkMinN);
     j->timeout = timeout_of(o);
     j->unissued = unissued_of(o);
     j->stream = (cudaStream_t)o->stream;

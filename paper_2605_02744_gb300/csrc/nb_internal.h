@@ -232,6 +232,10 @@ constexpr int64_t kSymBlock = 2048;
 constexpr int64_t kSymMinN = 24576;
 constexpr int64_t kSymMaxN = 1 << 24;
 constexpr int64_t kWsymMinN = 4800;
+// The same for the acceleration + jerk, whose direct kernel pays more per pair
+// (F64ACC, direct / symmetric: 31.8 / 20.6 us at 260; below two blocks of 128
+// there is nothing to share out).
+constexpr int64_t kWsymJerkMinN = 256;
 constexpr int kWsymComponents = 7;  // sums per particle at most
 // Largest system of the warp-granular path (its accumulators take 2^19 adds,
 // one per block of 128 slots and range end); an explicit request for
@@ -323,6 +327,7 @@ struct JerkJob {
     double h;
     int64_t nsteps;  // 0 = evaluate a, jerk, phi at the current state
     int precision;
+    bool sym;        // symmetric pairs (wsym_wanted)
     long long timeout;
     int64_t unissued;  // test hook (nb_opts.test_unissued_stage - 1; -1: off)
     cudaStream_t stream;

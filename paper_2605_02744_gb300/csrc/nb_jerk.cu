@@ -18,6 +18,7 @@
 
 #include "nb_device.cuh"
 #include "nb_internal.h"
+#include "nb_wsym.cuh"
 
 namespace nb {
 
@@ -290,6 +291,211 @@ static int launch_jerk_kernel(const JerkParams &p, cudaStream_t st) {
     return NB_OK;
 }
 
+// ------------------------------------------------- symmetric pairs
+// The same sums with each unordered pair evaluated once (nb_wsym.cuh): with
+// e = w - 3 r^2 (d . w) d and t = r^3, a_i += m_j t d, jerk_i += m_j t e,
+// a_j -= m_i t d, jerk_j -= m_i t e, i.e. 39 packed FP32 operations per two
+// unordered pairs (41 with the potential) instead of 2 x 34.
+namespace {
+
+using namespace wsym;
+
+template <bool IPAIR_, bool POT>
+struct JerkPh {
+    static constexpr bool IPAIR = IPAIR_;
+    static constexpr int K = 4, WARPS = 8, NJ = 10, NC = POT ? 7 : 6, GROUPS = 2;
+    struct S {
+        float2 nx[K], ny[K], nz[K], m[K], nvx[K], nvy[K], nvz[K];
+        LoT<IPAIR> nxl[K], nyl[K], nzl[K];
+        float2 a[K][NC];  // ax ay az jx jy jz (phi)
+    };
+    // exponents: the jerk's, then the others'
+    static __device__ __forceinline__ constexpr int group(int e) { return e >= 3 && e < 6 ? 0 : 1; }
+    static __device__ __forceinline__ constexpr bool jneg(int e) { return e < 6; }
+    static __device__ __forceinline__ double bound(const Params &p, int g) {
+        const double m = (double)__uint_as_float(__ldcg(p.mx + kMaxM));
+        const double v = (double)__uint_as_float(__ldcg(p.mx + p.vword));
+        return g == 0 ? p.scale[1] * m * v : p.scale[0] * m;
+    }
+    static __device__ __forceinline__ const float *plane(const Params &p, int a) {
+        return p.soa + a * p.Np;
+    }
+    static __device__ __forceinline__ void set_i(S &s, int k, const float2 (&v)[NJ]) {
+        s.nx[k] = neg(v[0]);
+        s.ny[k] = neg(v[1]);
+        s.nz[k] = neg(v[2]);
+        s.m[k] = v[3];
+        s.nxl[k] = lo_of<IPAIR>(neg(v[4]));
+        s.nyl[k] = lo_of<IPAIR>(neg(v[5]));
+        s.nzl[k] = lo_of<IPAIR>(neg(v[6]));
+        s.nvx[k] = neg(v[7]);
+        s.nvy[k] = neg(v[8]);
+        s.nvz[k] = neg(v[9]);
+    }
+    template <bool SYM, bool SELF>
+    static __device__ __forceinline__ void step(S &s, const float2 e2, const float2 (&J)[NJ],
+                                                float2 (&T)[NC], int self_h) {
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+            const float2 dx = add2(add2(J[0], s.nx[k]), add2(J[4], lo2(s.nxl[k])));
+            const float2 dy = add2(add2(J[1], s.ny[k]), add2(J[5], lo2(s.nyl[k])));
+            const float2 dz = add2(add2(J[2], s.nz[k]), add2(J[6], lo2(s.nzl[k])));
+            float2 r2 = fma2(dx, dx, e2);
+            r2 = fma2(dy, dy, r2);
+            r2 = fma2(dz, dz, r2);
+            const float2 wx = add2(J[7], s.nvx[k]);
+            const float2 wy = add2(J[8], s.nvy[k]);
+            const float2 wz = add2(J[9], s.nvz[k]);
+            float2 dw = mul2(dx, wx);
+            dw = fma2(dy, wy, dw);
+            dw = fma2(dz, wz, dw);
+            const float2 r = f2(rsqrt_approx(r2.x), rsqrt_approx(r2.y));
+            const float2 rr = mul2(r, r);
+            const float2 r3 = mul2(rr, r);
+            const float2 q = mul2(mul2(rr, f2(-3.f, -3.f)), dw);
+            const float2 ex = fma2(q, dx, wx);
+            const float2 ey = fma2(q, dy, wy);
+            const float2 ez = fma2(q, dz, wz);
+            float2 mj = J[3];
+            if (SELF) mj = mask_self<IPAIR>(mj, k, self_h);
+            const float2 sj = mul2(mj, r3);
+            s.a[k][0] = fma2(sj, dx, s.a[k][0]);
+            s.a[k][1] = fma2(sj, dy, s.a[k][1]);
+            s.a[k][2] = fma2(sj, dz, s.a[k][2]);
+            s.a[k][3] = fma2(sj, ex, s.a[k][3]);
+            s.a[k][4] = fma2(sj, ey, s.a[k][4]);
+            s.a[k][5] = fma2(sj, ez, s.a[k][5]);
+            if constexpr (POT) s.a[k][6] = fma2(mj, r, s.a[k][6]);
+            if (SYM) {
+                const float2 si = mul2(s.m[k], r3);
+                T[0] = k ? fma2(si, dx, T[0]) : mul2(si, dx);
+                T[1] = k ? fma2(si, dy, T[1]) : mul2(si, dy);
+                T[2] = k ? fma2(si, dz, T[2]) : mul2(si, dz);
+                T[3] = k ? fma2(si, ex, T[3]) : mul2(si, ex);
+                T[4] = k ? fma2(si, ey, T[4]) : mul2(si, ey);
+                T[5] = k ? fma2(si, ez, T[5]) : mul2(si, ez);
+                if constexpr (POT) T[6] = k ? fma2(s.m[k], r, T[6]) : mul2(s.m[k], r);
+            }
+        }
+    }
+};
+
+// hermite_predict_pack_kernel's pack, one particle a thread, with the largest
+// |m| and |v| component of the packed state.
+__global__ void __launch_bounds__(128) wsym_predict_pack_kernel(
+    const double *pos, const double *vel, const double *acc,
+    const double *jerk, const double *mass, int64_t N, int64_t Np,
+    double h, float *soa, unsigned *mx, int vword) {
+    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;  // < Np: whole blocks
+    float hi[3] = {0.f, 0.f, 0.f}, lo[3] = {0.f, 0.f, 0.f}, vf[3] = {0.f, 0.f, 0.f};
+    float m = 0.f, am = 0.f, av = 0.f;
+    dev::grid_trigger();
+    dev::grid_wait();
+    if (i < N) {
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            double x = pos[3 * i + c], v = vel[3 * i + c];
+            if (h != 0.0) {
+                const double a = acc[3 * i + c], j = jerk[3 * i + c];
+                x = x + v * h + a * h * h / 2.0 + j * h * h * h / 6.0;
+                v = v + a * h + j * h * h / 2.0;
+            }
+            hi[c] = __double2float_rn(x);
+            lo[c] = __double2float_rn(x - (double)hi[c]);
+            vf[c] = __double2float_rn(v);
+            av = fmaxf(av, fabsf(vf[c]));
+        }
+        const double md = mass[i];
+        m = __double2float_rn(md);
+        am = fabsf(m);
+    }
+    store_packed(soa, Np, i, hi, lo, m);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) soa[(7 + c) * Np + i] = vf[c];
+    warp_max(mx + kMaxM, am);
+    warp_max(mx + vword, av);
+}
+
+// The totals of every particle: read and zeroed, x G, then stored (h = 0) or
+// taken through the Hermite corrector, as jerk_kernel's epilogue.
+template <bool POT>
+__global__ void __launch_bounds__(128) wsym_jerk_fold_kernel(const Params p, const JerkParams q,
+                                                             unsigned *mx) {
+    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    dev::grid_trigger();
+    dev::grid_wait();
+    if (i == 0) mx[kMaxM] = mx[p.vword] = 0u;  // the pair kernel has read them
+    if (i >= p.N) return;
+    const int Fj = p.fxe[0], Fa = p.fxe[1];
+    const double h = q.h;
+    bool ok = true;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        const double a1 = q.G * take_fixed(p, c, i, Fa);
+        const double j1 = q.G * take_fixed(p, 3 + c, i, Fj);
+        if (h != 0.0) {
+            const double x0 = q.pos[3 * i + c], v0 = q.vel[3 * i + c];
+            const double a0 = q.acc[3 * i + c], j0 = q.jerk[3 * i + c];
+            const double v1 = v0 + (a0 + a1) * h / 2.0 + (j0 - j1) * h * h / 12.0;
+            q.pos[3 * i + c] = x0 + (v0 + v1) * h / 2.0 + (a0 - a1) * h * h / 12.0;
+            q.vel[3 * i + c] = v1;
+        }
+        q.acc[3 * i + c] = a1;
+        q.jerk[3 * i + c] = j1;
+        ok = ok && isfinite(a1) && isfinite(j1);
+    }
+    if (POT) q.pot[i] = -q.G * take_fixed(p, 6, i, Fa);
+    if (!ok) dev::set_status(p.status, kStatusNonFinite);
+}
+
+// From this size on a lane holds eight i-slots as four (x_a, x_b) pairs against
+// one j-particle instead of four broadcast i-slots against two j: half the
+// shuffles and half the adds to the totals per pair (802 / 862 us at 32768,
+// 12.3 / 13.4 ms at 131072), in blocks twice as wide, which smaller systems
+// fill less evenly (27 / 24 us at 2047).
+constexpr int64_t kJerkWideMinN = 12288;
+
+int launch_jerk_wsym(const JerkJob &j, JerkParams q) {
+    unsigned *mx = reinterpret_cast<unsigned *>(j.ws + j.L.wsym_head + 128);
+    Params p{};
+    p.soa = q.soa;
+    p.Np = j.L.Np;
+    p.N = j.N;
+    p.eps2 = q.eps2;
+    p.keep = j.precision != NB_PREC_FP32;
+    p.fx = reinterpret_cast<unsigned long long *>(j.ws + j.L.wsym_fx);
+    p.fxe = reinterpret_cast<int *>(j.ws + j.L.wsym_head + 64);
+    p.mx = mx;
+    p.status = q.status;
+    p.vword = kMaxV0;
+    // the bounds: N max|m| times the largest |d| r^3 or r (see nb_wsym.cu), and
+    // times the largest |e| r^3 <= |w| (1 + 3 |d|^2 r^2) r^3 <= 1.146 |w| /
+    // eps^3 (at |d|^2 r^2 = 1/5) with |w| <= 2 sqrt(3) max|v|
+    const double n = 1.02 * (double)j.N;
+    p.scale[0] = n * std::max(0.3849002 / (j.eps * j.eps), 1.0 / j.eps);
+    p.scale[1] = n * 1.146 * 3.4641017 / (j.eps * j.eps * j.eps);
+    for (int64_t n = 0; n < (j.nsteps > 0 ? j.nsteps : 1); ++n) {
+        q.h = j.nsteps > 0 ? j.h : 0.0;
+        int rc = launch_pdl(wsym_predict_pack_kernel, (unsigned)(j.L.Np / 128), 128, 0, j.stream,
+                            j.pos, j.vel, j.acc, j.jerk, j.mass, j.N, j.L.Np, q.h,
+                            reinterpret_cast<float *>(j.ws + j.L.packA), mx, p.vword);
+        if (rc) return rc;
+        if (j.N >= kJerkWideMinN)
+            rc = q.pot ? launch_pairs<JerkPh<true, true>>(p, j.stream)
+                       : launch_pairs<JerkPh<true, false>>(p, j.stream);
+        else
+            rc = q.pot ? launch_pairs<JerkPh<false, true>>(p, j.stream)
+                       : launch_pairs<JerkPh<false, false>>(p, j.stream);
+        if (rc) return rc;
+        auto fold = q.pot ? wsym_jerk_fold_kernel<true> : wsym_jerk_fold_kernel<false>;
+        rc = launch_pdl(fold, (unsigned)cdiv(j.N, 128), 128, 0, j.stream, p, q, mx);
+        if (rc) return rc;
+    }
+    return NB_OK;
+}
+
+}  // namespace
+
 int launch_jerk(const JerkJob &j) {
     if (j.precision == NB_PREC_FP64)
         return fail(NB_ERR_UNSUPPORTED, "the jerk kernel computes FP32 pairs (FP32, KAHAN, F64ACC)");
@@ -312,6 +518,7 @@ int launch_jerk(const JerkJob &j) {
     p.status = reinterpret_cast<uint32_t *>(j.ws + j.L.status);
     p.timeout = j.timeout;
     p.unissued = j.unissued;
+    if (j.sym) return launch_jerk_wsym(j, p);
     const bool guard = j.eps == 0.0;
     const int threads = 256;
     const int64_t pblocks = std::min<int64_t>(cdiv(j.L.Np, threads), 8192);

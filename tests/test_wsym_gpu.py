@@ -47,3 +47,20 @@ def test_forces_at_block_edges(n, prec):
                            positions="single", pairs="direct")
         ra, rp = host(d), host(dp)
     assert rel_vec_err(host(a), ra).max() <= 1e-5 and rel_err(host(p), rp).max() <= 1e-5
+
+
+@pytest.mark.parametrize("n", [256, 257, 3000, 12289])
+def test_jerk_at_block_edges(n):
+    s = ics.plummer_lognormal(n, seed=n)
+    ra, rj, rp = oracle.forces_jerk(s.pos, s.vel, s.mass, EPS)
+    o = binding.make_opts("kahan")
+    ws = binding.workspace(n, 1, o)
+    pos, vel, mass = dev(s.pos), dev(s.vel), dev(s.mass)
+    acc, jerk = torch.empty_like(pos), torch.empty_like(pos)
+    pot = torch.empty_like(mass)
+    for with_pot in (False, True):
+        binding.nb_forces_jerk(pos, vel, mass, EPS, acc, jerk, pot if with_pot else None, ws, o)
+        assert binding.nb_poll_status(ws, o) == binding.NB_OK
+        assert rel_vec_err(host(acc), ra).max() <= 1e-5
+        assert rel_vec_err(host(jerk), rj).max() <= 1e-4
+    assert rel_err(host(pot), rp).max() <= 1e-5
