@@ -271,9 +271,10 @@ bool sym_wanted(const nb_opts *o, int64_t N, int32_t B) {
            o->positions != NB_POS_ADAPTIVE && o->test_unissued_stage == 0;
 }
 
-// Whether the acceleration + jerk of N particles takes the
+// Whether the VJP or the acceleration + jerk of N particles takes the
 // warp-granular symmetric path (from min_n particles).  Direct pairs, a launch
-// shape or the ring's test hook ask for the direct kernel; eps = 0 needs it.
+// shape or the ring's test hook ask for the direct kernel; eps = 0 and row
+// ranges need it.
 static bool wsym_wanted(const nb_opts *o, int64_t N, double eps, int64_t min_n) {
     return o->precision != NB_PREC_FP64 && o->pairs != NB_PAIRS_DIRECT && eps > 0.0 && N >= min_n &&
            N <= kSymMaxN && !shape_asked(o) && o->test_unissued_stage == 0;
@@ -922,6 +923,7 @@ static int make_vjp_job(VjpJob *j, const double *pos, const double *mass, int64_
     // gradients are gated at 1e-4 (median) / 1e-3 (max): single-float
     // displacements unless the caller asks for the split form
     j->split = o->positions == NB_POS_SPLIT;
+    j->sym = wsym_wanted(o, N, eps, kWsymVjpMinN);
     j->timeout = timeout_of(o);
     j->unissued = unissued_of(o);
     j->stream = (cudaStream_t)o->stream;
@@ -960,6 +962,7 @@ int nb_forces_vjp_range(const double *pos, const double *mass, int64_t N, int64_
     j.acc_bar = acc_bar;
     j.pot_bar = pot_bar;
     j.kick_coef = coef;
+    j.sym = false;  // rows: the direct kernel
     j.i0 = i0;
     j.ni = i1 - i0;
     j.step_form = false;

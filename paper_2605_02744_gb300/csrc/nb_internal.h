@@ -232,9 +232,11 @@ constexpr int64_t kSymBlock = 2048;
 constexpr int64_t kSymMinN = 24576;
 constexpr int64_t kSymMaxN = 1 << 24;
 constexpr int64_t kWsymMinN = 4800;
-// The same for the acceleration + jerk, whose direct kernel pays more per pair
-// (F64ACC, direct / symmetric: 31.8 / 20.6 us at 260; below two blocks of 128
-// there is nothing to share out).
+// The same for the VJP and the acceleration + jerk, whose direct kernels pay
+// more per pair (F64ACC, direct / symmetric: VJP 23.8 / 14.7 us, acceleration
+// + jerk 31.8 / 20.6 us at 260; below two blocks of 128 there is nothing to
+// share out).
+constexpr int64_t kWsymVjpMinN = 256;
 constexpr int64_t kWsymJerkMinN = 256;
 constexpr int kWsymComponents = 7;  // sums per particle at most
 // Largest system of the warp-granular path (its accumulators take 2^19 adds,
@@ -297,6 +299,7 @@ struct VjpJob {
     double rewind_drift;
     int precision;
     bool split;  // hi/lo displacement (the VJP's default is single floats)
+    bool sym;    // symmetric pairs (wsym_wanted)
     long long timeout;
     int64_t unissued;  // test hook (nb_opts.test_unissued_stage - 1; -1: off)
     cudaStream_t stream;

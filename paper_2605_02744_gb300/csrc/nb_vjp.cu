@@ -23,6 +23,7 @@
 
 #include "nb_device.cuh"
 #include "nb_internal.h"
+#include "nb_wsym.cuh"
 
 namespace nb {
 
@@ -540,10 +541,276 @@ static int launch_vjp_variant(const VjpParams &p, bool guard, bool pb, bool fuse
                  : launch_vjp_variant2<NT, IR, TJ, ST, false>(p, guard, pb, fused, cps, st);
 }
 
+// ------------------------------------------------- symmetric pairs
+// The pair term of x_bar is antisymmetric under j <-> k (the VJP is the
+// gradient of a function of the displacements), so each unordered pair is
+// evaluated once (nb_wsym.cuh): with w = m_k c_j - m_j c_k and
+//   f = r^3 (w - (3 r^2 (d . w) + m_k pbar_j + m_j pbar_k) d),
+// x_bar_k += f, x_bar_j -= f, and the mass sums
+//   M_k += r^3 (c_j . d) + r pbar_j,   M_j += r pbar_k - r^3 (c_k . d)
+// (m_bar = -G M).  37 packed FP32 operations per two unordered pairs (45
+// fused with the force, 42 with pbar; hi/lo displacement +6) instead of 2 x
+// 26 (2 x 31, 2 x 30).  w is formed before it meets r^3, so close pairs with
+// similar cotangents lose nothing to cancellation between m_k sum r^3 c_j
+// and c_k sum r^3 m_j.
+namespace {
+
+using namespace wsym;
+
+template <bool PB, bool FUSED, bool SPLIT>
+struct VjpPh {
+    // four i-slots a lane as two (x_a, x_b) pairs against one j-particle, 16
+    // warps of 128 registers: 944 us fused at 32768, against 1001 us for four
+    // broadcast i-slots against two j with 8 warps (268 / 276 us at 16384)
+    static constexpr bool IPAIR = true;
+    static constexpr int K = 2, WARPS = 16;
+    static constexpr int NJ = 7 + (PB ? 1 : 0) + (SPLIT ? 3 : 0);
+    static constexpr int NC = FUSED ? 7 : 4, GROUPS = FUSED ? 3 : 2;
+    static constexpr int JL = PB ? 8 : 7;  // planes from here on: x.lo y.lo z.lo
+    struct S {
+        float2 nx[K], ny[K], nz[K], m[K], ncx[K], ncy[K], ncz[K];
+        LoT<IPAIR> nxl[K], nyl[K], nzl[K], pb[K];
+        float2 a[K][NC];  // f(3) M (force 3)
+    };
+    static __device__ __forceinline__ constexpr int group(int e) { return e < 3 ? 0 : (e == 3 ? 1 : 2); }
+    static __device__ __forceinline__ constexpr bool jneg(int e) { return e != 3; }
+    static __device__ __forceinline__ double bound(const Params &p, int g) {
+        const double m = (double)__uint_as_float(__ldcg(p.mx + kMaxM));
+        const double c = (double)__uint_as_float(__ldcg(p.mx + kMaxC));
+        const double b = (double)__uint_as_float(__ldcg(p.mx + kMaxP));
+        if (g == 0) return m * (p.scale[0] * c + p.scale[1] * b);
+        return g == 1 ? p.scale[2] * c + p.scale[3] * b : p.scale[4] * m;
+    }
+    // packed planes: x y z m, cx cy cz, (pbar,) (x.lo y.lo z.lo)
+    static __device__ __forceinline__ const float *plane(const Params &p, int a) {
+        if (a < 4) return p.soa + a * p.Np;
+        if (a < JL) return p.csoa + (a - 4) * p.Np;
+        return p.soa + (4 + a - JL) * p.Np;
+    }
+    static __device__ __forceinline__ void set_i(S &s, int k, const float2 (&v)[NJ]) {
+        s.nx[k] = neg(v[0]);
+        s.ny[k] = neg(v[1]);
+        s.nz[k] = neg(v[2]);
+        s.m[k] = v[3];
+        s.ncx[k] = neg(v[4]);
+        s.ncy[k] = neg(v[5]);
+        s.ncz[k] = neg(v[6]);
+        if constexpr (PB) s.pb[k] = lo_of<IPAIR>(v[7]);
+        if constexpr (SPLIT) {
+            s.nxl[k] = lo_of<IPAIR>(neg(v[JL]));
+            s.nyl[k] = lo_of<IPAIR>(neg(v[JL + 1]));
+            s.nzl[k] = lo_of<IPAIR>(neg(v[JL + 2]));
+        }
+    }
+    template <bool SYM, bool SELF>
+    static __device__ __forceinline__ void step(S &s, const float2 e2, const float2 (&J)[NJ],
+                                                float2 (&T)[NC], int self_h) {
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+            float2 dx = add2(J[0], s.nx[k]);
+            float2 dy = add2(J[1], s.ny[k]);
+            float2 dz = add2(J[2], s.nz[k]);
+            if constexpr (SPLIT) {
+                dx = add2(dx, add2(J[JL], lo2(s.nxl[k])));
+                dy = add2(dy, add2(J[JL + 1], lo2(s.nyl[k])));
+                dz = add2(dz, add2(J[JL + 2], lo2(s.nzl[k])));
+            }
+            float2 r2 = fma2(dx, dx, e2);
+            r2 = fma2(dy, dy, r2);
+            r2 = fma2(dz, dz, r2);
+            float2 r = f2(rsqrt_approx(r2.x), rsqrt_approx(r2.y));
+            if (SELF) r = mask_self<IPAIR>(r, k, self_h);
+            const float2 wx = fma2(s.m[k], J[4], mul2(J[3], s.ncx[k]));
+            const float2 wy = fma2(s.m[k], J[5], mul2(J[3], s.ncy[k]));
+            const float2 wz = fma2(s.m[k], J[6], mul2(J[3], s.ncz[k]));
+            float2 dw = mul2(dx, wx);
+            dw = fma2(dy, wy, dw);
+            dw = fma2(dz, wz, dw);
+            const float2 rr = mul2(r, r);
+            const float2 r3 = mul2(rr, r);
+            float2 q;
+            if constexpr (PB) {
+                // -(m_k pbar_j + m_j pbar_k) - 3 r^2 (d . w)
+                const float2 E = fma2(s.m[k], J[7], mul2(J[3], lo2(s.pb[k])));
+                q = fma2(mul2(rr, f2(-3.f, -3.f)), dw, f2(-E.x, -E.y));
+            } else {
+                q = mul2(mul2(rr, f2(-3.f, -3.f)), dw);
+            }
+            const float2 ex = fma2(q, dx, wx);
+            const float2 ey = fma2(q, dy, wy);
+            const float2 ez = fma2(q, dz, wz);
+            s.a[k][0] = fma2(r3, ex, s.a[k][0]);
+            s.a[k][1] = fma2(r3, ey, s.a[k][1]);
+            s.a[k][2] = fma2(r3, ez, s.a[k][2]);
+            float2 dcj = mul2(dx, J[4]);
+            dcj = fma2(dy, J[5], dcj);
+            dcj = fma2(dz, J[6], dcj);
+            s.a[k][3] = fma2(r3, dcj, s.a[k][3]);
+            if constexpr (PB) s.a[k][3] = fma2(r, J[7], s.a[k][3]);
+            if constexpr (FUSED) {
+                const float2 sj = mul2(J[3], r3);
+                s.a[k][4] = fma2(sj, dx, s.a[k][4]);
+                s.a[k][5] = fma2(sj, dy, s.a[k][5]);
+                s.a[k][6] = fma2(sj, dz, s.a[k][6]);
+            }
+            if (SYM) {
+                float2 dck = mul2(dx, s.ncx[k]);  // -(c_k . d)
+                dck = fma2(dy, s.ncy[k], dck);
+                dck = fma2(dz, s.ncz[k], dck);
+                T[0] = k ? fma2(r3, ex, T[0]) : mul2(r3, ex);
+                T[1] = k ? fma2(r3, ey, T[1]) : mul2(r3, ey);
+                T[2] = k ? fma2(r3, ez, T[2]) : mul2(r3, ez);
+                T[3] = k ? fma2(r3, dck, T[3]) : mul2(r3, dck);
+                if constexpr (PB) T[3] = fma2(r, lo2(s.pb[k]), T[3]);
+                if constexpr (FUSED) {
+                    const float2 si = mul2(s.m[k], r3);
+                    T[4] = k ? fma2(si, dx, T[4]) : mul2(si, dx);
+                    T[5] = k ? fma2(si, dy, T[5]) : mul2(si, dy);
+                    T[6] = k ? fma2(si, dz, T[6]) : mul2(si, dz);
+                }
+            }
+        }
+    }
+};
+
+// Positions, masses and cotangents in one pass: launch_pack's and
+// pack_cotangent_kernel's arrays, with the largest |m|, |c| and |pbar|.
+__global__ void __launch_bounds__(128) wsym_vjp_pack_kernel(
+    const double *pos, const double *mass,
+    const double *abar, const double *pbar, double *vbar,
+    const double *xbar, double drift, double coef, int step_form, int64_t N,
+    int64_t Np, float *soa, float *csoa, unsigned *mx) {
+    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;  // < Np: whole blocks
+    float hi[3] = {0.f, 0.f, 0.f}, lo[3] = {0.f, 0.f, 0.f}, cf[3] = {0.f, 0.f, 0.f};
+    float m = 0.f, pb = 0.f, ac = 0.f;
+    dev::grid_trigger();
+    dev::grid_wait();
+    if (i < N) {
+#pragma unroll
+        for (int e = 0; e < 3; ++e) {
+            const double x = pos[3 * i + e];
+            hi[e] = __double2float_rn(x);
+            lo[e] = __double2float_rn(x - (double)hi[e]);
+            double c;
+            if (step_form) {
+                const double v = vbar[3 * i + e] + drift * xbar[3 * i + e];
+                vbar[3 * i + e] = v;
+                c = coef * v;
+            } else {
+                c = coef * abar[3 * i + e];
+            }
+            cf[e] = __double2float_rn(c);
+            ac = fmaxf(ac, fabsf(cf[e]));
+        }
+        m = __double2float_rn(mass[i]);
+        if (!step_form && pbar) pb = __double2float_rn(coef * pbar[i]);
+    }
+    store_packed(soa, Np, i, hi, lo, m);
+#pragma unroll
+    for (int e = 0; e < 3; ++e) csoa[e * Np + i] = cf[e];
+    csoa[3 * Np + i] = pb;
+    warp_max(mx + kMaxM, fabsf(m));
+    warp_max(mx + kMaxC, ac);
+    warp_max(mx + kMaxP, fabsf(pb));
+}
+
+// The totals of every particle: read and zeroed, x G, stored or added;
+// FUSED: the acceleration and the rewind, as vjp_epilogue.
+template <bool FUSED>
+__global__ void __launch_bounds__(128) wsym_vjp_fold_kernel(const Params p, const VjpParams q,
+                                                            unsigned *mx) {
+    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    dev::grid_trigger();
+    dev::grid_wait();
+    if (i == 0) mx[kMaxM] = mx[kMaxC] = mx[kMaxP] = 0u;  // the pair kernel has read them
+    if (i >= p.N) return;
+    const int Fx = p.fxe[0], Fm = p.fxe[1];
+    bool ok = true;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        const double g = q.G * take_fixed(p, c, i, Fx);
+        q.pos_bar[3 * i + c] = q.accumulate ? q.pos_bar[3 * i + c] + g : g;
+        ok = ok && isfinite(g);
+    }
+    const double gm = -q.G * take_fixed(p, 3, i, Fm);
+    q.mass_bar[i] = q.accumulate ? q.mass_bar[i] + gm : gm;
+    ok = ok && isfinite(gm);
+    if (FUSED) {
+        const int Fa = p.fxe[2];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            const double a = q.G * take_fixed(p, 4 + c, i, Fa);
+            q.acc_out[3 * i + c] = a;
+            const double vh = q.vhalf[3 * i + c] - q.rewind_kick * a;
+            q.vhalf[3 * i + c] = vh;
+            q.pos_rw[3 * i + c] -= q.rewind_drift * vh;
+            ok = ok && isfinite(a);
+        }
+    }
+    if (!ok) dev::set_status(p.status, kStatusNonFinite);
+}
+
+int launch_vjp_wsym(const VjpJob &j, bool pb, bool fused) {
+    if (fused && pb) return fail(NB_ERR_UNSUPPORTED, "fused force with pot_bar is not built");
+    unsigned *mx = reinterpret_cast<unsigned *>(j.ws + j.L.wsym_head + 128);
+    float *soa = reinterpret_cast<float *>(j.ws + j.L.packA);
+    float *csoa = reinterpret_cast<float *>(j.ws + j.L.packB);
+    Params p{};
+    p.soa = soa;
+    p.csoa = csoa;
+    p.Np = j.L.Np;
+    p.N = j.N;
+    const float ef = (float)j.eps;
+    p.eps2 = ef * ef;
+    p.keep = true;
+    p.fx = reinterpret_cast<unsigned long long *>(j.ws + j.L.wsym_fx);
+    p.fxe = reinterpret_cast<int *>(j.ws + j.L.wsym_head + 64);
+    p.mx = mx;
+    p.status = reinterpret_cast<uint32_t *>(j.ws + j.L.status);
+    // a-priori bounds on every partial and total, with |w| <= 2 sqrt(3) max|m|
+    // max|c|, |e| r^3 <= 1.146 |w| / eps^3 (nb_jerk.cu), |d| r^3 <= 0.385 /
+    // eps^2 and r <= 1 / eps
+    const double n = 1.02 * (double)j.N, e1 = 1.0 / j.eps, e2 = 0.3849002 * e1 * e1;
+    p.scale[0] = n * 1.146 * 3.4641017 * e1 * e1 * e1;
+    p.scale[1] = n * 2.0 * e2;
+    p.scale[2] = n * 1.7320509 * e2;
+    p.scale[3] = n * e1;
+    p.scale[4] = n * e2;
+    int rc = launch_pdl(wsym_vjp_pack_kernel, (unsigned)(j.L.Np / 128), 128, 0, j.stream, j.pos,
+                        j.mass, j.acc_bar, j.pot_bar, j.vel_bar, j.pos_bar, j.drift_dt,
+                        j.kick_coef, j.step_form ? 1 : 0, j.N, j.L.Np, soa, csoa, mx);
+    if (rc) return rc;
+    if (fused)
+        rc = j.split ? launch_pairs<VjpPh<false, true, true>>(p, j.stream)
+                     : launch_pairs<VjpPh<false, true, false>>(p, j.stream);
+    else if (pb)
+        rc = j.split ? launch_pairs<VjpPh<true, false, true>>(p, j.stream)
+                     : launch_pairs<VjpPh<true, false, false>>(p, j.stream);
+    else
+        rc = j.split ? launch_pairs<VjpPh<false, false, true>>(p, j.stream)
+                     : launch_pairs<VjpPh<false, false, false>>(p, j.stream);
+    if (rc) return rc;
+    VjpParams q{};
+    q.G = j.G;
+    q.pos_bar = j.pos_bar;
+    q.mass_bar = j.mass_bar;
+    q.accumulate = j.accumulate ? 1 : 0;
+    q.acc_out = j.acc_out;
+    q.vhalf = j.vhalf;
+    q.pos_rw = j.pos_rw;
+    q.rewind_kick = j.rewind_kick;
+    q.rewind_drift = j.rewind_drift;
+    auto fold = fused ? wsym_vjp_fold_kernel<true> : wsym_vjp_fold_kernel<false>;
+    return launch_pdl(fold, (unsigned)cdiv(j.N, 128), 128, 0, j.stream, p, q, mx);
+}
+
+}  // namespace
+
 int launch_vjp(const VjpJob &j) {
     const bool guard = (j.eps == 0.0);
     const bool fused = j.acc_out != nullptr;
     const bool pb = !j.step_form && j.pot_bar != nullptr;
+    if (j.sym) return launch_vjp_wsym(j, pb, fused);
     uint32_t *status = reinterpret_cast<uint32_t *>(j.ws + j.L.status);
     float *csoa = reinterpret_cast<float *>(j.ws + j.L.packB);
     double *cdbl = reinterpret_cast<double *>(j.ws + j.L.cot64);

@@ -1,5 +1,6 @@
-// Warp-granular symmetric-pair evaluation of one system: the engine of
-// the forces (nb_wsym.cu) and the acceleration + jerk (nb_jerk.cu) when every pair takes the same displacement form.
+// Warp-granular symmetric-pair evaluation of one system: the engine shared by
+// the force (nb_wsym.cu), the VJP (nb_vjp.cu) and the acceleration + jerk
+// (nb_jerk.cu) when every pair takes the same displacement form.
 //
 // Each unordered pair is evaluated once for both particles, as in nb_sym.cu.
 // A warp keeps one block of i-slots in registers, four or eight per lane; the
