@@ -384,6 +384,9 @@ static int make_force_job(ForceJob *j, const double *pos, const double *mass, in
     // the default takes the symmetric path only where it applies (eps > 0);
     // an explicit NB_PAIRS_SYMMETRIC with eps = 0 is refused by the launcher
     j->sym = sym_wanted(o, N, 1) && (eps > 0.0 || o->pairs == NB_PAIRS_SYMMETRIC);
+    j->row = !j->sym && eps > 0.0 && o->precision != NB_PREC_FP64 &&
+             o->pairs == NB_PAIRS_DEFAULT && !shape_asked(o) &&
+             o->positions != NB_POS_ADAPTIVE && o->test_unissued_stage == 0 && row_fits(N);
     j->timeout = timeout_of(o);
     j->unissued = unissued_of(o);
     j->stream = (cudaStream_t)o->stream;
@@ -649,6 +652,7 @@ int nb_forces_range(const double *pos, const double *mass, int64_t N, int64_t i0
     // rows of the whole system in particle order: the direct kernel, no
     // Hilbert sort (ADAPTIVE is taken as SPLIT)
     j.sym = false;
+    j.row = false;
     j.adaptive = false;
     return launch_force(j);
 }
@@ -751,6 +755,10 @@ static int step_single_direct(nb_state *s, double dt, int64_t nsteps, const nb_o
     if (takes_wsym(j)) {
         if (nsteps == 0 && s->acc_valid) return NB_OK;
         return launch_step_wsym(j, s->vel, dt, nsteps, s->acc_valid != 0);
+    }
+    if (j.row) {
+        if (nsteps == 0 && s->acc_valid) return NB_OK;
+        return launch_step_row(j, s->vel, dt, nsteps, s->acc_valid != 0);
     }
     int64_t sorted_at = -1;  // step index of the last full Hilbert sort
     // the potential is evaluated only where the caller can see it: a

@@ -518,6 +518,7 @@ int launch_force(const ForceJob &j) {
     char *sb = j.ws + j.L.sortbuf;
     if (j.sym && guard) return fail(NB_ERR_UNSUPPORTED, "symmetric pairs need eps > 0");
     if (takes_wsym(j)) return launch_force_wsym(j);
+    if (j.row) return launch_force_row(j);
     if (adaptive) {
         // boxes per 64 j-slots and per warp of i-slots (direct kernel: 32 IR
         // slots; symmetric FP32 kernel: 256 slots)

@@ -144,6 +144,7 @@ struct ForceJob {
     float gamma;        // near/far threshold of the adaptive path
     bool packed_ready;  // packA already holds float positions of `pos`
     bool sym;           // symmetric-pair evaluation (nb_pairs resolved)
+    bool row;           // small systems: the row kernel
     long long timeout;
     int64_t unissued;  // test hook (nb_opts.test_unissued_stage - 1; -1: off)
     cudaStream_t stream;
@@ -227,8 +228,8 @@ constexpr int64_t kSymBlock = 2048;
 // totals, 268 MB at N = 2^22, plus 12 B per block pair of the adaptive path's
 // cost estimates, 25 MB at 2^22, 400 MB at 2^24).  Below kSymMinN, from
 // kWsymMinN, what has no use for a direct-kernel option takes the
-// warp-granular path (F64ACC step, direct / warp-granular: 34.6 / 19.4 us at
-// 4095, 77.5 / 40.9 at 8192).
+// warp-granular path (F64ACC step, row kernel / warp-granular: 16.5 / 19.4 us
+// at 4095, 19.6 / 19.2 at 4800, 30 / 27 at 6000).
 constexpr int64_t kSymMinN = 24576;
 constexpr int64_t kSymMaxN = 1 << 24;
 constexpr int64_t kWsymMinN = 4800;
@@ -270,6 +271,11 @@ inline bool takes_wsym(const ForceJob &j) {
 }
 int launch_force_wsym(const ForceJob &job);
 int launch_step_wsym(const ForceJob &job, double *vel, double dt, int64_t nsteps, bool acc_valid);
+
+// Small systems (nb_row.cu): whole rows per CTA, one kernel per evaluation.
+bool row_fits(int64_t N);
+int launch_force_row(const ForceJob &job);
+int launch_step_row(const ForceJob &job, double *vel, double dt, int64_t nsteps, bool acc_valid);
 
 struct VjpJob {
     const double *pos;
