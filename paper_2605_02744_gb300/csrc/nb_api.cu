@@ -384,6 +384,8 @@ static int make_force_job(ForceJob *j, const double *pos, const double *mass, in
     // the default takes the symmetric path only where it applies (eps > 0);
     // an explicit NB_PAIRS_SYMMETRIC with eps = 0 is refused by the launcher
     j->sym = sym_wanted(o, N, 1) && (eps > 0.0 || o->pairs == NB_PAIRS_SYMMETRIC);
+    if (o->precision == NB_PREC_FP64 && o->pairs == NB_PAIRS_DEFAULT)
+        j->sym = eps > 0.0 && N >= kSym64MinN && N <= kSymMaxN;
     j->row = !j->sym && eps > 0.0 && o->precision != NB_PREC_FP64 &&
              o->pairs == NB_PAIRS_DEFAULT && !shape_asked(o) &&
              o->positions != NB_POS_ADAPTIVE && o->test_unissued_stage == 0 && row_fits(N);
@@ -565,6 +567,20 @@ int nb_check_fp_conversions(int64_t n, uint64_t seed, int64_t *mismatches) {
             sum += (__int128)m * ((__int128)1 << sh);
         }
         if (fx::limb_value(x, Fs) != std::ldexp((double)sum, -Fs)) ++bad;
+        // an FP64 value by itself: exact unless its last bits are below the grid
+        const uint64_t de = (uint64_t)(1023 - F + (int)((r >> 20) % 200) - 10);
+        const double d = fpconv::from_bits_d((next() & 0x800fffffffffffffull) | (de << 52));
+        long long y[fx::kLimbs + 2] = {}, t[3], yl[fx::kLimbs];
+        int q = 0;
+        const bool dfits = (int)de - 1022 + F <= fx::kLimbs * fx::kLimbBits;
+        if (fx::split_limbs(d, F, q, t) != dfits) {
+            ++bad;
+        } else if (dfits) {
+            for (int i = 0; i < 3; ++i) y[q + i] += t[i];
+            for (int i = 0; i < fx::kLimbs; ++i) yl[i] = y[i];
+            const double err = std::fabs(fx::limb_value(yl, F) - d);
+            if (err > ((int)de - 1075 + F >= 0 ? 0.0 : std::ldexp(0.5, -F))) ++bad;
+        }
     }
     *mismatches = bad;
     return NB_OK;
@@ -752,6 +768,10 @@ static int step_single_direct(nb_state *s, double dt, int64_t nsteps, const nb_o
     ForceJob j;
     NB_TRY(make_force_job(&j, s->pos, s->mass, s->N, s->eps, s->acc, s->pot, s->ws, s->ws_bytes, o));
     j.adaptive = positions_adaptive(o, s->N, nsteps > 0);
+    if (takes_sym64(j)) {
+        if (nsteps == 0 && s->acc_valid) return NB_OK;
+        return launch_step_sym64(j, s->vel, dt, nsteps, s->acc_valid != 0);
+    }
     if (takes_wsym(j)) {
         if (nsteps == 0 && s->acc_valid) return NB_OK;
         return launch_step_wsym(j, s->vel, dt, nsteps, s->acc_valid != 0);

@@ -224,6 +224,39 @@ __host__ __device__ inline bool split_limbs(float v, int F, int &q, long long &l
     return true;
 }
 
+// The same for an FP64 value: limbs q, q + 1, q + 2 gain t[0..2].
+__host__ __device__ inline bool split_limbs(double v, int F, int &q, long long (&t)[3]) {
+    unsigned long long b;
+    memcpy(&b, &v, 8);
+    const int be = (int)((b >> 52) & 0x7ffu);
+    q = 0;
+    t[0] = t[1] = t[2] = 0;
+    if (be == 0x7ff) return false;  // inf or NaN
+    unsigned long long m = b & 0xfffffffffffffull;
+    if (be) m |= 1ull << 52;
+    if (!m) return true;  // +-0
+    int s = (be ? be : 1) - 1075 + F;  // X = m 2^s
+    if (s < 0) {
+        if (s < -54) return true;  // below half a grid step
+        m = (m + (1ull << (-s - 1))) >> (-s);
+        s = 0;
+    }
+    const unsigned long long mask = (1ull << kLimbBits) - 1;
+    q = s / kLimbBits;
+    const int r = s - q * kLimbBits;
+    const unsigned __int128 X = (unsigned __int128)m << r;  // < 2^97
+    const unsigned long long l[3] = {(unsigned long long)X & mask,
+                                     (unsigned long long)(X >> kLimbBits) & mask,
+                                     (unsigned long long)(X >> (2 * kLimbBits))};
+    if (q >= kLimbs || (q >= kLimbs - 1 && l[1]) || (q >= kLimbs - 2 && l[2])) {
+        q = 0;
+        return false;
+    }
+#pragma unroll
+    for (int k = 0; k < 3; ++k) t[k] = (b >> 63) ? -(long long)l[k] : (long long)l[k];
+    return true;
+}
+
 // The accumulated value of the limbs, rounded once to double.
 __host__ __device__ inline double limb_value(const long long (&w)[kLimbs], int F) {
     long long t[kLimbs];

@@ -497,7 +497,7 @@ int launch_force(const ForceJob &j) {
     if (j.precision == NB_PREC_FP64) {
         if (j.sym) {
             if (guard) return fail(NB_ERR_UNSUPPORTED, "symmetric pairs need eps > 0");
-            return launch_force_sym(j);
+            if (takes_sym64(j)) return launch_force_sym64(j);
         }
         constexpr int NT = 128;
         const int64_t grid = cdiv(j.ni, NT);

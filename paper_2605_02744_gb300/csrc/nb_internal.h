@@ -239,6 +239,9 @@ constexpr int64_t kWsymMinN = 4800;
 // share out).
 constexpr int64_t kWsymVjpMinN = 256;
 constexpr int64_t kWsymJerkMinN = 256;
+// FP64 pairs: from one block of 64 on (direct / symmetric: 49 / 16 us at 64, 683 /
+// 36 at 1024).
+constexpr int64_t kSym64MinN = 64;
 constexpr int kWsymComponents = 7;  // sums per particle at most
 // Largest system of the warp-granular path (its accumulators take 2^19 adds,
 // one per block of 128 slots and range end); an explicit request for
@@ -271,6 +274,14 @@ inline bool takes_wsym(const ForceJob &j) {
 }
 int launch_force_wsym(const ForceJob &job);
 int launch_step_wsym(const ForceJob &job, double *vel, double dt, int64_t nsteps, bool acc_valid);
+
+// FP64 pairs, each unordered pair once (nb_sym64.cu): one evaluation, and an
+// nb_step loop's.
+inline bool takes_sym64(const ForceJob &j) {
+    return j.sym && j.eps > 0.0 && j.precision == NB_PREC_FP64 && j.N <= kWsymMaxN;
+}
+int launch_force_sym64(const ForceJob &job);
+int launch_step_sym64(const ForceJob &job, double *vel, double dt, int64_t nsteps, bool acc_valid);
 
 // Small systems (nb_row.cu): whole rows per CTA, one kernel per evaluation.
 bool row_fits(int64_t N);

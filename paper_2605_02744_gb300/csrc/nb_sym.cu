@@ -68,10 +68,6 @@
 // closer than gamma * max|x| (a 32-bit mask per warp and item, from the
 // Hilbert-sorted pack's boxes of 256 i- and 64 j-slots), single floats
 // elsewhere.  Systems with one form for every pair go to nb_wsym.cu.
-//
-// FP64 pairs (force_sym64_kernel) keep the first form of this kernel: 16
-// warps of 128 slots (4 per lane, doubles), 32-slot j-sets of one particle
-// per lane, scalar j-side sums.
 #include <cuda_runtime.h>
 
 #include <stdlib.h>
@@ -108,8 +104,7 @@ using namespace symj;
 constexpr int BI = 2048;            // slots per row block
 static_assert(BI == kSymBlock, "row block size");
 constexpr int CPS = 1;              // resident CTAs per SM
-constexpr int US = 16;              // stream-K units per item (both kernels)
-// FP32 pairs (force_sym_kernel)
+constexpr int US = 16;              // stream-K units per item
 constexpr int NW = 8;               // warps per CTA
 constexpr int NT = NW * 32;         // threads per CTA
 constexpr int IRP = 8;              // i-slots per lane
@@ -122,19 +117,12 @@ constexpr int FL2P = 16;            // F64ACC: j-sets per FP64 add of the FP32 m
                                     // (1024 pair terms; 8 j-sets: 341.4 ms at 2^20, 16: 334.5)
 static_assert(NW * WS == BI && NJSP == 32 && NJSP / KBP == US, "FP32 kernel shape");
 constexpr size_t kRedBytes = 2 * KBP * 2 * NW * 32 * sizeof(float4);
-// FP64 pairs (force_sym64_kernel)
-constexpr int SW = 16;              // warps per CTA
-constexpr int SNT = SW * 32;        // threads per CTA
-constexpr int NJS = BI / JS;        // 32-slot j-sets per block
-constexpr int KB = 4;               // j-sets per cross-warp reduction
-static_assert(SW * 32 * IR == BI && NJS / KB == US, "FP64 kernel shape");
-
 struct SymParams {
     const float *soa;   // packed SoA [7][Np]
     int64_t Np;
     int64_t nb;         // row blocks
     int64_t T;          // items nb (nb + 1) / 2
-    int64_t U;          // stream-K units T * US (KB j-sets of one item each)
+    int64_t U;          // stream-K units T * US (KBP j-sets of one item each)
     int64_t ctas;       // grid size of the pair kernel
     float eps2;
     float gamma;        // adaptive threshold; the mode decides whether it is used
@@ -144,14 +132,6 @@ struct SymParams {
     const int *fx_exp;           // the call's fixed-point exponent F
     const int64_t *lo;  // [ctas + 1]: CTA c owns units [lo[c], lo[c + 1])
     uint32_t *status;
-};
-
-// FP64 pairs: the common layout plus positions [N][3] and masses in
-// particle order.
-struct SymParams64 : SymParams {
-    const double *pos64, *mass64;
-    int64_t N;
-    double eps2_64;
 };
 
 __host__ __device__ inline int64_t row_start(int64_t I, int64_t nb) {
@@ -404,175 +384,6 @@ __global__ void __launch_bounds__(256) sym_exponent_kernel(const double *__restr
     }
 }
 
-// ------------------------------------------------------------- FP64 pairs
-// The same decomposition with FP64 arithmetic throughout (positions, pairs,
-// sums), for the FP64 policy: each unordered pair once, its j-side sums
-// rotated through the lanes as doubles.  The slots are the particles in
-// their own order (no packing, no near/far choice); one rsqrt per unordered
-// pair instead of two.
-struct alignas(16) D4 {
-    double x, y, z, w;
-};
-
-struct ISet64 {
-    double x[IR], y[IR], z[IR], m[IR];
-    double ax[IR], ay[IR], az[IR], ph[IR];
-};
-
-template <bool SYM, bool SELF, bool POT>
-__device__ __forceinline__ void step64(ISet64 &S, double eps2, double jx, double jy, double jz,
-                                       double jm, double &bx, double &by, double &bz, double &bp,
-                                       int self_k) {
-#pragma unroll
-    for (int k = 0; k < IR; ++k) {
-        const double mj = (SELF && k == self_k) ? 0.0 : jm;
-        const double dx = jx - S.x[k], dy = jy - S.y[k], dz = jz - S.z[k];
-        const double r2 = fma(dx, dx, fma(dy, dy, fma(dz, dz, eps2)));
-        const double ri = rsqrt(r2);
-        const double ri3 = ri * ri * ri;
-        const double sj = mj * ri3;
-        S.ax[k] = fma(sj, dx, S.ax[k]);
-        S.ay[k] = fma(sj, dy, S.ay[k]);
-        S.az[k] = fma(sj, dz, S.az[k]);
-        if (POT) S.ph[k] = fma(mj, ri, S.ph[k]);
-        if (SYM) {
-            const double si = S.m[k] * ri3;
-            bx = fma(-si, dx, bx);
-            by = fma(-si, dy, by);
-            bz = fma(-si, dz, bz);
-            if (POT) bp = fma(S.m[k], ri, bp);
-        }
-    }
-}
-
-template <bool SYM, bool POT>
-__device__ __forceinline__ void rotate_set64(ISet64 &S, double eps2, const double (&j)[4],
-                                             D4 &b, int self_k) {
-    const int src = (threadIdx.x + 1) & 31;
-    double jx = j[0], jy = j[1], jz = j[2], jm = j[3];
-    double bx = 0.0, by = 0.0, bz = 0.0, bp = 0.0;
-    auto rotate = [&]() {
-        jx = __shfl_sync(0xffffffffu, jx, src);
-        jy = __shfl_sync(0xffffffffu, jy, src);
-        jz = __shfl_sync(0xffffffffu, jz, src);
-        jm = __shfl_sync(0xffffffffu, jm, src);
-        if (SYM) {
-            bx = __shfl_sync(0xffffffffu, bx, src);
-            by = __shfl_sync(0xffffffffu, by, src);
-            bz = __shfl_sync(0xffffffffu, bz, src);
-            if (POT) bp = __shfl_sync(0xffffffffu, bp, src);
-        }
-    };
-    int s0 = 0;
-    if (self_k >= 0) {
-        step64<SYM, true, POT>(S, eps2, jx, jy, jz, jm, bx, by, bz, bp, self_k);
-        rotate();
-        s0 = 1;
-    }
-#pragma unroll 2
-    for (int st = s0; st < JS; ++st) {
-        step64<SYM, false, POT>(S, eps2, jx, jy, jz, jm, bx, by, bz, bp, -1);
-        rotate();
-    }
-    b = D4{bx, by, bz, bp};
-}
-
-__device__ __forceinline__ void load_j64(const SymParams64 &p, int64_t s, double (&j)[4]) {
-    if (s < p.N) {
-        j[0] = __ldg(p.pos64 + 3 * s);
-        j[1] = __ldg(p.pos64 + 3 * s + 1);
-        j[2] = __ldg(p.pos64 + 3 * s + 2);
-        j[3] = __ldg(p.mass64 + s);
-    } else {
-        j[0] = j[1] = j[2] = j[3] = 0.0;  // padding: zero mass at the origin
-    }
-}
-
-constexpr size_t kRed64Bytes = 2 * KB * SW * 32 * sizeof(D4);
-
-template <bool POT>
-__global__ void __launch_bounds__(SNT, CPS) force_sym64_kernel(const SymParams64 p) {
-    extern __shared__ __align__(16) unsigned char smem64[];
-    D4 *red = reinterpret_cast<D4 *>(smem64);  // [2][KB][SW][32]
-    const int tid = threadIdx.x, w = tid >> 5, l = tid & 31;
-    const int64_t c = blockIdx.x;
-    int64_t u = __ldg(p.lo + c);
-    const int64_t u_end = __ldg(p.lo + c + 1);
-    if (u >= u_end) return;
-    const int F = __ldg(p.fx_exp);
-    const int64_t t0 = u / US;
-    int64_t I = 0;
-    while (row_start(I + 1, p.nb) <= t0) ++I;
-    int64_t J = I + (t0 - row_start(I, p.nb));
-    ISet64 S;
-    int half = 0;
-    bool row_open = false;
-    while (u < u_end) {
-        const int qa = (int)(u % US) * KB;
-        const int64_t item_end = (u / US + 1) * US;
-        const int64_t seg_end = item_end < u_end ? item_end : u_end;
-        const int qb = qa + (int)(seg_end - u) * KB;
-        const int64_t ib = I * BI + w * 128;
-        if (!row_open) {
-#pragma unroll
-            for (int k = 0; k < IR; ++k) {
-                double v[4];
-                load_j64(p, ib + 32 * k + l, v);
-                S.x[k] = v[0];
-                S.y[k] = v[1];
-                S.z[k] = v[2];
-                S.m[k] = v[3];
-                S.ax[k] = S.ay[k] = S.az[k] = S.ph[k] = 0.0;
-            }
-            row_open = true;
-        }
-        const bool sym = J != I;
-        const int64_t jb = J * BI;
-        double jn[4];
-        load_j64(p, jb + qa * JS + l, jn);
-        for (int q = qa; q < qb; ++q) {
-            double jc[4] = {jn[0], jn[1], jn[2], jn[3]};
-            if (q + 1 < qb) load_j64(p, jb + (q + 1) * JS + l, jn);
-            D4 b;
-            if (sym) {
-                rotate_set64<true, POT>(S, p.eps2_64, jc, b, -1);
-                red[((half * KB + (q % KB)) * SW + w) * 32 + l] = b;
-            } else {
-                rotate_set64<false, POT>(S, p.eps2_64, jc, b, (q >> 2) == w ? (q & 3) : -1);
-            }
-            if (sym && (q + 1) % KB == 0) {
-                __syncthreads();
-                for (int v = tid; v < KB * JS * 4; v += SNT) {
-                    const int qq = v >> 7, ll = (v >> 2) & 31, e = v & 3;
-                    const double *r = reinterpret_cast<const double *>(red) +
-                                      ((half * KB + qq) * SW * 32 + ll) * 4 + e;
-                    double sum = 0.0;
-#pragma unroll
-                    for (int w2 = 0; w2 < SW; ++w2) sum += r[w2 * 32 * 4];
-                    if (POT || e < 3) add_fixed(p, e, jb + (q + 1 - KB + qq) * JS + ll, sum, F);
-                }
-                half ^= 1;
-            }
-        }
-        u = seg_end;
-        if ((J == p.nb - 1 && qb == NJS) || u == u_end) {
-#pragma unroll
-            for (int kk = 0; kk < IR; ++kk) {
-                const int64_t slot = I * BI + w * 128 + 32 * kk + l;
-                add_fixed(p, 0, slot, S.ax[kk], F);
-                add_fixed(p, 1, slot, S.ay[kk], F);
-                add_fixed(p, 2, slot, S.az[kk], F);
-                if (POT) add_fixed(p, 3, slot, S.ph[kk], F);
-            }
-            row_open = false;
-        }
-        if (qb == NJS && ++J == p.nb) {
-            ++I;
-            J = I;
-        }
-    }
-}
-
 // ------------------------------------------------ cost-weighted stream-K
 // Relative cost of a stream-K unit (KBP j-sets of an item, at whose end
 // the CTA's warps meet at a barrier): the slowest warp's FP32-pipe cycles
@@ -582,7 +393,7 @@ __global__ void __launch_bounds__(SNT, CPS) force_sym64_kernel(const SymParams64
 // times grew with their number of units (regression slope ~40 % of a
 // unit's mean time); with 28 the last CTA of a 2^20 Plummer evaluation ends
 // 0.2 % after the mean (0.9 % with the earlier per-item sum of all warps'
-// j-sets), of a 2^18 one 1.1 %.  The FP64 kernel's units all cost the same.
+// j-sets), of a 2^18 one 1.1 %.
 constexpr uint32_t kCostSymFar = 18, kCostSymNear = 24, kCostDiagFar = 13, kCostDiagNear = 19;
 constexpr uint32_t kCostSymUnit = 28;
 
@@ -598,7 +409,7 @@ __device__ __forceinline__ void item_of(int64_t t, int64_t nb, int64_t &I, int64
 }
 
 // The adaptive FP32 kernel's unit costs of item t, one thread: the same
-// sums as sym_cost_kernel<true, NW, JSP> (which adds them up per item).
+// sums as sym_cost_kernel (which adds them up per item).
 __device__ void item_unit_costs(const SymParams &p, int64_t t, uint32_t (&uc)[US]) {
     int64_t I, J;
     item_of(t, p.nb, I, J);
@@ -622,14 +433,11 @@ __device__ void item_unit_costs(const SymParams &p, int64_t t, uint32_t (&uc)[US
     for (int u = 0; u < US; ++u) uc[u] += kCostSymUnit;
 }
 
-// One warp per item: the near/far decisions the pair kernel will take.  For
-// the FP32 kernel lane l takes j-set l (unit l / 2): the unit's cost is the
-// maximum over the warps of its two j-sets' sum; for FP64 pairs every unit
-// costs the same.
-template <bool NEARFAR, int NWK, int JSET>
+// One warp per item: the near/far decisions the pair kernel will take.  Lane l
+// takes j-set l (unit l / 2): the unit's cost is the maximum over the warps of
+// its two j-sets' sum.
 __global__ void __launch_bounds__(256) sym_cost_kernel(const SymParams p, uint32_t *cost) {
-    constexpr int NJ = BI / JSET;  // j-sets per block
-    constexpr int WS = BI / NWK;   // i-slots per warp
+    static_assert(NJSP == 32 && KBP == 2, "lane l: j-set l, unit l / 2");
     const int64_t t = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     const int l = threadIdx.x & 31;
     if (t >= p.T) return;  // whole warps
@@ -638,25 +446,19 @@ __global__ void __launch_bounds__(256) sym_cost_kernel(const SymParams p, uint32
     const bool sym = I != J;
     const uint32_t cn = sym ? kCostSymNear : kCostDiagNear;
     const uint32_t cf = sym ? kCostSymFar : kCostDiagFar;
-    uint32_t c = 0;
-    if constexpr (!NEARFAR) {
-        c = (l & 1) ? 0u : 2 * cf + kCostSymUnit;
-    } else {
-        static_assert(NJ == 32 && KBP == 2 && NWK == NW, "lane l: j-set l, unit l / 2");
-        float tb[7];
+    float tb[7];
 #pragma unroll
-        for (int a = 0; a < 7; ++a) tb[a] = __ldg(p.jbox + (J * NJ + l) * 8 + a);
-        uint32_t m = 0;
-        for (int w = 0; w < NWK; ++w) {
-            float wb[7];
+    for (int a = 0; a < 7; ++a) tb[a] = __ldg(p.jbox + (J * NJSP + l) * 8 + a);
+    uint32_t m = 0;
+    for (int w = 0; w < NW; ++w) {
+        float wb[7];
 #pragma unroll
-            for (int a = 0; a < 7; ++a) wb[a] = __ldg(p.wbox + ((I * BI + w * WS) / WS) * 8 + a);
-            const uint32_t v = boxes_near(wb, tb, p.gamma) ? cn : cf;
-            const uint32_t pair = v + __shfl_xor_sync(0xffffffffu, v, 1);
-            m = pair > m ? pair : m;
-        }
-        c = (l & 1) ? 0u : m + kCostSymUnit;
+        for (int a = 0; a < 7; ++a) wb[a] = __ldg(p.wbox + (I * NW + w) * 8 + a);
+        const uint32_t v = boxes_near(wb, tb, p.gamma) ? cn : cf;
+        const uint32_t pair = v + __shfl_xor_sync(0xffffffffu, v, 1);
+        m = pair > m ? pair : m;
     }
+    uint32_t c = (l & 1) ? 0u : m + kCostSymUnit;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
     if (l == 0) cost[t] = c;
@@ -691,10 +493,8 @@ __global__ void __launch_bounds__(1024) sym_scan_kernel(const uint32_t *cost, in
 }
 
 // lo[c] = the unit where the cumulative cost reaches c / ctas of the total
-// (the nearest unit boundary, from the item's unit costs for the adaptive
-// kernel, linearly inside an item otherwise); lo[0] = 0, lo[ctas] = U,
+// (the nearest unit boundary, from the item's unit costs); lo[0] = 0, lo[ctas] = U,
 // non-decreasing.
-template <bool NEARFAR>
 __global__ void sym_ranges_kernel(const SymParams p, const uint32_t *cost,
                                   const unsigned long long *prefix, int64_t T, int64_t ctas,
                                   int64_t *lo) {
@@ -714,18 +514,12 @@ __global__ void sym_ranges_kernel(const SymParams p, const uint32_t *cost,
                 b = m - 1;
         }
         const unsigned long long r = target - prefix[a];
-        int64_t off;
-        if (NEARFAR) {
-            uint32_t uc[US];
-            item_unit_costs(p, a, uc);
-            unsigned long long run = 0;
-            off = 0;
-            while (off < US && run + uc[off] <= r) run += uc[off++];
-            if (off < US && 2 * (r - run) > uc[off]) ++off;  // the nearer boundary
-        } else {
-            off = (int64_t)(r * (unsigned long long)US / cost[a]);
-            if (off > US) off = US;
-        }
+        uint32_t uc[US];
+        item_unit_costs(p, a, uc);
+        unsigned long long run = 0;
+        int64_t off = 0;
+        while (off < US && run + uc[off] <= r) run += uc[off++];
+        if (off < US && 2 * (r - run) > uc[off]) ++off;  // the nearer boundary
         lo[c] = a * US + off;
     }
 }
@@ -746,16 +540,10 @@ int launch_pair(const SymParams &p, cudaStream_t st) {
     return NB_OK;
 }
 
-// FP64: units of equal cost; FP32: the near/far estimate per (8 warps x
-// 64-slot j-sets).
-template <bool FP64>
 int launch_split(const SymParams &p, const ForceJob &j, const SymLayout &y) {
-    if constexpr (FP64)
-        sym_cost_kernel<false, SW, JS><<<(unsigned)cdiv(p.T * 32, 256), 256, 0, j.stream>>>(p, y.cost);
-    else
-        sym_cost_kernel<true, NW, JSP><<<(unsigned)cdiv(p.T * 32, 256), 256, 0, j.stream>>>(p, y.cost);
+    sym_cost_kernel<<<(unsigned)cdiv(p.T * 32, 256), 256, 0, j.stream>>>(p, y.cost);
     sym_scan_kernel<<<1, 1024, 0, j.stream>>>(y.cost, p.T, y.prefix);
-    sym_ranges_kernel<!FP64><<<(unsigned)cdiv(p.ctas + 1, 256), 256, 0, j.stream>>>(
+    sym_ranges_kernel<<<(unsigned)cdiv(p.ctas + 1, 256), 256, 0, j.stream>>>(
         p, y.cost, y.prefix, p.T, p.ctas, y.lo);
     sym_exponent_kernel<<<(unsigned)std::min<int64_t>(cdiv(j.N, 4 * 256), 1024), 256, 0,
                           j.stream>>>(j.mass, j.N, j.eps, y.fx_exp, y.mmax_bits, y.arrivals);
@@ -775,26 +563,9 @@ int launch_fold(const SymParams &p, const ForceJob &j, const int *perm) {
 
 template <int POL>
 int launch_sym_pol(const SymParams &p, const ForceJob &j, const SymLayout &y, const int *perm) {
-    NB_TRY_SYM(launch_split<false>(p, j, y));
+    NB_TRY_SYM(launch_split(p, j, y));
     NB_TRY_SYM(j.pot ? launch_pair<POL, true>(p, j.stream) : launch_pair<POL, false>(p, j.stream));
     return launch_fold(p, j, perm);
-}
-
-template <bool POT>
-int launch_pair64(const SymParams64 &p, cudaStream_t st) {
-    auto kern = force_sym64_kernel<POT>;
-    const int rc = smem_optin(reinterpret_cast<const void *>(kern), kRed64Bytes);
-    if (rc != NB_OK) return rc;
-    kern<<<(unsigned)p.ctas, SNT, kRed64Bytes, st>>>(p);
-    count_launch();
-    NB_CUDA(cudaGetLastError());
-    return NB_OK;
-}
-
-int launch_sym64(const SymParams64 &p, const ForceJob &j, const SymLayout &y) {
-    NB_TRY_SYM(launch_split<true>(p, j, y));
-    NB_TRY_SYM(j.pot ? launch_pair64<true>(p, j.stream) : launch_pair64<false>(p, j.stream));
-    return launch_fold(p, j, nullptr);
 }
 
 }  // namespace
@@ -850,15 +621,6 @@ int launch_force_sym(const ForceJob &j) {
     p.lo = y.lo;
     const int *perm = sort_perm(sb, j.L);
     p.status = reinterpret_cast<uint32_t *>(j.ws + j.L.status);
-    if (j.precision == NB_PREC_FP64) {
-        SymParams64 p64;
-        static_cast<SymParams &>(p64) = p;
-        p64.pos64 = j.pos;
-        p64.mass64 = j.mass;
-        p64.N = j.N;
-        p64.eps2_64 = j.eps * j.eps;
-        return launch_sym64(p64, j, y);
-    }
     switch (j.precision) {
         case NB_PREC_FP32: return launch_sym_pol<NB_PREC_FP32>(p, j, y, perm);
         case NB_PREC_KAHAN: return launch_sym_pol<NB_PREC_KAHAN>(p, j, y, perm);
