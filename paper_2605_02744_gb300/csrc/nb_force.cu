@@ -519,11 +519,11 @@ int launch_force(const ForceJob &j) {
     if (j.sym && guard) return fail(NB_ERR_UNSUPPORTED, "symmetric pairs need eps > 0");
     if (takes_wsym(j)) return launch_force_wsym(j);
     if (j.row) return launch_force_row(j);
+    if (j.sym && adaptive) return launch_force_sym(j);
     if (adaptive) {
-        // boxes per 64 j-slots and per warp of i-slots (direct kernel: 32 IR
-        // slots; symmetric FP32 kernel: 256 slots)
+        // boxes per 64 j-slots and per warp of i-slots (32 IR slots)
         const int tile_unit = 64;
-        const int block_unit = j.sym ? 256 : 32 * sh0.ipt;
+        const int block_unit = 32 * sh0.ipt;
         int rc = launch_sorted_pack(j.pos, j.mass, j.N, j.L.Np, soa, sort_perm(sb, j.L),
                                     sort_keys(sb), sort_box6(sb, j.L), sort_tile_boxes(sb, j.L),
                                     tile_unit, sort_block_boxes(sb, j.L), block_unit,
@@ -533,7 +533,6 @@ int launch_force(const ForceJob &j) {
         int rc = launch_pack(j.pos, j.mass, j.N, j.L.Np, soa, j.stream);
         if (rc) return rc;
     }
-    if (j.sym && adaptive) return launch_force_sym(j);
     const Shape &sh = j.shape;
     ForceParams p;
     p.soa = soa;

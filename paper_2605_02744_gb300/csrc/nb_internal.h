@@ -267,6 +267,7 @@ SymLayout sym_layout(char *ws, const WsLayout &L);
 // B clusters under opts (nb_pairs; FP32-pair policies, single systems).
 bool sym_wanted(const nb_opts *opts, int64_t N, int32_t B);
 int launch_force_sym(const ForceJob &job);
+int launch_step_sym(const ForceJob &job, double *vel, double dt, int64_t nsteps, bool acc_valid);
 // The warp-granular symmetric path (nb_wsym.cu; no adaptive displacement):
 // one evaluation, and an nb_step loop's evaluations with its O(N) work fused.
 inline bool takes_wsym(const ForceJob &j) {

@@ -126,8 +126,8 @@ struct SymParams {
     int64_t ctas;       // grid size of the pair kernel
     float eps2;
     float gamma;        // adaptive threshold; the mode decides whether it is used
-    const float *jbox;  // per 32 slots: lo[3], hi[3], max|x|, pad
-    const float *wbox;  // per 128 slots
+    const float *jbox;  // per 64 slots: lo[3], hi[3], max|x|, pad
+    const float *wbox;  // per 256 slots
     unsigned long long *acc_fx;  // [4 components][2 words][Np] fixed-point totals
     const int *fx_exp;           // the call's fixed-point exponent F
     const int64_t *lo;  // [ctas + 1]: CTA c owns units [lo[c], lo[c + 1])
@@ -340,6 +340,101 @@ __global__ void __launch_bounds__(256) sym_fold_kernel(const SymParams p, int64_
     if (bad) dev::set_status(p.status, kStatusNonFinite);
 }
 
+// Order-preserving image of a float as a signed integer, and back.
+__device__ __forceinline__ int ordered_f(float x) {
+    const int b = __float_as_int(x);
+    return b >= 0 ? b : b ^ 0x7fffffff;
+}
+__device__ __forceinline__ float from_ordered_f(int b) {
+    return __int_as_float(b >= 0 ? b : b ^ 0x7fffffff);
+}
+
+__device__ __forceinline__ void store_box(float *out, const float (&lo)[3], const float (&hi)[3]) {
+    float amax = 0.f;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        out[c] = lo[c];
+        out[3 + c] = hi[c];
+        amax = fmaxf(amax, fmaxf(fabsf(lo[c]), fabsf(hi[c])));
+    }
+    out[6] = hi[0] < lo[0] ? 0.f : amax;  // no real slot: never near
+    out[7] = 0.f;
+}
+
+// The fold of one step fused with the next one's opening where the Hilbert
+// order is kept: the totals (read and zeroed) x G, this step's closing kick,
+// the next one's opening kick and drift, the hi/lo pack of the new positions
+// in place and the boxes of 64 and 256 slots (a block is 256 slots), as
+// sym_fold_kernel, kick_drift_pack_kernel, pack_sorted_kernel and two
+// slot_boxes_kernel launches do one after the other.  The acceleration is not
+// stored: the next fold replaces it before anything reads it.  At 65536
+// particles the step's kernels besides the pair kernel took 76 us (ncu), the
+// ten launches of them; now four.
+__global__ void __launch_bounds__(256) sym_fold_next_kernel(
+    const SymParams p, int64_t N, const int *perm, double G, double *pos, double *vel, double kick,
+    double next_kick, double drift, float *soa, float *jbox, float *wbox) {
+    __shared__ int red[6][8];
+    const int64_t s = blockIdx.x * (int64_t)256 + threadIdx.x;
+    const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
+    dev::grid_trigger();
+    dev::grid_wait();
+    const int F = *p.fx_exp;
+    unsigned long long wd[6];
+#pragma unroll
+    for (int k = 0; k < 6; ++k) wd[k] = p.acc_fx[(int64_t)k * p.Np + s];
+#pragma unroll
+    for (int k = 0; k < 6; ++k)
+        if (wd[k]) p.acc_fx[(int64_t)k * p.Np + s] = 0ull;
+    int lo[3] = {ordered_f(3e38f), ordered_f(3e38f), ordered_f(3e38f)};
+    int hi[3] = {ordered_f(-3e38f), ordered_f(-3e38f), ordered_f(-3e38f)};
+    if (s < N) {
+        const int64_t i = perm[s];
+        bool ok = true;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            const double a = G * fx::value(wd[2 * c], wd[2 * c + 1], F);
+            ok = ok && isfinite(a);
+            double v = vel[3 * i + c] + kick * a;
+            v = v + next_kick * a;
+            const double x = pos[3 * i + c] + drift * v;
+            vel[3 * i + c] = v;
+            pos[3 * i + c] = x;
+            const float h = __double2float_rn(x);
+            soa[c * p.Np + s] = h;
+            soa[(4 + c) * p.Np + s] = __double2float_rn(x - (double)h);
+            lo[c] = hi[c] = ordered_f(h);
+        }
+        if (!ok) dev::set_status(p.status, kStatusNonFinite);
+    }
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        lo[c] = __reduce_min_sync(0xffffffffu, lo[c]);
+        hi[c] = __reduce_max_sync(0xffffffffu, hi[c]);
+        if (l == 0) {
+            red[c][w] = lo[c];
+            red[3 + c][w] = hi[c];
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x < 5) {  // four 64-slot boxes, then the block's
+        const int w0 = threadIdx.x < 4 ? 2 * threadIdx.x : 0, nw = threadIdx.x < 4 ? 2 : 8;
+        float bl[3], bh[3];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            int a = red[c][w0], b = red[3 + c][w0];
+            for (int k = 1; k < nw; ++k) {
+                a = min(a, red[c][w0 + k]);
+                b = max(b, red[3 + c][w0 + k]);
+            }
+            bl[c] = from_ordered_f(a);
+            bh[c] = from_ordered_f(b);
+        }
+        store_box(threadIdx.x < 4 ? jbox + (4 * (int64_t)blockIdx.x + threadIdx.x) * 8
+                                  : wbox + (int64_t)blockIdx.x * 8,
+                  bl, bh);
+    }
+}
+
 // The call's fixed-point exponent from the bound N max|m| max(0.385 / eps^2,
 // 1 / eps) (x 1.02 for the rounding of FP32 partial sums) on every partial
 // and total.  Every block takes the maximum of its share of the masses
@@ -408,39 +503,12 @@ __device__ __forceinline__ void item_of(int64_t t, int64_t nb, int64_t &I, int64
     J = r + (t - row_start(r, nb));
 }
 
-// The adaptive FP32 kernel's unit costs of item t, one thread: the same
-// sums as sym_cost_kernel (which adds them up per item).
-__device__ void item_unit_costs(const SymParams &p, int64_t t, uint32_t (&uc)[US]) {
-    int64_t I, J;
-    item_of(t, p.nb, I, J);
-    const bool sym = I != J;
-    const uint32_t cn = sym ? kCostSymNear : kCostDiagNear;
-    const uint32_t cf = sym ? kCostSymFar : kCostDiagFar;
-    for (int u = 0; u < US; ++u) uc[u] = 0;
-    for (int w = 0; w < NW; ++w) {
-        float wb[7];
-        for (int a = 0; a < 7; ++a) wb[a] = __ldg(p.wbox + (I * NW + w) * 8 + a);
-        for (int u = 0; u < US; ++u) {
-            uint32_t sum = 0;
-            for (int k = 0; k < KBP; ++k) {
-                float tb[7];
-                for (int a = 0; a < 7; ++a) tb[a] = __ldg(p.jbox + (J * NJSP + u * KBP + k) * 8 + a);
-                sum += boxes_near(wb, tb, p.gamma) ? cn : cf;
-            }
-            uc[u] = sum > uc[u] ? sum : uc[u];
-        }
-    }
-    for (int u = 0; u < US; ++u) uc[u] += kCostSymUnit;
-}
-
-// One warp per item: the near/far decisions the pair kernel will take.  Lane l
-// takes j-set l (unit l / 2): the unit's cost is the maximum over the warps of
-// its two j-sets' sum.
-__global__ void __launch_bounds__(256) sym_cost_kernel(const SymParams p, uint32_t *cost) {
+// The near/far decisions the pair kernel will take on item t, by a warp: lane l
+// takes j-set l (unit l / 2); a unit's cost, on its even lane, is the maximum
+// over the warps of its two j-sets' sum.
+__device__ __forceinline__ uint32_t unit_cost(const SymParams &p, int64_t t) {
     static_assert(NJSP == 32 && KBP == 2, "lane l: j-set l, unit l / 2");
-    const int64_t t = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     const int l = threadIdx.x & 31;
-    if (t >= p.T) return;  // whole warps
     int64_t I, J;
     item_of(t, p.nb, I, J);
     const bool sym = I != J;
@@ -448,79 +516,109 @@ __global__ void __launch_bounds__(256) sym_cost_kernel(const SymParams p, uint32
     const uint32_t cf = sym ? kCostSymFar : kCostDiagFar;
     float tb[7];
 #pragma unroll
-    for (int a = 0; a < 7; ++a) tb[a] = __ldg(p.jbox + (J * NJSP + l) * 8 + a);
+    for (int a = 0; a < 7; ++a) tb[a] = p.jbox[(J * NJSP + l) * 8 + a];
     uint32_t m = 0;
     for (int w = 0; w < NW; ++w) {
         float wb[7];
 #pragma unroll
-        for (int a = 0; a < 7; ++a) wb[a] = __ldg(p.wbox + (I * NW + w) * 8 + a);
+        for (int a = 0; a < 7; ++a) wb[a] = p.wbox[(I * NW + w) * 8 + a];
         const uint32_t v = boxes_near(wb, tb, p.gamma) ? cn : cf;
         const uint32_t pair = v + __shfl_xor_sync(0xffffffffu, v, 1);
         m = pair > m ? pair : m;
     }
-    uint32_t c = (l & 1) ? 0u : m + kCostSymUnit;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
-    if (l == 0) cost[t] = c;
+    return (l & 1) ? 0u : m + kCostSymUnit;
 }
 
-// prefix[t] = sum of cost[0, t), prefix[T] = total (one block, fixed order).
-__global__ void __launch_bounds__(1024) sym_scan_kernel(const uint32_t *cost, int64_t T,
-                                                        unsigned long long *prefix) {
-    __shared__ unsigned long long part[1024];
-    const int tid = threadIdx.x;
-    const int64_t per = (T + 1023) / 1024;
-    const int64_t a = tid * per, b = (a + per) < T ? (a + per) : T;
-    unsigned long long s = 0;
-    for (int64_t t = a; t < b; ++t) s += cost[t];
-    part[tid] = s;
+// One warp per item: the sum of its unit costs.
+__global__ void __launch_bounds__(256) sym_cost_kernel(const SymParams p, uint32_t *cost) {
+    const int64_t t = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+    dev::grid_trigger();
+    dev::grid_wait();
+    if (t >= p.T) return;  // whole warps
+    uint32_t c = unit_cost(p, t);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
+    if ((threadIdx.x & 31) == 0) cost[t] = c;
+}
+
+// One block: prefix[t] = sum of cost[0, t), prefix[T] = the total, and then
+// lo[c] = the unit where the cumulative cost reaches c / ctas of the total
+// (the nearest unit boundary, from the item's unit costs); lo[0] = 0,
+// lo[ctas] = U, non-decreasing.  A warp per range start: the item by a search
+// that probes 32 places at a time.  (A one-thread scan of the partial sums and
+// one thread per range start, its search and its 256 box tests, took 31 us of
+// a 65536-particle step.)
+__global__ void __launch_bounds__(1024) sym_ranges_kernel(const SymParams p, const uint32_t *cost,
+                                                          unsigned long long *prefix,
+                                                          int64_t *lo) {
+    __shared__ unsigned long long part[32];
+    const int tid = threadIdx.x, w = tid >> 5, l = tid & 31;
+    const int64_t per = (p.T + 1023) / 1024;
+    const int64_t i0 = tid * per < p.T ? tid * per : p.T;
+    const int64_t i1 = i0 + per < p.T ? i0 + per : p.T;
+    dev::grid_wait();
+    unsigned long long sum = 0;
+    for (int64_t t = i0; t < i1; ++t) sum += cost[t];
+    unsigned long long run = sum;  // inclusive scan over the warp, then the warps
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const unsigned long long v = __shfl_up_sync(0xffffffffu, run, o);
+        if (l >= o) run += v;
+    }
+    if (l == 31) part[w] = run;
     __syncthreads();
-    if (tid == 0) {
-        unsigned long long run = 0;
-        for (int i = 0; i < 1024; ++i) {
-            const unsigned long long v = part[i];
-            part[i] = run;
-            run += v;
+    if (w == 0) {
+        unsigned long long v = part[l];
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned long long x = __shfl_up_sync(0xffffffffu, v, o);
+            if (l >= o) v += x;
         }
-        prefix[T] = run;
+        part[l] = v;
     }
     __syncthreads();
-    unsigned long long run = part[tid];
-    for (int64_t t = a; t < b; ++t) {
+    run += (w ? part[w - 1] : 0ull) - sum;
+    for (int64_t t = i0; t < i1; ++t) {
         prefix[t] = run;
         run += cost[t];
     }
-}
-
-// lo[c] = the unit where the cumulative cost reaches c / ctas of the total
-// (the nearest unit boundary, from the item's unit costs); lo[0] = 0, lo[ctas] = U,
-// non-decreasing.
-__global__ void sym_ranges_kernel(const SymParams p, const uint32_t *cost,
-                                  const unsigned long long *prefix, int64_t T, int64_t ctas,
-                                  int64_t *lo) {
-    for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c <= ctas;
-         c += (int64_t)gridDim.x * blockDim.x) {
-        if (c == 0 || c == ctas) {
-            lo[c] = c == 0 ? 0 : T * US;
+    const unsigned long long total = part[31];
+    if (tid == 0) prefix[p.T] = total;
+    __syncthreads();
+    for (int64_t c = w; c <= p.ctas; c += 32) {
+        if (c == 0 || c == p.ctas) {
+            if (l == 0) lo[c] = c == 0 ? 0 : p.T * US;
             continue;
         }
-        const unsigned long long target = prefix[T] * (unsigned long long)c / (unsigned long long)ctas;
-        int64_t a = 0, b = T - 1;
-        while (a < b) {
-            const int64_t m = (a + b + 1) / 2;
-            if (prefix[m] <= target)
-                a = m;
-            else
-                b = m - 1;
+        const unsigned long long target = total * (unsigned long long)c / (unsigned long long)p.ctas;
+        int64_t a = 0, n = p.T;  // prefix[a] <= target; the item is one of n from a
+        while (n > 1) {
+            const int64_t st = (n + 31) / 32, t = a + l * st;
+            const unsigned le =
+                __ballot_sync(0xffffffffu, l * st < n && prefix[t < p.T ? t : p.T] <= target);
+            const int h = 31 - __clz((int)le);  // lane 0 always holds
+            n = n - h * st < st ? n - h * st : st;
+            a += h * st;
         }
         const unsigned long long r = target - prefix[a];
-        uint32_t uc[US];
-        item_unit_costs(p, a, uc);
-        unsigned long long run = 0;
-        int64_t off = 0;
-        while (off < US && run + uc[off] <= r) run += uc[off++];
-        if (off < US && 2 * (r - run) > uc[off]) ++off;  // the nearer boundary
-        lo[c] = a * US + off;
+        const uint32_t uc = unit_cost(p, a);
+        unsigned long long acc = 0;
+        int off = 0;
+        for (int u = 0; u < US; ++u) {
+            const uint32_t v = __shfl_sync(0xffffffffu, uc, 2 * u);
+            if (off == u) {
+                if (acc + v <= r) {
+                    acc += v;
+                    ++off;
+                } else if (2 * (r - acc) > v) {
+                    off = u + 1;  // the nearer boundary
+                    break;
+                } else {
+                    break;
+                }
+            }
+        }
+        if (l == 0) lo[c] = a * US + off;
     }
 }
 
@@ -540,32 +638,72 @@ int launch_pair(const SymParams &p, cudaStream_t st) {
     return NB_OK;
 }
 
-int launch_split(const SymParams &p, const ForceJob &j, const SymLayout &y) {
-    sym_cost_kernel<<<(unsigned)cdiv(p.T * 32, 256), 256, 0, j.stream>>>(p, y.cost);
-    sym_scan_kernel<<<1, 1024, 0, j.stream>>>(y.cost, p.T, y.prefix);
-    sym_ranges_kernel<<<(unsigned)cdiv(p.ctas + 1, 256), 256, 0, j.stream>>>(
-        p, y.cost, y.prefix, p.T, p.ctas, y.lo);
+// The stream-K ranges of the packed positions; with `exponent`, also the
+// call's fixed-point exponent (masses do not change within a step loop).
+int launch_split(const SymParams &p, const ForceJob &j, const SymLayout &y, bool exponent) {
+    NB_TRY_SYM(launch_pdl(sym_cost_kernel, (unsigned)cdiv(p.T * 32, 256), 256, 0, j.stream, p,
+                          y.cost));
+    NB_TRY_SYM(launch_pdl(sym_ranges_kernel, 1, 1024, 0, j.stream, p, y.cost, y.prefix, y.lo));
+    if (!exponent) return NB_OK;
     sym_exponent_kernel<<<(unsigned)std::min<int64_t>(cdiv(j.N, 4 * 256), 1024), 256, 0,
                           j.stream>>>(j.mass, j.N, j.eps, y.fx_exp, y.mmax_bits, y.arrivals);
-    count_launch(4);
+    count_launch();
     NB_CUDA(cudaGetLastError());
     return NB_OK;
 }
 
-int launch_fold(const SymParams &p, const ForceJob &j, const int *perm) {
+int launch_fold(const SymParams &p, const ForceJob &j, const int *perm, double *pot, double *vel,
+                double kick) {
     const int64_t fold_blocks = std::min<int64_t>(cdiv(p.Np, 256), 64 * (int64_t)device_sm_count());
-    sym_fold_kernel<<<(unsigned)fold_blocks, 256, 0, j.stream>>>(p, j.N, perm, j.G, j.acc, j.pot,
-                                                                 j.vel, j.kick);
+    sym_fold_kernel<<<(unsigned)fold_blocks, 256, 0, j.stream>>>(p, j.N, perm, j.G, j.acc, pot,
+                                                                 vel, kick);
     count_launch();
     NB_CUDA(cudaGetLastError());
     return NB_OK;
 }
 
 template <int POL>
-int launch_sym_pol(const SymParams &p, const ForceJob &j, const SymLayout &y, const int *perm) {
-    NB_TRY_SYM(launch_split(p, j, y));
-    NB_TRY_SYM(j.pot ? launch_pair<POL, true>(p, j.stream) : launch_pair<POL, false>(p, j.stream));
-    return launch_fold(p, j, perm);
+int launch_pair_pot(const SymParams &p, bool pot, cudaStream_t st) {
+    return pot ? launch_pair<POL, true>(p, st) : launch_pair<POL, false>(p, st);
+}
+
+int launch_pair_pol(const SymParams &p, int precision, bool pot, cudaStream_t st) {
+    switch (precision) {
+        case NB_PREC_FP32: return launch_pair_pot<NB_PREC_FP32>(p, pot, st);
+        case NB_PREC_KAHAN: return launch_pair_pot<NB_PREC_KAHAN>(p, pot, st);
+        case NB_PREC_F64ACC: return launch_pair_pot<NB_PREC_F64ACC>(p, pot, st);
+    }
+    return fail(NB_ERR_INVALID, "unknown precision %d", precision);
+}
+
+SymParams params_of(const ForceJob &j, const SymLayout &y) {
+    const SymSizes z = sym_sizes(j.L.Np);
+    SymParams p;
+    char *sb = j.ws + j.L.sortbuf;
+    p.soa = reinterpret_cast<const float *>(j.ws + j.L.packA);
+    p.Np = z.nb * kSymBlock;
+    p.nb = z.nb;
+    p.T = z.T;
+    p.U = z.U;
+    p.ctas = z.ctas;
+    const float ef = (float)j.eps;
+    p.eps2 = ef * ef;
+    p.gamma = j.gamma;
+    p.jbox = sort_tile_boxes(sb, j.L);
+    p.wbox = sort_block_boxes(sb, j.L);
+    p.acc_fx = y.acc_fx;
+    p.fx_exp = y.fx_exp;
+    p.lo = y.lo;
+    p.status = reinterpret_cast<uint32_t *>(j.ws + j.L.status);
+    return p;
+}
+
+int sorted_pack(const ForceJob &j, bool reuse_order) {
+    char *sb = j.ws + j.L.sortbuf;
+    return launch_sorted_pack(j.pos, j.mass, j.N, j.L.Np, reinterpret_cast<float *>(j.ws + j.L.packA),
+                              sort_perm(sb, j.L), sort_keys(sb), sort_box6(sb, j.L),
+                              sort_tile_boxes(sb, j.L), JSP, sort_block_boxes(sb, j.L), WS,
+                              reuse_order, j.stream);
 }
 
 }  // namespace
@@ -597,36 +735,59 @@ SymLayout sym_layout(char *ws, const WsLayout &L) {
     return y;
 }
 
-int launch_force_sym(const ForceJob &j) {
+static int check_sym(const ForceJob &j) {
     if (j.eps <= 0.0) return fail(NB_ERR_UNSUPPORTED, "symmetric pairs need eps > 0");
     if (j.L.sym_fx_bytes == 0)
         return fail(NB_ERR_WORKSPACE, "workspace has no symmetric-pair buffers");
-    const SymSizes z = sym_sizes(j.L.Np);
+    return NB_OK;
+}
+
+int launch_force_sym(const ForceJob &j) {
+    NB_TRY_SYM(check_sym(j));
     const SymLayout y = sym_layout(j.ws, j.L);
-    SymParams p;
+    const SymParams p = params_of(j, y);
+    NB_TRY_SYM(sorted_pack(j, j.reuse_order));
+    NB_TRY_SYM(launch_split(p, j, y, true));
+    NB_TRY_SYM(launch_pair_pol(p, j.precision, j.pot != nullptr, j.stream));
+    return launch_fold(p, j, sort_perm(j.ws + j.L.sortbuf, j.L), j.pot, j.vel, j.kick);
+}
+
+int launch_step_sym(const ForceJob &j, double *vel, double dt, int64_t nsteps, bool acc_valid) {
+    NB_TRY_SYM(check_sym(j));
+    const SymLayout y = sym_layout(j.ws, j.L);
+    const SymParams p = params_of(j, y);
     char *sb = j.ws + j.L.sortbuf;
-    p.soa = reinterpret_cast<const float *>(j.ws + j.L.packA);
-    p.Np = z.nb * kSymBlock;
-    p.nb = z.nb;
-    p.T = z.T;
-    p.U = z.U;
-    p.ctas = z.ctas;
-    const float ef = (float)j.eps;
-    p.eps2 = ef * ef;
-    p.gamma = j.gamma;
-    p.jbox = sort_tile_boxes(sb, j.L);
-    p.wbox = sort_block_boxes(sb, j.L);
-    p.acc_fx = y.acc_fx;
-    p.fx_exp = y.fx_exp;
-    p.lo = y.lo;
     const int *perm = sort_perm(sb, j.L);
-    p.status = reinterpret_cast<uint32_t *>(j.ws + j.L.status);
-    switch (j.precision) {
-        case NB_PREC_FP32: return launch_sym_pol<NB_PREC_FP32>(p, j, y, perm);
-        case NB_PREC_KAHAN: return launch_sym_pol<NB_PREC_KAHAN>(p, j, y, perm);
-        case NB_PREC_F64ACC: return launch_sym_pol<NB_PREC_F64ACC>(p, j, y, perm);
+    const double half = 0.5 * dt;
+    const int64_t e0 = acc_valid ? 1 : 0;  // evaluation 0 primes a(x)
+    int64_t sorted_at = -1;
+    bool opened = !acc_valid, packed = false;  // evaluation e's positions are there, are packed
+    for (int64_t e = e0; e <= nsteps; ++e) {
+        if (!opened)
+            NB_TRY_SYM(launch_kick_drift_pack(const_cast<double *>(j.pos), vel, j.acc, j.mass, j.N,
+                                              j.L.Np, dt, nullptr, j.stream));
+        if (!packed) {
+            const bool reuse = sorted_at >= 0 && e - sorted_at < kResortEvery;
+            if (!reuse) sorted_at = e;
+            NB_TRY_SYM(sorted_pack(j, reuse));
+        }
+        const bool last = e == nsteps;
+        double *pot = last ? j.pot : nullptr;
+        NB_TRY_SYM(launch_split(p, j, y, e == e0));
+        NB_TRY_SYM(launch_pair_pol(p, j.precision, pot != nullptr, j.stream));
+        // the next evaluation keeps the order: its kick, drift and pack in the fold
+        packed = !last && e + 1 - sorted_at < kResortEvery;
+        opened = packed;
+        if (packed)
+            NB_TRY_SYM(launch_pdl(sym_fold_next_kernel, (unsigned)(p.Np / 256), 256, 0, j.stream, p,
+                                  j.N, perm, j.G, const_cast<double *>(j.pos), vel,
+                                  e ? half : 0.0, half, dt,
+                                  reinterpret_cast<float *>(j.ws + j.L.packA),
+                                  sort_tile_boxes(sb, j.L), sort_block_boxes(sb, j.L)));
+        else
+            NB_TRY_SYM(launch_fold(p, j, perm, pot, e ? vel : nullptr, half));
     }
-    return fail(NB_ERR_INVALID, "unknown precision %d", j.precision);
+    return NB_OK;
 }
 
 }  // namespace nb
