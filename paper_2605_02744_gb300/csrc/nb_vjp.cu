@@ -548,9 +548,9 @@ static int launch_vjp_variant(const VjpParams &p, bool guard, bool pb, bool fuse
 //   f = r^3 (w - (3 r^2 (d . w) + m_k pbar_j + m_j pbar_k) d),
 // x_bar_k += f, x_bar_j -= f, and the mass sums
 //   M_k += r^3 (c_j . d) + r pbar_j,   M_j += r pbar_k - r^3 (c_k . d)
-// (m_bar = -G M).  37 packed FP32 operations per two unordered pairs (45
-// fused with the force, 42 with pbar; hi/lo displacement +6) instead of 2 x
-// 26 (2 x 31, 2 x 30).  w is formed before it meets r^3, so close pairs with
+// (m_bar = -G M).  d . w is taken as m_k (c_j . d) - m_j (c_k . d).  35 packed
+// FP32 operations per two unordered pairs (43 fused with the force, 40 with
+// pbar; hi/lo displacement +6) instead of 2 x 26 (2 x 31, 2 x 30).  w is formed before it meets r^3, so close pairs with
 // similar cotangents lose nothing to cancellation between m_k sum r^3 c_j
 // and c_k sum r^3 m_j.
 namespace {
@@ -623,9 +623,13 @@ struct VjpPh {
             const float2 wx = fma2(s.m[k], J[4], mul2(J[3], s.ncx[k]));
             const float2 wy = fma2(s.m[k], J[5], mul2(J[3], s.ncy[k]));
             const float2 wz = fma2(s.m[k], J[6], mul2(J[3], s.ncz[k]));
-            float2 dw = mul2(dx, wx);
-            dw = fma2(dy, wy, dw);
-            dw = fma2(dz, wz, dw);
+            float2 dcj = mul2(dx, J[4]);
+            dcj = fma2(dy, J[5], dcj);
+            dcj = fma2(dz, J[6], dcj);
+            float2 dck = mul2(dx, s.ncx[k]);  // -(c_k . d)
+            dck = fma2(dy, s.ncy[k], dck);
+            dck = fma2(dz, s.ncz[k], dck);
+            const float2 dw = fma2(s.m[k], dcj, mul2(J[3], dck));
             const float2 rr = mul2(r, r);
             const float2 r3 = mul2(rr, r);
             float2 q;
@@ -642,9 +646,6 @@ struct VjpPh {
             s.a[k][0] = fma2(r3, ex, s.a[k][0]);
             s.a[k][1] = fma2(r3, ey, s.a[k][1]);
             s.a[k][2] = fma2(r3, ez, s.a[k][2]);
-            float2 dcj = mul2(dx, J[4]);
-            dcj = fma2(dy, J[5], dcj);
-            dcj = fma2(dz, J[6], dcj);
             s.a[k][3] = fma2(r3, dcj, s.a[k][3]);
             if constexpr (PB) s.a[k][3] = fma2(r, J[7], s.a[k][3]);
             if constexpr (FUSED) {
@@ -654,9 +655,6 @@ struct VjpPh {
                 s.a[k][6] = fma2(sj, dz, s.a[k][6]);
             }
             if (SYM) {
-                float2 dck = mul2(dx, s.ncx[k]);  // -(c_k . d)
-                dck = fma2(dy, s.ncy[k], dck);
-                dck = fma2(dz, s.ncz[k], dck);
                 T[0] = k ? fma2(r3, ex, T[0]) : mul2(r3, ex);
                 T[1] = k ? fma2(r3, ey, T[1]) : mul2(r3, ey);
                 T[2] = k ? fma2(r3, ez, T[2]) : mul2(r3, ez);
