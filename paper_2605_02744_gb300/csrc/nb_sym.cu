@@ -541,21 +541,15 @@ __global__ void __launch_bounds__(256) sym_cost_kernel(const SymParams p, uint32
     if ((threadIdx.x & 31) == 0) cost[t] = c;
 }
 
-// One block: prefix[t] = sum of cost[0, t), prefix[T] = the total, and then
-// lo[c] = the unit where the cumulative cost reaches c / ctas of the total
-// (the nearest unit boundary, from the item's unit costs); lo[0] = 0,
-// lo[ctas] = U, non-decreasing.  A warp per range start: the item by a search
-// that probes 32 places at a time.  (A one-thread scan of the partial sums and
-// one thread per range start, its search and its 256 box tests, took 31 us of
-// a 65536-particle step.)
-__global__ void __launch_bounds__(1024) sym_ranges_kernel(const SymParams p, const uint32_t *cost,
-                                                          unsigned long long *prefix,
-                                                          int64_t *lo) {
+// One block: prefix[t] = sum of cost[0, t), prefix[T] = the total.
+__global__ void __launch_bounds__(1024) sym_scan_kernel(const SymParams p, const uint32_t *cost,
+                                                        unsigned long long *prefix) {
     __shared__ unsigned long long part[32];
     const int tid = threadIdx.x, w = tid >> 5, l = tid & 31;
     const int64_t per = (p.T + 1023) / 1024;
     const int64_t i0 = tid * per < p.T ? tid * per : p.T;
     const int64_t i1 = i0 + per < p.T ? i0 + per : p.T;
+    dev::grid_trigger();
     dev::grid_wait();
     unsigned long long sum = 0;
     for (int64_t t = i0; t < i1; ++t) sum += cost[t];
@@ -582,44 +576,55 @@ __global__ void __launch_bounds__(1024) sym_ranges_kernel(const SymParams p, con
         prefix[t] = run;
         run += cost[t];
     }
-    const unsigned long long total = part[31];
-    if (tid == 0) prefix[p.T] = total;
-    __syncthreads();
-    for (int64_t c = w; c <= p.ctas; c += 32) {
-        if (c == 0 || c == p.ctas) {
-            if (l == 0) lo[c] = c == 0 ? 0 : p.T * US;
-            continue;
-        }
-        const unsigned long long target = total * (unsigned long long)c / (unsigned long long)p.ctas;
-        int64_t a = 0, n = p.T;  // prefix[a] <= target; the item is one of n from a
-        while (n > 1) {
-            const int64_t st = (n + 31) / 32, t = a + l * st;
-            const unsigned le =
-                __ballot_sync(0xffffffffu, l * st < n && prefix[t < p.T ? t : p.T] <= target);
-            const int h = 31 - __clz((int)le);  // lane 0 always holds
-            n = n - h * st < st ? n - h * st : st;
-            a += h * st;
-        }
-        const unsigned long long r = target - prefix[a];
-        const uint32_t uc = unit_cost(p, a);
-        unsigned long long acc = 0;
-        int off = 0;
-        for (int u = 0; u < US; ++u) {
-            const uint32_t v = __shfl_sync(0xffffffffu, uc, 2 * u);
-            if (off == u) {
-                if (acc + v <= r) {
-                    acc += v;
-                    ++off;
-                } else if (2 * (r - acc) > v) {
-                    off = u + 1;  // the nearer boundary
-                    break;
-                } else {
-                    break;
-                }
+    if (tid == 0) prefix[p.T] = part[31];
+}
+
+// A warp per range start: lo[c] = the unit where the cumulative cost reaches c / ctas of the total
+// (the nearest unit boundary, from the item's unit costs); lo[0] = 0,
+// lo[ctas] = U, non-decreasing; the item by a search that probes 32 places at a
+// time.  (A one-thread scan of the partial sums and one thread per range
+// start, its search and its 256 box tests, took 31 us of a 65536-particle
+// step.)
+__global__ void __launch_bounds__(128) sym_ranges_kernel(const SymParams p,
+                                                         const unsigned long long *prefix,
+                                                         int64_t *lo) {
+    const int l = threadIdx.x & 31;
+    const int64_t c = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+    dev::grid_wait();
+    if (c > p.ctas) return;  // whole warps
+    if (c == 0 || c == p.ctas) {
+        if (l == 0) lo[c] = c == 0 ? 0 : p.T * US;
+        return;
+    }
+    const unsigned long long target = prefix[p.T] * (unsigned long long)c / (unsigned long long)p.ctas;
+    int64_t a = 0, n = p.T;  // prefix[a] <= target; the item is one of n from a
+    while (n > 1) {
+        const int64_t st = (n + 31) / 32, t = a + l * st;
+        const unsigned le =
+            __ballot_sync(0xffffffffu, l * st < n && prefix[t < p.T ? t : p.T] <= target);
+        const int h = 31 - __clz((int)le);  // lane 0 always holds
+        n = n - h * st < st ? n - h * st : st;
+        a += h * st;
+    }
+    const unsigned long long r = target - prefix[a];
+    const uint32_t uc = unit_cost(p, a);
+    unsigned long long acc = 0;
+    int off = 0;
+    for (int u = 0; u < US; ++u) {
+        const uint32_t v = __shfl_sync(0xffffffffu, uc, 2 * u);
+        if (off == u) {
+            if (acc + v <= r) {
+                acc += v;
+                ++off;
+            } else if (2 * (r - acc) > v) {
+                off = u + 1;  // the nearer boundary
+                break;
+            } else {
+                break;
             }
         }
-        if (l == 0) lo[c] = a * US + off;
     }
+    if (l == 0) lo[c] = a * US + off;
 }
 
 template <int POL, bool POT>
@@ -643,7 +648,9 @@ int launch_pair(const SymParams &p, cudaStream_t st) {
 int launch_split(const SymParams &p, const ForceJob &j, const SymLayout &y, bool exponent) {
     NB_TRY_SYM(launch_pdl(sym_cost_kernel, (unsigned)cdiv(p.T * 32, 256), 256, 0, j.stream, p,
                           y.cost));
-    NB_TRY_SYM(launch_pdl(sym_ranges_kernel, 1, 1024, 0, j.stream, p, y.cost, y.prefix, y.lo));
+    NB_TRY_SYM(launch_pdl(sym_scan_kernel, 1, 1024, 0, j.stream, p, y.cost, y.prefix));
+    NB_TRY_SYM(launch_pdl(sym_ranges_kernel, (unsigned)cdiv((p.ctas + 1) * 32, 128), 128, 0,
+                          j.stream, p, y.prefix, y.lo));
     if (!exponent) return NB_OK;
     sym_exponent_kernel<<<(unsigned)std::min<int64_t>(cdiv(j.N, 4 * 256), 1024), 256, 0,
                           j.stream>>>(j.mass, j.N, j.eps, y.fx_exp, y.mmax_bits, y.arrivals);
