@@ -203,21 +203,42 @@ __global__ void __launch_bounds__(1024) bsym_setup_kernel(BsParams p, int64_t N)
     const int64_t per = (nitems + 1023) / 1024;
     const int64_t lo = tid * per, hi = (lo + per) < nitems ? (lo + per) : nitems;
     for (int k = 0; k < BG; ++k) cnt[tid][k] = 0;
+#pragma unroll 8
     for (int64_t i = lo; i < hi; ++i) {
         const int4 it = p.items[i];
         cnt[tid][it.w - it.z - 1] += 1;
     }
     __syncthreads();
-    if (tid == 0) {
-        int32_t run = 0;
-        for (int k = BG - 1; k >= 0; --k)
-            for (int t = 0; t < 1024; ++t) {
-                const int32_t v = cnt[t][k];
-                cnt[t][k] = run;
-                run += v;
+    // a scan over the threads per size (one thread running over the 8 x 1024
+    // counts took most of this kernel's 100 us)
+    __shared__ int32_t wsum[32];
+    const int lane = tid & 31, wid = tid >> 5;
+    int32_t before = 0;  // items of the larger sizes
+    for (int k = BG - 1; k >= 0; --k) {
+        const int32_t own_k = cnt[tid][k];
+        int32_t incl = own_k;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int32_t v = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += v;
+        }
+        if (lane == 31) wsum[wid] = incl;
+        __syncthreads();
+        if (wid == 0) {
+            int32_t v = wsum[lane];
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int32_t x = __shfl_up_sync(0xffffffffu, v, o);
+                if (lane >= o) v += x;
             }
+            wsum[lane] = v;
+        }
+        __syncthreads();
+        cnt[tid][k] = before + (wid ? wsum[wid - 1] : 0) + incl - own_k;
+        before += wsum[31];
+        __syncthreads();
     }
-    __syncthreads();
+#pragma unroll 8
     for (int64_t i = lo; i < hi; ++i) {
         const int4 it = p.items[i];
         p.order[cnt[tid][it.w - it.z - 1]++] = (int32_t)i;
@@ -225,15 +246,20 @@ __global__ void __launch_bounds__(1024) bsym_setup_kernel(BsParams p, int64_t N)
 }
 
 // Hilbert order of each system (one CTA per system): FP64 bounding box,
-// 30-bit codes, keys code << 13 | source index, shared-memory bitonic sort;
+// 30-bit codes, keys code << 13 | source index, bitonic sort mostly in
+// registers (512 clusters of 64 to 8192: 389 us with the
+// sort in shared memory and FP64 compares, 211 us now);
 // then the state is gathered into the other buffer in the new order: from
 // the caller's arrays (from_user: particle order) or from the current
 // slot-order buffer (a re-sort).  The real particles of a system always fill
 // its first n slots; the padding slots hold zeros and perm = -1.
-__global__ void __launch_bounds__(512) bsym_sort_kernel(BsParams p, int from_user) {
+constexpr int kSortThreads = 512;
+static_assert(kBsMaxN == 16 * kSortThreads, "the largest system's keys");
+
+__global__ void __launch_bounds__(kSortThreads) bsym_sort_kernel(BsParams p, int from_user) {
     extern __shared__ unsigned long long keys[];  // kBsMaxN keys, then kBsMaxN old perm entries
     int *old_perm = reinterpret_cast<int *>(keys + kBsMaxN);
-    __shared__ double red[6][16];
+    __shared__ long long red[6][16];
     const int c = blockIdx.x;
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
     const int64_t sb = p.sbase[c], ns = p.sbase[c + 1] - sb;
@@ -244,19 +270,26 @@ __global__ void __launch_bounds__(512) bsym_sort_kernel(BsParams p, int from_use
     auto xsrc = [&](int e, int d) -> double {
         return from_user ? p.pos[3 * (o0 + e) + d] : st_arr(p, src, d)[sb + e];
     };
-    double lo[3] = {1e308, 1e308, 1e308}, hi[3] = {-1e308, -1e308, -1e308};
+    // minima and maxima of order-preserving integer images (FP64 compares are slow)
+    long long lo[3], hi[3];
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+        lo[d] = dev::ordered_bits(1e308);
+        hi[d] = dev::ordered_bits(-1e308);
+    }
+#pragma unroll 4
     for (int e = tid; e < n; e += blockDim.x)
 #pragma unroll
         for (int d = 0; d < 3; ++d) {
-            const double x = xsrc(e, d);
-            lo[d] = fmin(lo[d], x);
-            hi[d] = fmax(hi[d], x);
+            const long long x = dev::ordered_bits(xsrc(e, d));
+            lo[d] = min(lo[d], x);
+            hi[d] = max(hi[d], x);
         }
 #pragma unroll
     for (int d = 0; d < 3; ++d)
         for (int o = 16; o > 0; o >>= 1) {
-            lo[d] = fmin(lo[d], __shfl_xor_sync(0xffffffffu, lo[d], o));
-            hi[d] = fmax(hi[d], __shfl_xor_sync(0xffffffffu, hi[d], o));
+            lo[d] = min(lo[d], __shfl_xor_sync(0xffffffffu, lo[d], o));
+            hi[d] = max(hi[d], __shfl_xor_sync(0xffffffffu, hi[d], o));
         }
     if (lane == 0)
 #pragma unroll
@@ -270,15 +303,16 @@ __global__ void __launch_bounds__(512) bsym_sort_kernel(BsParams p, int from_use
     double blo[3], scale[3];
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
-        double a = 1e308, b = -1e308;
-        for (int k = 0; k < (int)(blockDim.x / 32); ++k) {
-            a = fmin(a, red[d][k]);
-            b = fmax(b, red[3 + d][k]);
+        long long la = red[d][0], lb = red[3 + d][0];
+        for (int k = 1; k < (int)(blockDim.x / 32); ++k) {
+            la = min(la, red[d][k]);
+            lb = max(lb, red[3 + d][k]);
         }
+        const double a = dev::from_ordered(la), b = dev::from_ordered(lb);
         blo[d] = a;
         scale[d] = b > a ? 1023.0 / (b - a) : 0.0;
     }
-    int P2 = 1;
+    int P2 = kSortThreads;
     while (P2 < n) P2 <<= 1;
     for (int e = tid; e < P2; e += blockDim.x) {
         unsigned long long k = ~0ull;
@@ -291,7 +325,13 @@ __global__ void __launch_bounds__(512) bsym_sort_kernel(BsParams p, int from_use
         keys[e] = k;
     }
     __syncthreads();
-    dev::block_bitonic_sort(keys, P2);
+    switch (P2 / kSortThreads) {
+        case 1: dev::block_sort_regs<kSortThreads, 1>(keys); break;
+        case 2: dev::block_sort_regs<kSortThreads, 2>(keys); break;
+        case 4: dev::block_sort_regs<kSortThreads, 4>(keys); break;
+        case 8: dev::block_sort_regs<kSortThreads, 8>(keys); break;
+        default: dev::block_sort_regs<kSortThreads, 16>(keys); break;
+    }
     for (int64_t s = tid; s < ns; s += blockDim.x) {
         double v[10];
         int pi = -1;
@@ -701,7 +741,7 @@ int launch_bsym_steps(BsParams p, const BatchedJob &j, int64_t nb_max) {
     }
     p.cur = 0;
     auto sort = [&](int from_user) {
-        bsym_sort_kernel<<<(unsigned)p.B, 512, sort_smem, st>>>(p, from_user);
+        bsym_sort_kernel<<<(unsigned)p.B, kSortThreads, sort_smem, st>>>(p, from_user);
         p.cur ^= 1;
         count_launch();
     };

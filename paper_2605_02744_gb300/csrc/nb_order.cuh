@@ -49,11 +49,21 @@ __device__ __forceinline__ uint32_t hilbert30(uint32_t x, uint32_t y, uint32_t z
     return (spread3(X[0]) << 2) | (spread3(X[1]) << 1) | spread3(X[2]);
 }
 
-// The cell of one coordinate: (x - lo) * scale clamped to [0, 1023].
+// The cell of one coordinate: (x - lo) * scale truncated and clamped to [0,
+// 1023] (as an integer: the conversion saturates, and FP64 compares are slow on
+// this part).
 __device__ __forceinline__ uint32_t cell10(double x, double lo, double scale) {
-    double q = (x - lo) * scale;
-    q = q < 0.0 ? 0.0 : (q > 1023.0 ? 1023.0 : q);
-    return (uint32_t)q;
+    const int q = __double2int_rz((x - lo) * scale);
+    return (uint32_t)min(max(q, 0), 1023);
+}
+
+// Order-preserving image of a double as a signed integer, and back.
+__device__ __forceinline__ long long ordered_bits(double x) {
+    const long long b = __double_as_longlong(x);
+    return b >= 0 ? b : (b ^ 0x7fffffffffffffffLL);
+}
+__device__ __forceinline__ double from_ordered(long long b) {
+    return __longlong_as_double(b >= 0 ? b : (b ^ 0x7fffffffffffffffLL));
 }
 
 // Ascending bitonic sort of P (a power of two) 64-bit keys in shared memory
@@ -74,6 +84,69 @@ __device__ __forceinline__ void block_bitonic_sort(unsigned long long *keys, int
             }
             __syncthreads();
         }
+}
+
+// Ascending bitonic sort of T E 64-bit keys by a CTA of T threads (every thread
+// calls it).  Thread t holds elements t E .. t E + E - 1 in registers: strides
+// below E are exchanges within the thread, strides below 32 E shuffles within
+// the warp, and only the longer ones (10 of the 91 stages of 8192 keys) go
+// through shared memory, where block_bitonic_sort takes every stage there with
+// a barrier each.  keys: in linear order on entry and, after the barrier at
+// the end, on exit.
+// Only the stages k_lo .. k_hi, with directions from the elements' global index
+// base + ..., when the keys are a chunk of a longer sequence (strides of a chunk
+// or more are done elsewhere).
+template <int T, int E>
+__device__ __forceinline__ void block_sort_regs(unsigned long long *keys, int64_t k_lo = 2,
+                                                int64_t k_hi = T * E, int64_t base = 0) {
+    const int t = threadIdx.x;
+    unsigned long long v[E];
+#pragma unroll
+    for (int e = 0; e < E; ++e) v[e] = keys[t * E + e];
+    __syncthreads();
+    // keeps the smaller of own and other on the lower side of an ascending run
+    auto keep = [](unsigned long long own, unsigned long long other, bool small) {
+        return (own < other) == small ? own : other;
+    };
+    for (int64_t k = k_lo; k <= k_hi; k <<= 1) {
+        for (int j = k >= T * E ? T * E / 2 : (int)(k >> 1); j >= E; j >>= 1) {
+            const int m = j / E;
+            const bool lower = !(t & m);
+            if (m >= 32) {  // the shared copy is [E][T]: no bank conflicts
+#pragma unroll
+                for (int e = 0; e < E; ++e) keys[e * T + t] = v[e];
+                __syncthreads();
+#pragma unroll
+                for (int e = 0; e < E; ++e) {
+                    const bool asc = ((base + t * E + e) & k) == 0;
+                    v[e] = keep(v[e], keys[e * T + (t ^ m)], lower == asc);
+                }
+                __syncthreads();
+            } else {
+#pragma unroll
+                for (int e = 0; e < E; ++e) {
+                    const bool asc = ((base + t * E + e) & k) == 0;
+                    v[e] = keep(v[e], __shfl_xor_sync(0xffffffffu, v[e], m), lower == asc);
+                }
+            }
+        }
+#pragma unroll
+        for (int j = E / 2; j > 0; j >>= 1)
+            if (j < k) {
+#pragma unroll
+                for (int e = 0; e < E; ++e)
+                    if (!(e & j)) {
+                        const bool asc = ((base + t * E + e) & k) == 0;
+                        const unsigned long long a = v[e], b = v[e + j];
+                        const bool swap = (a > b) == asc;
+                        v[e] = swap ? b : a;
+                        v[e + j] = swap ? a : b;
+                    }
+            }
+    }
+#pragma unroll
+    for (int e = 0; e < E; ++e) keys[t * E + e] = v[e];
+    __syncthreads();
 }
 
 }  // namespace dev

@@ -11,8 +11,8 @@
 //   bbox:     FP64 min/max of the positions (atomics on order-preserving
 //             integer images; min/max do not depend on order)
 //   keys:     30-bit Hilbert index of the position's cell in that box << 32 | index
-//   sort:     bitonic network on 64-bit keys (shared-memory passes for
-//             strides below 2048, global passes above); keys are unique, so
+//   sort:     bitonic network on 64-bit keys (passes over chunks of 4096 keys in
+//             registers and shared memory, global passes for longer strides); keys are unique, so
 //             the order is fully determined
 //   pack:     split hi/lo SoA in sorted order + permutation (slot -> index)
 //   boxes:    per group of `unit` slots: lo[3], hi[3], max |coordinate|
@@ -26,13 +26,8 @@ namespace nb {
 
 constexpr int kSortChunk = 4096;  // keys per shared-memory bitonic block
 
-__device__ __forceinline__ long long ordered_bits(double x) {
-    const long long b = __double_as_longlong(x);
-    return b >= 0 ? b : (b ^ 0x7fffffffffffffffLL);
-}
-__device__ __forceinline__ double from_ordered(long long b) {
-    return __longlong_as_double(b >= 0 ? b : (b ^ 0x7fffffffffffffffLL));
-}
+using dev::from_ordered;
+using dev::ordered_bits;
 
 __global__ void bbox_init_kernel(long long *box) {
     if (threadIdx.x < 3) {
@@ -106,24 +101,7 @@ __global__ void bitonic_smem_kernel(unsigned long long *keys, int64_t k_lo, int6
     const int64_t base = (int64_t)blockIdx.x * kSortChunk;
     for (int e = threadIdx.x; e < kSortChunk; e += blockDim.x) s[e] = keys[base + e];
     __syncthreads();
-    for (int64_t k = k_lo; k <= k_hi; k <<= 1) {
-        int64_t j0 = k >> 1;
-        if (j0 >= kSortChunk) j0 = kSortChunk >> 1;
-        for (int64_t j = j0; j > 0; j >>= 1) {
-            for (int e = threadIdx.x; e < kSortChunk; e += blockDim.x) {
-                const int x = e ^ (int)j;
-                if (x > e) {
-                    const bool asc = ((base + e) & k) == 0;
-                    const unsigned long long a = s[e], b = s[x];
-                    if ((a > b) == asc) {
-                        s[e] = b;
-                        s[x] = a;
-                    }
-                }
-            }
-            __syncthreads();
-        }
-    }
+    dev::block_sort_regs<1024, kSortChunk / 1024>(s, k_lo, k_hi, base);
     for (int e = threadIdx.x; e < kSortChunk; e += blockDim.x) keys[base + e] = s[e];
 }
 
