@@ -183,13 +183,20 @@ __host__ __device__ inline double value(unsigned long long word_hi, unsigned lon
 constexpr int kLimbs = 4, kLimbBits = 44;
 constexpr int kLimbMagBits = kLimbs * kLimbBits - 2;  // |X| < 2^174
 
+// The exponent of a bound that is not finite: no grid, every total a NaN.
+constexpr int kNoGrid = -900;
+// A partial that is not finite, or beyond the bound, poisons its accumulator:
+// atomicMax of the top limb with this value, 2^18 times what sums reach there,
+// and the total reads as a NaN.
+constexpr long long kPoison = 1ll << 62;
+
 __host__ __device__ inline int limb_exponent_for(double bound) {
+    if (!isfinite(bound)) return kNoGrid;
     if (!(bound > 0.0)) return 0;
-    if (!isfinite(bound)) return -900;
     int e = 0;
     frexp(bound, &e);  // bound < 2^e
     const int F = kLimbMagBits - e;
-    return F < -900 ? -900 : (F > 900 ? 900 : F);
+    return F <= kNoGrid ? kNoGrid + 1 : (F > 900 ? 900 : F);
 }
 
 // v 2^F rounded half away from zero: limb q gains lo, limb q + 1 hi (both with
@@ -257,8 +264,15 @@ __host__ __device__ inline bool split_limbs(double v, int F, int &q, long long (
     return true;
 }
 
-// The accumulated value of the limbs, rounded once to double.
+// The accumulated value of the limbs, rounded once to double; a NaN for a
+// poisoned accumulator or without a grid.
 __host__ __device__ inline double limb_value(const long long (&w)[kLimbs], int F) {
+    if (F == kNoGrid || w[kLimbs - 1] >= kPoison / 2) {
+        const unsigned long long nan_bits = 0x7ff8000000000000ull;
+        double d;
+        memcpy(&d, &nan_bits, 8);
+        return d;
+    }
     long long t[kLimbs];
     long long c = 0;  // carries: every limb but the top one into [0, 2^44)
 #pragma unroll

@@ -98,7 +98,7 @@ struct WsLayout {
     size_t scratch;   // O(N) reduction scratch (energy partials, batched queue)
     size_t sym_fx;    // symmetric-pair path: fixed-point totals, 64 B per slot
     size_t sym_cost;  // symmetric-pair path: exponent, item costs, their prefix, CTA ranges
-    size_t wsym_head; // warp-granular path: exponents (at 64), input maxima (at 128, zero between calls)
+    size_t wsym_head; // warp-granular path: exponents (at 64), input maxima (at 128, FP64 192; zero between calls)
     size_t wsym_fx;   // its fixed-point totals, 7 components x 4 limbs per slot (zero between calls)
     size_t bsym, bsym_bytes;  // batched symmetric-pair path (0 bytes: not provisioned)
     size_t sym_fx_bytes;      // 0 when the symmetric path is not provisioned

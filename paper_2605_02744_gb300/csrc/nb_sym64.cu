@@ -41,7 +41,7 @@ struct Params64 {
     double eps2;
     unsigned long long *fx;    // [4][4 limbs][Np]
     int *fxe;
-    const unsigned *mx;
+    const unsigned long long *mx;  // max |m|, the bits of a double
     double scale;              // bound of every partial and total / max|m|
     uint32_t *status;
 };
@@ -144,7 +144,7 @@ __global__ void __launch_bounds__(NTHR) sym64_kernel(const Params64 p) {
     }
     dev::grid_wait();
     if (tid == 0) {
-        sF = fx::limb_exponent_for(p.scale * (double)__uint_as_float(__ldcg(p.mx + kMaxM)));
+        sF = fx::limb_exponent_for(p.scale * __longlong_as_double((long long)__ldcg(p.mx)));
         if (blockIdx.x == 0) *p.fxe = sF;
     }
     __syncthreads();
@@ -154,9 +154,13 @@ __global__ void __launch_bounds__(NTHR) sym64_kernel(const Params64 p) {
     auto add = [&](int e, int slot, double v) {
         int q;
         long long t[3];
-        if (!fx::split_limbs(v, F, q, t)) bad = 1;
+        const bool ok = fx::split_limbs(v, F, q, t);
         if (slot >= p.N) return;
         unsigned long long *wd = p.fx + (int64_t)(fx::kLimbs * e + q) * p.Np + slot;
+        if (!ok) {
+            bad = 1;
+            poison(wd + (fx::kLimbs - 1) * p.Np);  // q is 0
+        }
 #pragma unroll
         for (int k = 0; k < 3; ++k)
             if (t[k]) atomicAdd(wd + k * p.Np, (unsigned long long)t[k]);
@@ -210,11 +214,11 @@ __global__ void __launch_bounds__(NTHR) sym64_kernel(const Params64 p) {
 __global__ void __launch_bounds__(128) sym64_open_kernel(double *pos, double *vel,
                                                          const double *acc, const double *mass,
                                                          int64_t N, double kick, double drift,
-                                                         unsigned *mx) {
+                                                         unsigned long long *mx) {
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     dev::grid_trigger();
     dev::grid_wait();
-    float am = 0.f;
+    unsigned long long am = 0ull;  // non-negative doubles order like their bits
     if (i < N) {
         if (vel) {
 #pragma unroll
@@ -224,9 +228,14 @@ __global__ void __launch_bounds__(128) sym64_open_kernel(double *pos, double *ve
                 pos[3 * i + c] += drift * v;
             }
         }
-        am = __double2float_ru(fabs(mass[i]));
+        am = (unsigned long long)__double_as_longlong(fabs(mass[i]));
     }
-    warp_max(mx + kMaxM, am);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const unsigned long long v = __shfl_xor_sync(0xffffffffu, am, o);
+        am = v > am ? v : am;
+    }
+    if ((threadIdx.x & 31) == 0 && am) atomicMax(mx, am);
 }
 
 // The totals of every particle, as wsym_fold_kernel; NEXT: also the next
@@ -235,11 +244,12 @@ template <bool NEXT>
 __global__ void __launch_bounds__(128) sym64_fold_kernel(const Params64 p, double G, double *acc,
                                                          double *pot, double *pos, double *vel,
                                                          double kick, double next_kick,
-                                                         double drift, unsigned *mx) {
+                                                         double drift,
+                                                         unsigned long long *mx) {
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     dev::grid_trigger();
     dev::grid_wait();
-    if (!NEXT && i == 0) mx[kMaxM] = 0u;  // for the next call
+    if (!NEXT && i == 0) *mx = 0ull;  // for the next call
     if (i >= p.N) return;
     Params t{};
     t.fx = p.fx;
@@ -271,10 +281,10 @@ __global__ void __launch_bounds__(128) sym64_fold_kernel(const Params64 p, doubl
 struct Run64 {
     const ForceJob &j;
     Params64 p{};
-    unsigned *mx;
+    unsigned long long *mx;
 
     explicit Run64(const ForceJob &job) : j(job) {
-        mx = reinterpret_cast<unsigned *>(j.ws + j.L.wsym_head + 128);
+        mx = reinterpret_cast<unsigned long long *>(j.ws + j.L.wsym_head + 192);
         p.pos = j.pos;
         p.mass = j.mass;
         p.N = j.N;

@@ -115,6 +115,10 @@ __host__ __device__ __forceinline__ void item_of(int64_t t, int64_t nb, int &I, 
     J = (int)(r + (t - row_start(r, nb)));
 }
 
+__device__ __forceinline__ void poison(unsigned long long *top_limb) {
+    atomicMax(reinterpret_cast<long long *>(top_limb), fx::kPoison);
+}
+
 // TwoSum (Knuth): s + c + x kept as an unevaluated pair; without `keep` (the
 // FP32 policy's plain running sums) the rounding error of the add is dropped.
 __device__ __forceinline__ float2 two_add(float2 t, float x, bool keep = true) {
@@ -278,9 +282,13 @@ __global__ void __launch_bounds__(Geo<PH>::NTHR, 1) wsym_kernel(const Params p) 
     auto add = [&](int e, int slot, float v, int Fe) {
         int q;
         long long lo, hi;
-        if (!fx::split_limbs(v, Fe, q, lo, hi)) bad = 1;
+        const bool ok = fx::split_limbs(v, Fe, q, lo, hi);
         if (slot >= p.N) return;
         unsigned long long *wd = p.fx + (int64_t)(fx::kLimbs * e + q) * p.Np + slot;
+        if (!ok) {
+            bad = 1;
+            poison(wd + (fx::kLimbs - 1) * p.Np);  // q is 0
+        }
         if (lo) atomicAdd(wd, (unsigned long long)lo);
         if (hi) atomicAdd(wd + p.Np, (unsigned long long)hi);
     };
