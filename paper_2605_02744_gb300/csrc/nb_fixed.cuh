@@ -184,7 +184,7 @@ constexpr int kLimbs = 4, kLimbBits = 44;
 constexpr int kLimbMagBits = kLimbs * kLimbBits - 2;  // |X| < 2^174
 
 // The exponent of a bound that is not finite: no grid, every total a NaN.
-constexpr int kNoGrid = -900;
+constexpr int kNoGrid = -100000;
 // A partial that is not finite, or beyond the bound, poisons its accumulator:
 // atomicMax of the top limb with this value, 2^18 times what sums reach there,
 // and the total reads as a NaN.
@@ -196,7 +196,15 @@ __host__ __device__ inline int limb_exponent_for(double bound) {
     int e = 0;
     frexp(bound, &e);  // bound < 2^e
     const int F = kLimbMagBits - e;
-    return F <= kNoGrid ? kNoGrid + 1 : (F > 900 ? 900 : F);
+    return F < -900 ? -900 : (F > 900 ? 900 : F);
+}
+
+// The same from an exponent e with bound < 2^e (kNoBound: not finite).
+constexpr int kNoBound = 4096;
+__host__ __device__ inline int limb_exponent(int e) {
+    if (e >= kNoBound / 2) return kNoGrid;
+    const int F = kLimbMagBits - e;
+    return F < -900 ? -900 : (F > 900 ? 900 : F);
 }
 
 // v 2^F rounded half away from zero: limb q gains lo, limb q + 1 hi (both with

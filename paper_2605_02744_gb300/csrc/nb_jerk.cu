@@ -303,19 +303,23 @@ using namespace wsym;
 template <bool IPAIR_, bool POT>
 struct JerkPh {
     static constexpr bool IPAIR = IPAIR_;
-    static constexpr int K = 4, WARPS = 8, NJ = 10, NC = POT ? 7 : 6, GROUPS = 2;
+    static constexpr int K = 4, WARPS = 8, NJ = 10, NC = POT ? 7 : 6, GROUPS = POT ? 3 : 2;
     struct S {
         float2 nx[K], ny[K], nz[K], m[K], nvx[K], nvy[K], nvz[K];
         LoT<IPAIR> nxl[K], nyl[K], nzl[K];
         float2 a[K][NC];  // ax ay az jx jy jz (phi)
     };
-    // exponents: the jerk's, then the others'
-    static __device__ __forceinline__ constexpr int group(int e) { return e >= 3 && e < 6 ? 0 : 1; }
+    // groups: jerk, acceleration, potential
+    static __device__ __forceinline__ constexpr int group(int e) { return e < 3 ? 1 : (e < 6 ? 0 : 2); }
     static __device__ __forceinline__ constexpr bool jneg(int e) { return e < 6; }
-    static __device__ __forceinline__ double bound(const Params &p, int g) {
-        const double m = (double)__uint_as_float(__ldcg(p.mx + kMaxM));
-        const double v = (double)__uint_as_float(__ldcg(p.mx + p.vword));
-        return g == 0 ? p.scale[1] * m * v : p.scale[0] * m;
+    static __device__ __forceinline__ int bound(const Params &p, const Maxima &x, int g) {
+        return p.sexp[g] + x.m + (g == 0 ? x.v : 0);
+    }
+    static __device__ __forceinline__ int shift(const Scales &z, int g) {
+        return g == 0 ? z.m - 3 * z.x : (g == 1 ? z.m - 2 * z.x : z.m - z.x);
+    }
+    static __device__ __forceinline__ constexpr int factor(int a) {
+        return a == 3 ? kFm : (a < 7 ? kFx : kFone);
     }
     static __device__ __forceinline__ const float *plane(const Params &p, int a) {
         return p.soa + a * p.Np;
@@ -381,14 +385,14 @@ struct JerkPh {
 };
 
 // hermite_predict_pack_kernel's pack, one particle a thread, with the largest
-// |m| and |v| component of the packed state.
+// |m|, |v| and |x| component of the packed state.
 __global__ void __launch_bounds__(128) wsym_predict_pack_kernel(
     const double *pos, const double *vel, const double *acc,
     const double *jerk, const double *mass, int64_t N, int64_t Np,
-    double h, float *soa, unsigned *mx, int vword) {
+    double h, float *soa, unsigned *mx) {
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;  // < Np: whole blocks
     float hi[3] = {0.f, 0.f, 0.f}, lo[3] = {0.f, 0.f, 0.f}, vf[3] = {0.f, 0.f, 0.f};
-    float m = 0.f, am = 0.f, av = 0.f;
+    float m = 0.f, am = 0.f, av = 0.f, ax = 0.f;
     dev::grid_trigger();
     dev::grid_wait();
     if (i < N) {
@@ -404,6 +408,7 @@ __global__ void __launch_bounds__(128) wsym_predict_pack_kernel(
             lo[c] = __double2float_rn(x - (double)hi[c]);
             vf[c] = __double2float_rn(v);
             av = fmaxf(av, fabsf(vf[c]));
+            ax = fmaxf(ax, fabsf(hi[c]));
         }
         const double md = mass[i];
         m = __double2float_rn(md);
@@ -413,7 +418,8 @@ __global__ void __launch_bounds__(128) wsym_predict_pack_kernel(
 #pragma unroll
     for (int c = 0; c < 3; ++c) soa[(7 + c) * Np + i] = vf[c];
     warp_max(mx + kMaxM, am);
-    warp_max(mx + vword, av);
+    warp_max(mx + kMaxV, av);
+    warp_max(mx + kMaxX, ax);
 }
 
 // The totals of every particle: read and zeroed, x G, then stored (h = 0) or
@@ -424,7 +430,7 @@ __global__ void __launch_bounds__(128) wsym_jerk_fold_kernel(const Params p, con
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     dev::grid_trigger();
     dev::grid_wait();
-    if (i == 0) mx[kMaxM] = mx[p.vword] = 0u;  // the pair kernel has read them
+    if (i == 0) mx[kMaxM] = mx[kMaxV] = mx[kMaxX] = 0u;  // the pair kernel has read them
     if (i >= p.N) return;
     const int Fj = p.fxe[0], Fa = p.fxe[1];
     const double h = q.h;
@@ -444,7 +450,7 @@ __global__ void __launch_bounds__(128) wsym_jerk_fold_kernel(const Params p, con
         q.jerk[3 * i + c] = j1;
         ok = ok && isfinite(a1) && isfinite(j1);
     }
-    if (POT) q.pot[i] = -q.G * take_fixed(p, 6, i, Fa);
+    if (POT) q.pot[i] = -q.G * take_fixed(p, 6, i, p.fxe[2]);
     if (!ok) dev::set_status(p.status, kStatusNonFinite);
 }
 
@@ -467,18 +473,18 @@ int launch_jerk_wsym(const JerkJob &j, JerkParams q) {
     p.fxe = reinterpret_cast<int *>(j.ws + j.L.wsym_head + 64);
     p.mx = mx;
     p.status = q.status;
-    p.vword = kMaxV0;
     // the bounds: N max|m| times the largest |d| r^3 or r (see nb_wsym.cu), and
     // times the largest |e| r^3 <= |w| (1 + 3 |d|^2 r^2) r^3 <= 1.146 |w| /
     // eps^3 (at |d|^2 r^2 = 1/5) with |w| <= 2 sqrt(3) max|v|
     const double n = 1.02 * (double)j.N;
-    p.scale[0] = n * std::max(0.3849002 / (j.eps * j.eps), 1.0 / j.eps);
-    p.scale[1] = n * 1.146 * 3.4641017 / (j.eps * j.eps * j.eps);
+    p.set_scale(0, n * 1.146 * 3.4641017 / (j.eps * j.eps * j.eps));
+    p.set_scale(1, n * 0.3849002 / (j.eps * j.eps));
+    p.set_scale(2, n / j.eps);
     for (int64_t n = 0; n < (j.nsteps > 0 ? j.nsteps : 1); ++n) {
         q.h = j.nsteps > 0 ? j.h : 0.0;
         int rc = launch_pdl(wsym_predict_pack_kernel, (unsigned)(j.L.Np / 128), 128, 0, j.stream,
                             j.pos, j.vel, j.acc, j.jerk, j.mass, j.N, j.L.Np, q.h,
-                            reinterpret_cast<float *>(j.ws + j.L.packA), mx, p.vword);
+                            reinterpret_cast<float *>(j.ws + j.L.packA), mx);
         if (rc) return rc;
         if (j.N >= kJerkWideMinN)
             rc = q.pot ? launch_pairs<JerkPh<true, true>>(p, j.stream)

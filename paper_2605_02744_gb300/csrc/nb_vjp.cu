@@ -574,12 +574,15 @@ struct VjpPh {
     };
     static __device__ __forceinline__ constexpr int group(int e) { return e < 3 ? 0 : (e == 3 ? 1 : 2); }
     static __device__ __forceinline__ constexpr bool jneg(int e) { return e != 3; }
-    static __device__ __forceinline__ double bound(const Params &p, int g) {
-        const double m = (double)__uint_as_float(__ldcg(p.mx + kMaxM));
-        const double c = (double)__uint_as_float(__ldcg(p.mx + kMaxC));
-        const double b = (double)__uint_as_float(__ldcg(p.mx + kMaxP));
-        if (g == 0) return m * (p.scale[0] * c + p.scale[1] * b);
-        return g == 1 ? p.scale[2] * c + p.scale[3] * b : p.scale[4] * m;
+    static __device__ __forceinline__ int bound(const Params &p, const Maxima &x, int g) {
+        if (g == 0) return x.m + max(p.sexp[0] + x.c, p.sexp[1] + x.p) + 1;
+        return g == 1 ? max(p.sexp[2] + x.c, p.sexp[3] + x.p) + 1 : p.sexp[4] + x.m;
+    }
+    static __device__ __forceinline__ int shift(const Scales &z, int g) {
+        return g == 0 ? z.m + z.c - 3 * z.x : (g == 1 ? z.c : z.m) - 2 * z.x;
+    }
+    static __device__ __forceinline__ constexpr int factor(int a) {
+        return a == 3 ? kFm : (a < 3 || a >= JL ? kFx : (a < 7 ? kFc : kFp));
     }
     // packed planes: x y z m, cx cy cz, (pbar,) (x.lo y.lo z.lo)
     static __device__ __forceinline__ const float *plane(const Params &p, int a) {
@@ -672,7 +675,7 @@ struct VjpPh {
 };
 
 // Positions, masses and cotangents in one pass: launch_pack's and
-// pack_cotangent_kernel's arrays, with the largest |m|, |c| and |pbar|.
+// pack_cotangent_kernel's arrays, with the largest |m|, |x|, |c| and |pbar|.
 __global__ void __launch_bounds__(128) wsym_vjp_pack_kernel(
     const double *pos, const double *mass,
     const double *abar, const double *pbar, double *vbar,
@@ -680,7 +683,7 @@ __global__ void __launch_bounds__(128) wsym_vjp_pack_kernel(
     int64_t Np, float *soa, float *csoa, unsigned *mx) {
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;  // < Np: whole blocks
     float hi[3] = {0.f, 0.f, 0.f}, lo[3] = {0.f, 0.f, 0.f}, cf[3] = {0.f, 0.f, 0.f};
-    float m = 0.f, pb = 0.f, ac = 0.f;
+    float m = 0.f, pb = 0.f, ac = 0.f, ax = 0.f;
     dev::grid_trigger();
     dev::grid_wait();
     if (i < N) {
@@ -689,6 +692,7 @@ __global__ void __launch_bounds__(128) wsym_vjp_pack_kernel(
             const double x = pos[3 * i + e];
             hi[e] = __double2float_rn(x);
             lo[e] = __double2float_rn(x - (double)hi[e]);
+            ax = fmaxf(ax, fabsf(hi[e]));
             double c;
             if (step_form) {
                 const double v = vbar[3 * i + e] + drift * xbar[3 * i + e];
@@ -708,6 +712,7 @@ __global__ void __launch_bounds__(128) wsym_vjp_pack_kernel(
     for (int e = 0; e < 3; ++e) csoa[e * Np + i] = cf[e];
     csoa[3 * Np + i] = pb;
     warp_max(mx + kMaxM, fabsf(m));
+    warp_max(mx + kMaxX, ax);
     warp_max(mx + kMaxC, ac);
     warp_max(mx + kMaxP, fabsf(pb));
 }
@@ -720,7 +725,7 @@ __global__ void __launch_bounds__(128) wsym_vjp_fold_kernel(const Params p, cons
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     dev::grid_trigger();
     dev::grid_wait();
-    if (i == 0) mx[kMaxM] = mx[kMaxC] = mx[kMaxP] = 0u;  // the pair kernel has read them
+    if (i == 0) mx[kMaxM] = mx[kMaxX] = mx[kMaxC] = mx[kMaxP] = 0u;  // the pair kernel has read them
     if (i >= p.N) return;
     const int Fx = p.fxe[0], Fm = p.fxe[1];
     bool ok = true;
@@ -769,11 +774,11 @@ int launch_vjp_wsym(const VjpJob &j, bool pb, bool fused) {
     // max|c|, |e| r^3 <= 1.146 |w| / eps^3 (nb_jerk.cu), |d| r^3 <= 0.385 /
     // eps^2 and r <= 1 / eps
     const double n = 1.02 * (double)j.N, e1 = 1.0 / j.eps, e2 = 0.3849002 * e1 * e1;
-    p.scale[0] = n * 1.146 * 3.4641017 * e1 * e1 * e1;
-    p.scale[1] = n * 2.0 * e2;
-    p.scale[2] = n * 1.7320509 * e2;
-    p.scale[3] = n * e1;
-    p.scale[4] = n * e2;
+    p.set_scale(0, n * 1.146 * 3.4641017 * e1 * e1 * e1);
+    p.set_scale(1, n * 2.0 * e2);
+    p.set_scale(2, n * 1.7320509 * e2);
+    p.set_scale(3, n * e1);
+    p.set_scale(4, n * e2);
     int rc = launch_pdl(wsym_vjp_pack_kernel, (unsigned)(j.L.Np / 128), 128, 0, j.stream, j.pos,
                         j.mass, j.acc_bar, j.pot_bar, j.vel_bar, j.pos_bar, j.drift_dt,
                         j.kick_coef, j.step_form ? 1 : 0, j.N, j.L.Np, soa, csoa, mx);

@@ -20,17 +20,23 @@ namespace {
 template <bool IPAIR_, int K_, int WARPS_, bool SPLIT, bool POT>
 struct ForcePh {
     static constexpr bool IPAIR = IPAIR_;
-    static constexpr int K = K_, WARPS = WARPS_, NJ = SPLIT ? 7 : 4, NC = POT ? 4 : 3, GROUPS = 1;
+    static constexpr int K = K_, WARPS = WARPS_, NJ = SPLIT ? 7 : 4, NC = POT ? 4 : 3;
+    static constexpr int GROUPS = POT ? 2 : 1;
     struct S {
         float2 nx[K], ny[K], nz[K], m[K];
         LoT<IPAIR> nxl[K], nyl[K], nzl[K];
         float2 a[K][NC];
     };
-    static __device__ __forceinline__ constexpr int group(int) { return 0; }
+    static __device__ __forceinline__ constexpr int group(int e) { return e < 3 ? 0 : 1; }
     static __device__ __forceinline__ constexpr bool jneg(int e) { return e < 3; }
-    static __device__ __forceinline__ double bound(const Params &p, int) {
-        return p.scale[0] * (double)__uint_as_float(__ldcg(p.mx + kMaxM));
+    static __device__ __forceinline__ int bound(const Params &p, const Maxima &x, int g) {
+        return p.sexp[g] + x.m;
     }
+    // groups: accelerations, potential
+    static __device__ __forceinline__ int shift(const Scales &z, int g) {
+        return g == 0 ? z.m - 2 * z.x : z.m - z.x;
+    }
+    static __device__ __forceinline__ constexpr int factor(int a) { return a == 3 ? kFm : kFx; }
     static __device__ __forceinline__ const float *plane(const Params &p, int a) {
         return p.soa + a * p.Np;
     }
@@ -82,7 +88,7 @@ struct ForcePh {
 };
 
 // Pack of the positions and masses after an optional kick and drift
-// (v += kick a; x += drift v), and the largest |m|.
+// (v += kick a; x += drift v), and the largest |m| and |x|.
 __global__ void __launch_bounds__(128) wsym_pack_kernel(double *pos,
                                                         double *vel,
                                                         const double *acc,
@@ -90,7 +96,7 @@ __global__ void __launch_bounds__(128) wsym_pack_kernel(double *pos,
                                                         int64_t Np, double kick, double drift,
                                                         float *soa, unsigned *mx) {
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;  // < Np: whole blocks
-    float hi[3] = {0.f, 0.f, 0.f}, lo[3] = {0.f, 0.f, 0.f}, m = 0.f, am = 0.f;
+    float hi[3] = {0.f, 0.f, 0.f}, lo[3] = {0.f, 0.f, 0.f}, m = 0.f, am = 0.f, ax = 0.f;
     dev::grid_trigger();
     dev::grid_wait();
     if (i < N) {
@@ -109,9 +115,11 @@ __global__ void __launch_bounds__(128) wsym_pack_kernel(double *pos,
         const double md = mass[i];
         m = __double2float_rn(md);
         am = __double2float_ru(fabs(md));
+        ax = fmaxf(fabsf(hi[0]), fmaxf(fabsf(hi[1]), fabsf(hi[2])));
     }
     store_packed(soa, Np, i, hi, lo, m);
     warp_max(mx + kMaxM, am);
+    warp_max(mx + kMaxX, ax);
 }
 
 // The totals of every particle: read and zeroed, x G, stored, with an optional
@@ -129,7 +137,7 @@ __global__ void __launch_bounds__(128) wsym_fold_kernel(const Params p, double G
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     dev::grid_trigger();
     dev::grid_wait();
-    if (!NEXT && i == 0) mx[kMaxM] = 0u;  // for the next call
+    if (!NEXT && i == 0) mx[kMaxM] = mx[kMaxX] = 0u;  // for the next call
     if (i >= p.N) return;
     const int F = *p.fxe;
     double x0[3], v0[3];
@@ -162,7 +170,7 @@ __global__ void __launch_bounds__(128) wsym_fold_kernel(const Params p, double G
         }
     }
     if (!NEXT && pot) {
-        const double gp = -G * take_fixed(p, 3, i, F);
+        const double gp = -G * take_fixed(p, 3, i, p.fxe[1]);
         pot[i] = gp;
         ok = ok && isfinite(gp);
     }
@@ -186,9 +194,10 @@ Params params_of(const ForceJob &j) {
     p.mx = maxima(j);
     p.status = reinterpret_cast<uint32_t *>(j.ws + j.L.status);
     // every partial and total: N max|m| times the largest |d| (|d|^2 +
-    // eps^2)^-3/2 (0.385 / eps^2) or (|d|^2 + eps^2)^-1/2 (1 / eps), x 1.02
+    // eps^2)^-3/2 (0.385 / eps^2) and (|d|^2 + eps^2)^-1/2 (1 / eps), x 1.02
     // for the rounding of the FP32 partial sums
-    p.scale[0] = 1.02 * (double)j.N * std::max(0.3849002 / (j.eps * j.eps), 1.0 / j.eps);
+    p.set_scale(0, 1.02 * (double)j.N * 0.3849002 / (j.eps * j.eps));
+    p.set_scale(1, 1.02 * (double)j.N / j.eps);
     return p;
 }
 

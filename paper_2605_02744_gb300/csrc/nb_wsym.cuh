@@ -48,6 +48,7 @@
 #pragma once
 
 #include <cuda_runtime.h>
+#include <math.h>
 #include <stdint.h>
 
 #include <algorithm>
@@ -82,15 +83,43 @@ struct Params {
     unsigned long long *fx;  // [components][4 limbs][Np] fixed-point totals
     int *fxe;                // [kMaxGroups] the call's exponents (written here)
     const unsigned *mx;      // maxima of the inputs (float bits), see MaxWord
-    int vword;               // which of the two max |v| words this evaluation reads
-    double scale[5];         // factors of the a-priori bounds, see each physics' bound()
+    int sexp[5];             // exponents of the factors of the a-priori bounds (set_scale), see
+                             // each physics' bound()
+    void set_scale(int k, double v) { frexp(v, &sexp[k]); }  // v < 2^sexp[k]
     uint32_t *status;
 };
 
-// Words of `mx`: the largest |m|, |v| component (two, used in turn by the
-// steps of a Hermite loop), |c| component and |pbar| of the packed inputs,
+// Words of `mx`: the largest |m|, |v|, |x| and |c| component and |pbar| of the
+// packed inputs,
 // as float bits rounded up (non-negative floats order like their bits).
-enum MaxWord { kMaxM = 0, kMaxV0 = 1, kMaxV1 = 2, kMaxC = 3, kMaxP = 4, kMaxWords = 8 };
+enum MaxWord { kMaxM = 0, kMaxV = 1, kMaxX = 2, kMaxC = 3, kMaxP = 4 };
+
+// Powers of two that bring the packed inputs to order one where they are
+// loaded: lengths, masses, cotangents.  r^-3 leaves the range of FP32 at
+// distances of 4e12 (metres, say), and products of masses and cotangents
+// sooner; powers of two change no rounding, and the fold's exponents undo them.
+struct Scales {
+    int x, m, c;
+};
+// Exponents of the maxima (v < 2^e; fx::kNoBound: not finite), for the bounds:
+// integers, because a few dependent FP64 operations at the start of every
+// kernel cost microseconds on this part.
+struct Maxima {
+    int m, v, c, p;
+};
+enum Factor { kFx = 0, kFm = 1, kFc = 2, kFp = 3, kFone = 4 };  // 2^-x 2^-m 2^-c 2^(x - c)
+
+// e with v < 2^e for the float with these bits (0 for 0, inf and NaN), within
+// +-60, so that every factor is a normal float.
+__device__ __forceinline__ int exponent_of(unsigned bits) {
+    const int f = (int)(bits >> 23);
+    return f == 0 || f == 0xff ? 0 : min(max(f - 126, -60), 60);
+}
+__device__ __forceinline__ int bound_exponent(unsigned bits) {
+    const int f = (int)(bits >> 23);
+    return f == 0xff ? fx::kNoBound : f == 0 ? -126 : f - 126;
+}
+__device__ __forceinline__ float pow2f(int e) { return __uint_as_float((unsigned)(127 + e) << 23); }
 
 // Folds the warp's largest |v| into a max word (all 32 lanes call it).
 __device__ __forceinline__ void warp_max(unsigned *word, float v) {
@@ -233,13 +262,13 @@ __global__ void __launch_bounds__(Geo<PH>::NTHR, 1) wsym_kernel(const Params p) 
     float2 *tot = reinterpret_cast<float2 *>(wsym_smem);  // [NV][NTHR]
     __shared__ int sF[kMaxGroups];
     __shared__ int stag[NWARP];
+    __shared__ float sFac[4];
     const int tid = threadIdx.x, w = tid >> 5, l = tid & 31;
     // the first `extra` warps take one unit more than the others
     const int64_t gw = (int64_t)blockIdx.x * NWARP + w;
     int64_t u = gw * p.per_warp + (gw < p.extra ? gw : p.extra);
     const int64_t u_end = u + p.per_warp + (gw < p.extra ? 1 : 0);
     const int nslots = (int)(p.nb * BW);
-    const float2 e2 = f2(p.eps2, p.eps2);
     uint32_t bad = 0;
     int I = 0, jb = 0, tag = -1;
     if (u < u_end) {
@@ -250,11 +279,34 @@ __global__ void __launch_bounds__(Geo<PH>::NTHR, 1) wsym_kernel(const Params p) 
     // no grid_trigger(): placing the fold's blocks while this kernel fills the
     // SMs cost 10 us a step (2047: 21.8 / 11.6 us, 16384: 128.6 / 117.6 us)
     dev::grid_wait();
-    if (tid < PH::GROUPS) {
-        sF[tid] = fx::limb_exponent_for(PH::bound(p, tid));
-        if (blockIdx.x == 0) p.fxe[tid] = sF[tid];
+    if (w == 0) {
+        const unsigned bx = __ldcg(p.mx + kMaxX), bm = __ldcg(p.mx + kMaxM),
+                       bv = __ldcg(p.mx + kMaxV), bc = __ldcg(p.mx + kMaxC),
+                       bp = __ldcg(p.mx + kMaxP);
+        Scales z;
+        z.x = exponent_of(bx);
+        z.m = exponent_of(bm);
+        z.c = min(max(exponent_of(bc), exponent_of(bp) + z.x), 60);
+        const Maxima mm = {bound_exponent(bm), bound_exponent(bv), bound_exponent(bc),
+                           bound_exponent(bp)};
+        if (l < PH::GROUPS) {
+            const int up = PH::shift(z, l);
+            const int Fg = fx::limb_exponent(PH::bound(p, mm, l) - up);
+            sF[l] = Fg;
+            // value = 2^up (scaled value)
+            if (blockIdx.x == 0) p.fxe[l] = Fg == fx::kNoGrid ? Fg : Fg - up;
+        }
+        if (l == 0) {
+            sFac[kFx] = pow2f(-z.x);
+            sFac[kFm] = pow2f(-z.m);
+            sFac[kFc] = pow2f(-z.c);
+            sFac[kFp] = pow2f(z.x - z.c);
+        }
     }
     __syncthreads();
+    // eps^2 in scaled lengths (at least the smallest normal float)
+    const float es = fmaxf(p.eps2 * sFac[kFx] * sFac[kFx], 1.17549435e-38f);
+    const float2 e2 = f2(es, es);
     int F[PH::GROUPS];
 #pragma unroll
     for (int g = 0; g < PH::GROUPS; ++g) F[g] = sF[g];
@@ -306,8 +358,9 @@ __global__ void __launch_bounds__(Geo<PH>::NTHR, 1) wsym_kernel(const Params p) 
 #pragma unroll
                 for (int a = 0; a < PH::NJ; ++a) {
                     const float *q = PH::plane(p, a) + I * BW + (PH::IPAIR ? 64 : 32) * k + l;
-                    v[a].x = q[0];
-                    v[a].y = PH::IPAIR ? q[32] : v[a].x;
+                    const float fa = PH::factor(a) == kFone ? 1.f : sFac[PH::factor(a)];
+                    v[a].x = q[0] * fa;
+                    v[a].y = PH::IPAIR ? q[32] * fa : v[a].x;
                 }
                 PH::set_i(S, k, v);
 #pragma unroll
@@ -320,7 +373,10 @@ __global__ void __launch_bounds__(Geo<PH>::NTHR, 1) wsym_kernel(const Params p) 
         }
         float jc[GE::JL * PH::NJ];
 #pragma unroll
-        for (int a = 0; a < GE::JL * PH::NJ; ++a) jc[a] = jn[a];
+        for (int a = 0; a < GE::JL * PH::NJ; ++a) {  // scaled here: the prefetch must not wait
+            const int fa = PH::factor(a % PH::NJ);
+            jc[a] = fa == kFone ? jn[a] : jn[a] * sFac[fa];
+        }
         u += un;
         const int jnext = jb + JSET;
         const bool row_end = jnext >= nslots;

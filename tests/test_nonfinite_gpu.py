@@ -77,3 +77,32 @@ def test_fp64_masses_outside_the_fp32_range(scale):
     ra, rp = oracle.forces(s.pos, s.mass, EPS)
     assert rel_vec_err(host(acc) / scale, ra).max() <= 1e-12
     assert rel_err(host(pot) / scale, rp).max() <= 1e-12
+
+
+@pytest.mark.parametrize("length,mass_unit", [(3e12, 2e30), (1e-9, 1e-20), (1e15, 1e-3)])
+def test_units_far_from_one(length, mass_unit):
+    """Systems in units where r^-3 or products of masses and cotangents leave
+    the range of FP32 give the scaled results of the same system in units of
+    order one."""
+    n = 5000
+    s = ics.plummer_lognormal(n, seed=6)
+    o = binding.make_opts("f64acc", positions="split")
+    ws = binding.workspace(n, 1, o)
+    cot = np.random.default_rng(6).normal(size=(n, 3)) * 1e-12
+    pbar = np.random.default_rng(7).normal(size=n) * 1e-12 / length
+    ra, rj, rp = oracle.forces_jerk(s.pos, s.vel, s.mass, EPS)
+    rx, rm = oracle.forces_vjp(s.pos, s.mass, EPS, cot, pbar * length)
+    pos, vel, mass = dev(s.pos * length), dev(s.vel), dev(s.mass * mass_unit)
+    acc, jerk, xb = (torch.empty_like(pos) for _ in range(3))
+    pot, mb = torch.empty_like(mass), torch.empty_like(mass)
+    ka, kp = mass_unit / length ** 2, mass_unit / length
+    binding.nb_forces(pos, mass, EPS * length, acc, pot, ws, o)
+    assert rel_vec_err(host(acc) / ka, ra).max() <= 1e-5
+    assert rel_err(host(pot) / kp, rp).max() <= 1e-5
+    binding.nb_forces_jerk(pos, vel, mass, EPS * length, acc, jerk, pot, ws, o)
+    assert rel_vec_err(host(acc) / ka, ra).max() <= 1e-5
+    assert rel_vec_err(host(jerk) / (ka / length), rj).max() <= 1e-4
+    binding.nb_forces_vjp(pos, mass, EPS * length, dev(cot), dev(pbar), xb, mb, ws, o)
+    assert binding.nb_poll_status(ws, o) == binding.NB_OK
+    assert np.abs(host(xb) / (ka / length) - rx).max() <= 2e-6 * np.abs(rx).max()
+    assert np.abs(host(mb) * length ** 2 - rm).max() <= 2e-6 * np.abs(rm).max()
