@@ -368,8 +368,8 @@ __device__ __forceinline__ void store_box(float *out, const float (&lo)[3], cons
 // sym_fold_kernel, kick_drift_pack_kernel, pack_sorted_kernel and two
 // slot_boxes_kernel launches do one after the other.  The acceleration is not
 // stored: the next fold replaces it before anything reads it.  At 65536
-// particles the step's kernels besides the pair kernel took 76 us (ncu), the
-// ten launches of them; now four.
+// particles the ten launches of a step besides the pair kernel took 76 us
+// (ncu); now they are four, 28 us.
 __global__ void __launch_bounds__(256) sym_fold_next_kernel(
     const SymParams p, int64_t N, const int *perm, double G, double *pos, double *vel, double kick,
     double next_kick, double drift, float *soa, float *jbox, float *wbox) {

@@ -560,8 +560,8 @@ using namespace wsym;
 template <bool PB, bool FUSED, bool SPLIT>
 struct VjpPh {
     // four i-slots a lane as two (x_a, x_b) pairs against one j-particle, 16
-    // warps of 128 registers: 944 us fused at 32768, against 1001 us for four
-    // broadcast i-slots against two j with 8 warps (268 / 276 us at 16384)
+    // warps of 128 registers: 949 us fused at 32768, against 1054 us for four
+    // broadcast i-slots against two j with 8 warps (265 / 284 us at 16384)
     static constexpr bool IPAIR = true;
     static constexpr int K = 2, WARPS = 16;
     static constexpr int NJ = 7 + (PB ? 1 : 0) + (SPLIT ? 3 : 0);

@@ -40,11 +40,11 @@
 // operands reads six registers and issues at 64 % of the FP32 peak (two
 // distinct: 95 %; measured on chains of independent operations), and 6 of a
 // force pair's 16, 17 of a jerk pair's 39 operations are of that kind: about
-// 80 % of the peak is the ceiling, 62 to 70 % is reached (ncu, 16384 and 32768
-// particles), whatever the number of warps, the order of the operations in
-// the source or the unrolling.  GB300, 16384 particles, one evaluation: F64ACC
-// forces 195 -> 118 us, acceleration + jerk 945 -> 245 us, VJP 333 -> 202 us
-// against the direct kernels.
+// 80 % of the peak is the ceiling, and the pipe is busy 70 % of the time (ncu,
+// 16384 and 32768 particles), whatever the number of warps, the order of the
+// operations in the source or the unrolling.  GB300, 16384 particles, one
+// evaluation with its pack and fold: F64ACC forces 195 -> 123 us, acceleration
+// + jerk 945 -> 252 us, VJP 333 -> 200 us against the direct kernels.
 #pragma once
 
 #include <cuda_runtime.h>
