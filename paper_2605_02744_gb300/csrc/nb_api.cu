@@ -226,7 +226,7 @@ WsLayout ws_layout(int64_t N, int32_t B, const nb_opts *opts) {
         L.wsym_fx = off;
         off = align256(off + 8 * fx::kLimbs * kWsymComponents * (size_t)L.Np);
     }
-    if (sym_wanted(opts, N, B)) {
+    if (sym_provisioned(opts, N, B)) {
         const SymSizes z = sym_sizes(L.Np);
         L.sym_fx = off;
         L.sym_fx_bytes = z.fx_bytes;
@@ -259,16 +259,20 @@ static bool shape_asked(const nb_opts *o) {
     return t && (t->threads || t->i_per_thread || t->tile_j || t->stages || t->ctas_per_sm);
 }
 
-bool sym_wanted(const nb_opts *o, int64_t N, int32_t B) {
+bool sym_provisioned(const nb_opts *o, int64_t N, int32_t B) {
     if (!o || B != 1) return false;
     if (o->pairs == NB_PAIRS_SYMMETRIC) return true;
-    if (o->pairs != NB_PAIRS_DEFAULT || N > kSymMaxN) return false;
-    if (N >= kSymMinN) return true;
+    return o->pairs == NB_PAIRS_DEFAULT && N >= kSymMinN && N <= kSymMaxN;
+}
+
+bool sym_wanted(const nb_opts *o, int64_t N, int32_t B) {
+    if (sym_provisioned(o, N, B)) return true;
     // below kSymMinN what asks for the direct kernel gets it: a launch shape,
     // the adaptive displacement (its sorted symmetric form needs large
     // systems), the ring's test hook
-    return o->precision != NB_PREC_FP64 && N >= kWsymMinN && !shape_asked(o) &&
-           o->positions != NB_POS_ADAPTIVE && o->test_unissued_stage == 0;
+    return o && B == 1 && o->pairs == NB_PAIRS_DEFAULT && N >= kWsymMinN && N <= kSymMaxN &&
+           o->precision != NB_PREC_FP64 && !shape_asked(o) && o->positions != NB_POS_ADAPTIVE &&
+           o->test_unissued_stage == 0;
 }
 
 // Whether the VJP or the acceleration + jerk of N particles takes the

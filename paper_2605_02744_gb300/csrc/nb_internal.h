@@ -263,8 +263,11 @@ struct SymLayout {
     unsigned long long *acc_fx;    // [4][2][Np]
 };
 SymLayout sym_layout(char *ws, const WsLayout &L);
-// Whether the symmetric-pair path is provisioned / taken for N particles in
-// B clusters under opts (nb_pairs; FP32-pair policies, single systems).
+// Whether the symmetric-pair path of large systems (adaptive displacement) is
+// provisioned, and whether symmetric pairs are taken, for N particles in B
+// clusters under opts (single systems).  The warp-granular path's region is in
+// every workspace, so below kSymMinN all options need the same size.
+bool sym_provisioned(const nb_opts *opts, int64_t N, int32_t B);
 bool sym_wanted(const nb_opts *opts, int64_t N, int32_t B);
 int launch_force_sym(const ForceJob &job);
 int launch_step_sym(const ForceJob &job, double *vel, double dt, int64_t nsteps, bool acc_valid);
