@@ -15,10 +15,12 @@
  *           8-byte aligned (256-byte for the workspace), C-contiguous.  The
  *           library never allocates or frees device memory; scratch space is
  *           the caller's workspace `ws` of `ws_bytes` bytes, sized with
- *           nb_workspace_bytes() and ZERO-FILLED once before its first use
- *           (the kernels leave their arrival counters at zero on exit, so
- *           later calls need no clearing unless a call reported
- *           NB_ERR_TIMEOUT).  One workspace serves one stream at a time.
+ *           nb_workspace_bytes() and ZERO-FILLED once before its first use.
+ *           From then on it serves any entry point, size and options that it
+ *           is large enough for, in any order, without clearing unless a
+ *           call reported NB_ERR_TIMEOUT (only its first 256 bytes carry
+ *           anything from one call to the next).  One workspace serves one
+ *           stream at a time.
  * Layout:   positions, velocities, accelerations and their cotangents are
  *           double [N][3] row-major; masses, potentials and their cotangents
  *           double [N].  Batched sets concatenate clusters and describe them

@@ -221,8 +221,6 @@ WsLayout ws_layout(int64_t N, int32_t B, const nb_opts *opts) {
     off = align256(off + kScratchBase + batched_scratch_bytes(B));
     if (B == 1 && (N <= kSymMaxN ||
                    (N <= kWsymMaxN && opts && opts->pairs == NB_PAIRS_SYMMETRIC))) {
-        L.wsym_head = off;
-        off = align256(off + 256);
         L.wsym_fx = off;
         off = align256(off + 8 * fx::kLimbs * kWsymComponents * (size_t)L.Np);
     }
@@ -800,7 +798,9 @@ static int step_single_direct(nb_state *s, double dt, int64_t nsteps, const nb_o
     for (int64_t n = 0; n < nsteps; ++n) {
         // the adaptive path packs in Hilbert order inside launch_force
         NB_TRY(launch_kick_drift_pack(s->pos, s->vel, s->acc, s->mass, s->N, j.L.Np, dt,
-                                      j.adaptive ? nullptr : soa, j.stream));
+                                      j.adaptive ? nullptr : soa,
+                                      reinterpret_cast<uint32_t *>(j.ws + j.L.counters),
+                                      j.L.max_blocks, j.stream));
         ForceJob k = j;
         k.packed_ready = !j.adaptive;
         k.reuse_order = j.adaptive && sorted_at >= 0 && n + 1 - sorted_at < kResortEvery;

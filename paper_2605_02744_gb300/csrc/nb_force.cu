@@ -35,10 +35,12 @@ using dev::pair2;
 // FP32 (the split "double-single" representation); entries N..Np-1 are
 // zero-mass particles at the origin.
 __global__ void pack_soa_kernel(const double *__restrict__ pos, const double *__restrict__ mass,
-                                int64_t N, int64_t Np, float *__restrict__ soa) {
+                                int64_t N, int64_t Np, float *__restrict__ soa,
+                                uint32_t *__restrict__ counters, int64_t ncounters) {
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < Np;
          i += (int64_t)gridDim.x * blockDim.x) {
         float hi[3] = {0.f, 0.f, 0.f}, lo[3] = {0.f, 0.f, 0.f}, m = 0.f;
+        if (i < ncounters) counters[i] = 0u;  // fewer than N / 64 + 2
         if (i < N) {
 #pragma unroll
             for (int c = 0; c < 3; ++c) {
@@ -53,10 +55,11 @@ __global__ void pack_soa_kernel(const double *__restrict__ pos, const double *__
 }
 
 int launch_pack(const double *pos, const double *mass, int64_t N, int64_t Np, float *soa,
-                cudaStream_t st) {
+                uint32_t *counters, int64_t ncounters, cudaStream_t st) {
     const int threads = 256;
     const int64_t blocks = std::min<int64_t>(cdiv(Np, threads), 8192);
-    pack_soa_kernel<<<(unsigned)blocks, threads, 0, st>>>(pos, mass, N, Np, soa);
+    pack_soa_kernel<<<(unsigned)blocks, threads, 0, st>>>(pos, mass, N, Np, soa, counters,
+                                                        ncounters);
     count_launch();
     NB_CUDA(cudaGetLastError());
     return NB_OK;
@@ -516,6 +519,7 @@ int launch_force(const ForceJob &j) {
     const Shape &sh0 = j.shape;
     const bool adaptive = j.adaptive && !guard;
     char *sb = j.ws + j.L.sortbuf;
+    uint32_t *counters = reinterpret_cast<uint32_t *>(j.ws + j.L.counters);
     if (j.sym && guard) return fail(NB_ERR_UNSUPPORTED, "symmetric pairs need eps > 0");
     if (takes_wsym(j)) return launch_force_wsym(j);
     if (j.row) return launch_force_row(j);
@@ -524,13 +528,13 @@ int launch_force(const ForceJob &j) {
         // boxes per 64 j-slots and per warp of i-slots (32 IR slots)
         const int tile_unit = 64;
         const int block_unit = 32 * sh0.ipt;
-        int rc = launch_sorted_pack(j.pos, j.mass, j.N, j.L.Np, soa, sort_perm(sb, j.L),
-                                    sort_keys(sb), sort_box6(sb, j.L), sort_tile_boxes(sb, j.L),
+        int rc = launch_sorted_pack(j.pos, j.mass, j.N, j.L.Np, soa, counters, j.L.max_blocks,
+                                    sort_perm(sb, j.L), sort_keys(sb), sort_box6(sb, j.L), sort_tile_boxes(sb, j.L),
                                     tile_unit, sort_block_boxes(sb, j.L), block_unit,
                                     j.reuse_order, j.stream);
         if (rc) return rc;
     } else if (!j.packed_ready) {
-        int rc = launch_pack(j.pos, j.mass, j.N, j.L.Np, soa, j.stream);
+        int rc = launch_pack(j.pos, j.mass, j.N, j.L.Np, soa, counters, j.L.max_blocks, j.stream);
         if (rc) return rc;
     }
     const Shape &sh = j.shape;
@@ -550,7 +554,7 @@ int launch_force(const ForceJob &j) {
     p.vel = j.vel;
     p.kick = j.kick;
     p.records = reinterpret_cast<Record *>(j.ws + j.L.records);
-    p.counters = reinterpret_cast<uint32_t *>(j.ws + j.L.counters);
+    p.counters = counters;
     p.status = status;
     p.timeout = j.timeout;
     p.unissued = j.unissued;

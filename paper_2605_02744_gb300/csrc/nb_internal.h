@@ -88,8 +88,8 @@ int launch_pdl(void (*kernel)(P...), unsigned grid, unsigned block, size_t smem,
 // --------------------------------------------------------- workspace
 // Byte offsets inside the caller's workspace.  Everything is 256-B aligned.
 struct WsLayout {
-    size_t status;    // uint32 status word (+ padding to 256 B)
-    size_t counters;  // uint32 arrival counters, one per i-block
+    size_t status;    // uint32 status word, then the words of HeadWord (256 B)
+    size_t counters;  // uint32 arrival counters, one per i-block (cleared by each call's pack)
     size_t packA;     // float SoA [7][Np]: x.hi y.hi z.hi m x.lo y.lo z.lo
     size_t packB;     // float SoA [4][Np]: VJP cotangents (cx, cy, cz, pbar/3)
     size_t cot64;     // double SoA [4][Np]: the same cotangents in FP64
@@ -97,9 +97,8 @@ struct WsLayout {
     size_t records;   // stream-K partial records
     size_t scratch;   // O(N) reduction scratch (energy partials, batched queue)
     size_t sym_fx;    // symmetric-pair path: fixed-point totals, 64 B per slot
-    size_t sym_cost;  // symmetric-pair path: exponent, item costs, their prefix, CTA ranges
-    size_t wsym_head; // warp-granular path: exponents (at 64), input maxima (at 128, FP64 192; zero between calls)
-    size_t wsym_fx;   // its fixed-point totals, 7 components x 4 limbs per slot (zero between calls)
+    size_t sym_cost;  // symmetric-pair path: item costs, their prefix, CTA ranges
+    size_t wsym_fx;   // warp-granular path: fixed-point totals, 7 components x 4 limbs per slot
     size_t bsym, bsym_bytes;  // batched symmetric-pair path (0 bytes: not provisioned)
     size_t sym_fx_bytes;      // 0 when the symmetric path is not provisioned
     size_t total;
@@ -107,6 +106,20 @@ struct WsLayout {
     int64_t max_blocks;
     int64_t max_grid;
     int64_t record_bytes_per_i;
+};
+
+// Words of the status block beside the status itself.  Maxima and arrivals are
+// zero between calls; they are here because this block is the only part of a
+// workspace that lies at the same place for every size and option, and one
+// workspace serves problems of several: whatever else has to be zero on entry
+// (arrival counters, fixed-point totals) is cleared by the call that uses it.
+enum HeadWord : size_t {
+    kHeadExponents = 64,    // int [3]: the warp-granular and FP64 paths' grids
+    kHeadMaxima = 128,      // uint32 [5]: wsym::MaxWord
+    kHeadSymExponent = 160, // int: the adaptive symmetric path's grid
+    kHeadSymArrivals = 164, // uint32: its blocks done with the reduction
+    kHeadSymMaxMass = 168,  // uint64: its largest |m|, the bits of a double
+    kHeadMaxMass64 = 192,   // uint64: the FP64 path's
 };
 
 WsLayout ws_layout(int64_t N, int32_t B, const nb_opts *opts);
@@ -196,8 +209,9 @@ inline size_t sortbuf_bytes(int64_t Np) {
 // reuse_order: the keys already hold a Hilbert order of these N particles
 // (an earlier call of the same step loop); only the pack and the boxes are
 // redone from the current positions.
+// counters: ncounters arrival counters to clear (0: none).
 int launch_sorted_pack(const double *pos, const double *mass, int64_t N, int64_t Np, float *soa,
-                       int *perm, unsigned long long *keys, long long *box6, float *tile_boxes,
+                       uint32_t *counters, int64_t ncounters, int *perm, unsigned long long *keys, long long *box6, float *tile_boxes,
                        int tile_unit, float *block_boxes, int block_unit, bool reuse_order,
                        cudaStream_t st);
 
@@ -216,8 +230,9 @@ __host__ __device__ inline void store_packed(float *soa, int64_t Np, int64_t i, 
     soa[6 * Np + i] = lo[2];
 }
 
+// Packs the positions and masses and clears ncounters arrival counters.
 int launch_pack(const double *pos, const double *mass, int64_t N, int64_t Np, float *soa,
-                cudaStream_t st);
+                uint32_t *counters, int64_t ncounters, cudaStream_t st);
 int launch_force(const ForceJob &job);
 
 // ------------------------------------------------- symmetric-pair path
@@ -331,7 +346,8 @@ struct VjpJob {
 int launch_vjp(const VjpJob &job);
 
 int launch_kick_drift_pack(double *pos, double *vel, const double *acc, const double *mass,
-                           int64_t N, int64_t Np, double dt, float *soa, cudaStream_t st);
+                           int64_t N, int64_t Np, double dt, float *soa, uint32_t *counters,
+                           int64_t ncounters, cudaStream_t st);
 // v += kick a; x += drift v for n particles (FP64).
 int launch_kick_drift(double *pos, double *vel, const double *acc, int64_t n, double kick,
                       double drift, cudaStream_t st);

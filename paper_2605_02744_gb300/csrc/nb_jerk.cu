@@ -385,16 +385,17 @@ struct JerkPh {
 };
 
 // hermite_predict_pack_kernel's pack, one particle a thread, with the largest
-// |m|, |v| and |x| component of the packed state.
+// |m|, |v| and |x| component of the packed state, and cleared totals.
 __global__ void __launch_bounds__(128) wsym_predict_pack_kernel(
     const double *pos, const double *vel, const double *acc,
     const double *jerk, const double *mass, int64_t N, int64_t Np,
-    double h, float *soa, unsigned *mx) {
+    double h, float *soa, unsigned *mx, unsigned long long *fx, int nc) {
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;  // < Np: whole blocks
     float hi[3] = {0.f, 0.f, 0.f}, lo[3] = {0.f, 0.f, 0.f}, vf[3] = {0.f, 0.f, 0.f};
     float m = 0.f, am = 0.f, av = 0.f, ax = 0.f;
     dev::grid_trigger();
     dev::grid_wait();
+    if (clear_totals(fx, Np, N, Np, nc)) return;
     if (i < N) {
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
@@ -422,7 +423,7 @@ __global__ void __launch_bounds__(128) wsym_predict_pack_kernel(
     warp_max(mx + kMaxX, ax);
 }
 
-// The totals of every particle: read and zeroed, x G, then stored (h = 0) or
+// The totals of every particle: read, x G, then stored (h = 0) or
 // taken through the Hermite corrector, as jerk_kernel's epilogue.
 template <bool POT>
 __global__ void __launch_bounds__(128) wsym_jerk_fold_kernel(const Params p, const JerkParams q,
@@ -437,8 +438,8 @@ __global__ void __launch_bounds__(128) wsym_jerk_fold_kernel(const Params p, con
     bool ok = true;
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-        const double a1 = q.G * take_fixed(p, c, i, Fa);
-        const double j1 = q.G * take_fixed(p, 3 + c, i, Fj);
+        const double a1 = q.G * take_fixed<false>(p, c, i, Fa);
+        const double j1 = q.G * take_fixed<false>(p, 3 + c, i, Fj);
         if (h != 0.0) {
             const double x0 = q.pos[3 * i + c], v0 = q.vel[3 * i + c];
             const double a0 = q.acc[3 * i + c], j0 = q.jerk[3 * i + c];
@@ -450,7 +451,7 @@ __global__ void __launch_bounds__(128) wsym_jerk_fold_kernel(const Params p, con
         q.jerk[3 * i + c] = j1;
         ok = ok && isfinite(a1) && isfinite(j1);
     }
-    if (POT) q.pot[i] = -q.G * take_fixed(p, 6, i, p.fxe[2]);
+    if (POT) q.pot[i] = -q.G * take_fixed<false>(p, 6, i, p.fxe[2]);
     if (!ok) dev::set_status(p.status, kStatusNonFinite);
 }
 
@@ -462,7 +463,7 @@ __global__ void __launch_bounds__(128) wsym_jerk_fold_kernel(const Params p, con
 constexpr int64_t kJerkWideMinN = 12288;
 
 int launch_jerk_wsym(const JerkJob &j, JerkParams q) {
-    unsigned *mx = reinterpret_cast<unsigned *>(j.ws + j.L.wsym_head + 128);
+    unsigned *mx = reinterpret_cast<unsigned *>(j.ws + j.L.status + kHeadMaxima);
     Params p{};
     p.soa = q.soa;
     p.Np = j.L.Np;
@@ -470,7 +471,7 @@ int launch_jerk_wsym(const JerkJob &j, JerkParams q) {
     p.eps2 = q.eps2;
     p.keep = j.precision != NB_PREC_FP32;
     p.fx = reinterpret_cast<unsigned long long *>(j.ws + j.L.wsym_fx);
-    p.fxe = reinterpret_cast<int *>(j.ws + j.L.wsym_head + 64);
+    p.fxe = reinterpret_cast<int *>(j.ws + j.L.status + kHeadExponents);
     p.mx = mx;
     p.status = q.status;
     // the bounds: N max|m| times the largest |d| r^3 or r (see nb_wsym.cu), and
@@ -480,11 +481,13 @@ int launch_jerk_wsym(const JerkJob &j, JerkParams q) {
     p.set_scale(0, n * 1.146 * 3.4641017 / (j.eps * j.eps * j.eps));
     p.set_scale(1, n * 0.3849002 / (j.eps * j.eps));
     p.set_scale(2, n / j.eps);
+    const int nc = q.pot ? 7 : 6;
     for (int64_t n = 0; n < (j.nsteps > 0 ? j.nsteps : 1); ++n) {
         q.h = j.nsteps > 0 ? j.h : 0.0;
-        int rc = launch_pdl(wsym_predict_pack_kernel, (unsigned)(j.L.Np / 128), 128, 0, j.stream,
+        int rc = launch_pdl(wsym_predict_pack_kernel, pack_blocks(j.L.Np, j.N), 128, 0, j.stream,
                             j.pos, j.vel, j.acc, j.jerk, j.mass, j.N, j.L.Np, q.h,
-                            reinterpret_cast<float *>(j.ws + j.L.packA), mx);
+                            reinterpret_cast<float *>(j.ws + j.L.packA), mx, p.fx,
+                            nc);
         if (rc) return rc;
         if (j.N >= kJerkWideMinN)
             rc = q.pot ? launch_pairs<JerkPh<true, true>>(p, j.stream)

@@ -122,11 +122,13 @@ __global__ void bitonic_global_kernel(unsigned long long *keys, int64_t P, int64
 
 __global__ void pack_sorted_kernel(const double *__restrict__ pos, const double *__restrict__ mass,
                                    const unsigned long long *__restrict__ keys, int64_t N,
-                                   int64_t Np, float *__restrict__ soa, int *__restrict__ perm) {
+                                   int64_t Np, float *__restrict__ soa, int *__restrict__ perm,
+                                   uint32_t *__restrict__ counters, int64_t ncounters) {
     for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < Np;
          s += (int64_t)gridDim.x * blockDim.x) {
         float hi[3] = {0.f, 0.f, 0.f}, lo[3] = {0.f, 0.f, 0.f}, m = 0.f;
         int idx = -1;
+        if (s < ncounters) counters[s] = 0u;
         if (s < N) {
             idx = (int)(uint32_t)(keys[s] & 0xffffffffull);
 #pragma unroll
@@ -195,7 +197,7 @@ int64_t sort_keys_len(int64_t N) {
 }
 
 int launch_sorted_pack(const double *pos, const double *mass, int64_t N, int64_t Np, float *soa,
-                       int *perm, unsigned long long *keys, long long *box6, float *tile_boxes,
+                       uint32_t *counters, int64_t ncounters, int *perm, unsigned long long *keys, long long *box6, float *tile_boxes,
                        int tile_unit, float *block_boxes, int block_unit, bool reuse_order,
                        cudaStream_t st) {
     const int64_t P = sort_keys_len(N);
@@ -225,7 +227,7 @@ int launch_sorted_pack(const double *pos, const double *mass, int64_t N, int64_t
     }
 pack:
     pack_sorted_kernel<<<(unsigned)std::min<int64_t>(cdiv(Np, threads), 8192), threads, 0, st>>>(
-        pos, mass, keys, N, Np, soa, perm);
+        pos, mass, keys, N, Np, soa, perm, counters, ncounters);
     count_launch();
     // every unit up to Np: units past N get an empty box (never near)
     slot_boxes_kernel<<<(unsigned)(Np / tile_unit), 256, 0, st>>>(soa, N, Np, tile_unit,

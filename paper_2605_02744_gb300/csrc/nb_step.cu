@@ -19,7 +19,8 @@ namespace nb {
 __global__ void kick_drift_pack_kernel(double *__restrict__ pos, double *__restrict__ vel,
                                        const double *__restrict__ acc,
                                        const double *__restrict__ mass, int64_t N, int64_t Np,
-                                       double dt, float *__restrict__ soa) {
+                                       double dt, float *__restrict__ soa,
+                                       uint32_t *__restrict__ counters, int64_t ncounters) {
     const double half = 0.5 * dt;
     const int64_t n_iter = soa ? Np : N;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n_iter;
@@ -38,16 +39,20 @@ __global__ void kick_drift_pack_kernel(double *__restrict__ pos, double *__restr
             }
             m = __double2float_rn(mass[i]);
         }
-        if (soa) store_packed(soa, Np, i, hi, lo, m);
+        if (soa) {
+            store_packed(soa, Np, i, hi, lo, m);
+            if (i < ncounters) counters[i] = 0u;
+        }
     }
 }
 
 int launch_kick_drift_pack(double *pos, double *vel, const double *acc, const double *mass,
-                           int64_t N, int64_t Np, double dt, float *soa, cudaStream_t st) {
+                           int64_t N, int64_t Np, double dt, float *soa, uint32_t *counters,
+                           int64_t ncounters, cudaStream_t st) {
     const int threads = 256;
     const int64_t blocks = std::min<int64_t>(cdiv(Np, threads), 8192);
     kick_drift_pack_kernel<<<(unsigned)blocks, threads, 0, st>>>(pos, vel, acc, mass, N, Np, dt,
-                                                                 soa);
+                                                                 soa, counters, ncounters);
     count_launch();
     NB_CUDA(cudaGetLastError());
     return NB_OK;

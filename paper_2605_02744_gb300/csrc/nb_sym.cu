@@ -441,16 +441,20 @@ __global__ void __launch_bounds__(256) sym_fold_next_kernel(
 // (independent loads, four per thread in flight) and folds it into one word
 // with an integer atomicMax on the bits (non-negative doubles order like
 // their bit patterns, so the maximum is exact and F reproducible); the last
-// block to finish (arrival counter) computes F and resets both words.
+// block to finish (arrival counter) computes F and resets both words.  The
+// totals are cleared here too: the workspace may have served another size.
 __global__ void __launch_bounds__(256) sym_exponent_kernel(const double *__restrict__ mass,
                                                            int64_t N, double eps,
                                                            int *__restrict__ F,
                                                            unsigned long long *mmax_bits,
-                                                           unsigned *arrivals) {
+                                                           unsigned *arrivals, ulonglong2 *totals,
+                                                           int64_t ntotals) {
     __shared__ double part[8];
     __shared__ bool last;
     double m = 0.0;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < ntotals; i += stride)
+        totals[i] = make_ulonglong2(0ull, 0ull);
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < N; i += 4 * stride) {
         double v[4];
 #pragma unroll
@@ -653,7 +657,8 @@ int launch_split(const SymParams &p, const ForceJob &j, const SymLayout &y, bool
                           j.stream, p, y.prefix, y.lo));
     if (!exponent) return NB_OK;
     sym_exponent_kernel<<<(unsigned)std::min<int64_t>(cdiv(j.N, 4 * 256), 1024), 256, 0,
-                          j.stream>>>(j.mass, j.N, j.eps, y.fx_exp, y.mmax_bits, y.arrivals);
+                          j.stream>>>(j.mass, j.N, j.eps, y.fx_exp, y.mmax_bits, y.arrivals,
+                                      reinterpret_cast<ulonglong2 *>(y.acc_fx), 4 * p.Np);
     count_launch();
     NB_CUDA(cudaGetLastError());
     return NB_OK;
@@ -708,7 +713,7 @@ SymParams params_of(const ForceJob &j, const SymLayout &y) {
 int sorted_pack(const ForceJob &j, bool reuse_order) {
     char *sb = j.ws + j.L.sortbuf;
     return launch_sorted_pack(j.pos, j.mass, j.N, j.L.Np, reinterpret_cast<float *>(j.ws + j.L.packA),
-                              sort_perm(sb, j.L), sort_keys(sb), sort_box6(sb, j.L),
+                              nullptr, 0, sort_perm(sb, j.L), sort_keys(sb), sort_box6(sb, j.L),
                               sort_tile_boxes(sb, j.L), JSP, sort_block_boxes(sb, j.L), WS,
                               reuse_order, j.stream);
 }
@@ -722,7 +727,7 @@ SymSizes sym_sizes(int64_t Np) {
     z.U = z.T * US;
     z.ctas = std::min<int64_t>(CPS * (int64_t)device_sm_count(), z.U);
     z.fx_bytes = 8 * 8 * (size_t)(z.nb * kSymBlock);  // 4 components x 2 words per slot
-    z.cost_bytes = 256 + align_up(4 * (size_t)z.T, 256) + align_up(8 * (size_t)(z.T + 1), 256) +
+    z.cost_bytes = align_up(4 * (size_t)z.T, 256) + align_up(8 * (size_t)(z.T + 1), 256) +
                    8 * (size_t)(z.ctas + 1);
     return z;
 }
@@ -730,13 +735,13 @@ SymSizes sym_sizes(int64_t Np) {
 SymLayout sym_layout(char *ws, const WsLayout &L) {
     const SymSizes z = sym_sizes(L.Np);
     SymLayout y;
-    char *c = ws + L.sym_cost;
-    y.fx_exp = reinterpret_cast<int *>(c);
-    y.mmax_bits = reinterpret_cast<unsigned long long *>(c + 8);
-    y.arrivals = reinterpret_cast<unsigned *>(c + 16);
-    y.cost = reinterpret_cast<uint32_t *>(c + 256);
-    y.prefix = reinterpret_cast<unsigned long long *>(c + 256 + align_up(4 * (size_t)z.T, 256));
-    y.lo = reinterpret_cast<int64_t *>(c + 256 + align_up(4 * (size_t)z.T, 256) +
+    char *c = ws + L.sym_cost, *head = ws + L.status;
+    y.fx_exp = reinterpret_cast<int *>(head + kHeadSymExponent);
+    y.mmax_bits = reinterpret_cast<unsigned long long *>(head + kHeadSymMaxMass);
+    y.arrivals = reinterpret_cast<unsigned *>(head + kHeadSymArrivals);
+    y.cost = reinterpret_cast<uint32_t *>(c);
+    y.prefix = reinterpret_cast<unsigned long long *>(c + align_up(4 * (size_t)z.T, 256));
+    y.lo = reinterpret_cast<int64_t *>(c + align_up(4 * (size_t)z.T, 256) +
                                        align_up(8 * (size_t)(z.T + 1), 256));
     y.acc_fx = reinterpret_cast<unsigned long long *>(ws + L.sym_fx);
     return y;
@@ -772,7 +777,7 @@ int launch_step_sym(const ForceJob &j, double *vel, double dt, int64_t nsteps, b
     for (int64_t e = e0; e <= nsteps; ++e) {
         if (!opened)
             NB_TRY_SYM(launch_kick_drift_pack(const_cast<double *>(j.pos), vel, j.acc, j.mass, j.N,
-                                              j.L.Np, dt, nullptr, j.stream));
+                                              j.L.Np, dt, nullptr, nullptr, 0, j.stream));
         if (!packed) {
             const bool reuse = sorted_at >= 0 && e - sorted_at < kResortEvery;
             if (!reuse) sorted_at = e;

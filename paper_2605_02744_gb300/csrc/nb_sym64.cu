@@ -210,14 +210,18 @@ __global__ void __launch_bounds__(NTHR) sym64_kernel(const Params64 p) {
     if (bad) dev::set_status(p.status, kStatusNonFinite);
 }
 
-// The largest |m|, after an optional kick and drift (v += kick a; x += drift v).
+// The largest |m|, after an optional kick and drift (v += kick a; x += drift v),
+// and cleared totals.
 __global__ void __launch_bounds__(128) sym64_open_kernel(double *pos, double *vel,
                                                          const double *acc, const double *mass,
                                                          int64_t N, double kick, double drift,
-                                                         unsigned long long *mx) {
+                                                         unsigned long long *mx,
+                                                         unsigned long long *fx, int64_t Np,
+                                                         int nc) {
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     dev::grid_trigger();
     dev::grid_wait();
+    if (clear_totals(fx, N, N, Np, nc)) return;
     unsigned long long am = 0ull;  // non-negative doubles order like their bits
     if (i < N) {
         if (vel) {
@@ -258,7 +262,7 @@ __global__ void __launch_bounds__(128) sym64_fold_kernel(const Params64 p, doubl
     bool ok = true;
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-        const double a = G * take_fixed(t, c, i, F);
+        const double a = G * take_fixed<NEXT>(t, c, i, F);
         ok = ok && isfinite(a);
         if (!NEXT) acc[3 * i + c] = a;
         if (vel) {
@@ -271,7 +275,7 @@ __global__ void __launch_bounds__(128) sym64_fold_kernel(const Params64 p, doubl
         }
     }
     if (!NEXT && pot) {
-        const double gp = -G * take_fixed(t, 3, i, F);
+        const double gp = -G * take_fixed<false>(t, 3, i, F);
         pot[i] = gp;
         ok = ok && isfinite(gp);
     }
@@ -284,14 +288,14 @@ struct Run64 {
     unsigned long long *mx;
 
     explicit Run64(const ForceJob &job) : j(job) {
-        mx = reinterpret_cast<unsigned long long *>(j.ws + j.L.wsym_head + 192);
+        mx = reinterpret_cast<unsigned long long *>(j.ws + j.L.status + kHeadMaxMass64);
         p.pos = j.pos;
         p.mass = j.mass;
         p.N = j.N;
         p.Np = j.L.Np;
         p.eps2 = j.eps * j.eps;
         p.fx = reinterpret_cast<unsigned long long *>(j.ws + j.L.wsym_fx);
-        p.fxe = reinterpret_cast<int *>(j.ws + j.L.wsym_head + 64);
+        p.fxe = reinterpret_cast<int *>(j.ws + j.L.status + kHeadExponents);
         p.mx = mx;
         p.status = reinterpret_cast<uint32_t *>(j.ws + j.L.status);
         // as params_of in nb_wsym.cu
@@ -299,8 +303,10 @@ struct Run64 {
         p.nb = cdiv(j.N, BW);
     }
     int open(double *vel, double kick, double drift) {
-        return launch_pdl(sym64_open_kernel, (unsigned)cdiv(j.N, 128), 128, 0, j.stream,
-                          const_cast<double *>(j.pos), vel, j.acc, j.mass, j.N, kick, drift, mx);
+        const int nc = j.pot ? 4 : 3;
+        return launch_pdl(sym64_open_kernel, pack_blocks(j.N, j.N), 128, 0, j.stream,
+                          const_cast<double *>(j.pos), vel, j.acc, j.mass, j.N, kick, drift, mx, p.fx,
+                          p.Np, nc);
     }
     int pairs(bool pot) {
         auto kern = pot ? sym64_kernel<true> : sym64_kernel<false>;

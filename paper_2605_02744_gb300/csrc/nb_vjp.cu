@@ -675,17 +675,19 @@ struct VjpPh {
 };
 
 // Positions, masses and cotangents in one pass: launch_pack's and
-// pack_cotangent_kernel's arrays, with the largest |m|, |x|, |c| and |pbar|.
+// pack_cotangent_kernel's arrays, with the largest |m|, |x|, |c| and |pbar|,
+// and cleared totals.
 __global__ void __launch_bounds__(128) wsym_vjp_pack_kernel(
     const double *pos, const double *mass,
     const double *abar, const double *pbar, double *vbar,
     const double *xbar, double drift, double coef, int step_form, int64_t N,
-    int64_t Np, float *soa, float *csoa, unsigned *mx) {
+    int64_t Np, float *soa, float *csoa, unsigned *mx, unsigned long long *fx, int nc) {
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;  // < Np: whole blocks
     float hi[3] = {0.f, 0.f, 0.f}, lo[3] = {0.f, 0.f, 0.f}, cf[3] = {0.f, 0.f, 0.f};
     float m = 0.f, pb = 0.f, ac = 0.f, ax = 0.f;
     dev::grid_trigger();
     dev::grid_wait();
+    if (clear_totals(fx, Np, N, Np, nc)) return;
     if (i < N) {
 #pragma unroll
         for (int e = 0; e < 3; ++e) {
@@ -717,7 +719,7 @@ __global__ void __launch_bounds__(128) wsym_vjp_pack_kernel(
     warp_max(mx + kMaxP, fabsf(pb));
 }
 
-// The totals of every particle: read and zeroed, x G, stored or added;
+// The totals of every particle: read, x G, stored or added;
 // FUSED: the acceleration and the rewind, as vjp_epilogue.
 template <bool FUSED>
 __global__ void __launch_bounds__(128) wsym_vjp_fold_kernel(const Params p, const VjpParams q,
@@ -731,18 +733,18 @@ __global__ void __launch_bounds__(128) wsym_vjp_fold_kernel(const Params p, cons
     bool ok = true;
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-        const double g = q.G * take_fixed(p, c, i, Fx);
+        const double g = q.G * take_fixed<false>(p, c, i, Fx);
         q.pos_bar[3 * i + c] = q.accumulate ? q.pos_bar[3 * i + c] + g : g;
         ok = ok && isfinite(g);
     }
-    const double gm = -q.G * take_fixed(p, 3, i, Fm);
+    const double gm = -q.G * take_fixed<false>(p, 3, i, Fm);
     q.mass_bar[i] = q.accumulate ? q.mass_bar[i] + gm : gm;
     ok = ok && isfinite(gm);
     if (FUSED) {
         const int Fa = p.fxe[2];
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
-            const double a = q.G * take_fixed(p, 4 + c, i, Fa);
+            const double a = q.G * take_fixed<false>(p, 4 + c, i, Fa);
             q.acc_out[3 * i + c] = a;
             const double vh = q.vhalf[3 * i + c] - q.rewind_kick * a;
             q.vhalf[3 * i + c] = vh;
@@ -755,7 +757,7 @@ __global__ void __launch_bounds__(128) wsym_vjp_fold_kernel(const Params p, cons
 
 int launch_vjp_wsym(const VjpJob &j, bool pb, bool fused) {
     if (fused && pb) return fail(NB_ERR_UNSUPPORTED, "fused force with pot_bar is not built");
-    unsigned *mx = reinterpret_cast<unsigned *>(j.ws + j.L.wsym_head + 128);
+    unsigned *mx = reinterpret_cast<unsigned *>(j.ws + j.L.status + kHeadMaxima);
     float *soa = reinterpret_cast<float *>(j.ws + j.L.packA);
     float *csoa = reinterpret_cast<float *>(j.ws + j.L.packB);
     Params p{};
@@ -767,7 +769,7 @@ int launch_vjp_wsym(const VjpJob &j, bool pb, bool fused) {
     p.eps2 = ef * ef;
     p.keep = true;
     p.fx = reinterpret_cast<unsigned long long *>(j.ws + j.L.wsym_fx);
-    p.fxe = reinterpret_cast<int *>(j.ws + j.L.wsym_head + 64);
+    p.fxe = reinterpret_cast<int *>(j.ws + j.L.status + kHeadExponents);
     p.mx = mx;
     p.status = reinterpret_cast<uint32_t *>(j.ws + j.L.status);
     // a-priori bounds on every partial and total, with |w| <= 2 sqrt(3) max|m|
@@ -779,9 +781,11 @@ int launch_vjp_wsym(const VjpJob &j, bool pb, bool fused) {
     p.set_scale(2, n * 1.7320509 * e2);
     p.set_scale(3, n * e1);
     p.set_scale(4, n * e2);
-    int rc = launch_pdl(wsym_vjp_pack_kernel, (unsigned)(j.L.Np / 128), 128, 0, j.stream, j.pos,
+    const int nc = fused ? 7 : 4;
+    int rc = launch_pdl(wsym_vjp_pack_kernel, pack_blocks(j.L.Np, j.N), 128, 0, j.stream, j.pos,
                         j.mass, j.acc_bar, j.pot_bar, j.vel_bar, j.pos_bar, j.drift_dt,
-                        j.kick_coef, j.step_form ? 1 : 0, j.N, j.L.Np, soa, csoa, mx);
+                        j.kick_coef, j.step_form ? 1 : 0, j.N, j.L.Np, soa, csoa, mx, p.fx,
+                        nc);
     if (rc) return rc;
     if (fused)
         rc = j.split ? launch_pairs<VjpPh<false, true, true>>(p, j.stream)
@@ -841,7 +845,8 @@ int launch_vjp(const VjpJob &j) {
         return NB_OK;
     }
     float *soa = reinterpret_cast<float *>(j.ws + j.L.packA);
-    int rc = launch_pack(j.pos, j.mass, j.N, j.L.Np, soa, j.stream);
+    uint32_t *counters = reinterpret_cast<uint32_t *>(j.ws + j.L.counters);
+    int rc = launch_pack(j.pos, j.mass, j.N, j.L.Np, soa, counters, j.L.max_blocks, j.stream);
     if (rc) return rc;
     const Shape &sh = j.shape;
     VjpParams p;
@@ -868,7 +873,7 @@ int launch_vjp(const VjpJob &j) {
     p.rewind_kick = j.rewind_kick;
     p.rewind_drift = j.rewind_drift;
     p.records = reinterpret_cast<double *>(j.ws + j.L.records);
-    p.counters = reinterpret_cast<uint32_t *>(j.ws + j.L.counters);
+    p.counters = counters;
     p.status = status;
     p.timeout = j.timeout;
     p.unissued = j.unissued;

@@ -88,17 +88,20 @@ struct ForcePh {
 };
 
 // Pack of the positions and masses after an optional kick and drift
-// (v += kick a; x += drift v), and the largest |m| and |x|.
+// (v += kick a; x += drift v), the largest |m| and |x|, and cleared totals (nc
+// components).
 __global__ void __launch_bounds__(128) wsym_pack_kernel(double *pos,
                                                         double *vel,
                                                         const double *acc,
                                                         const double *mass, int64_t N,
                                                         int64_t Np, double kick, double drift,
-                                                        float *soa, unsigned *mx) {
+                                                        float *soa, unsigned *mx,
+                                                        unsigned long long *fx, int nc) {
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;  // < Np: whole blocks
     float hi[3] = {0.f, 0.f, 0.f}, lo[3] = {0.f, 0.f, 0.f}, m = 0.f, am = 0.f, ax = 0.f;
     dev::grid_trigger();
     dev::grid_wait();
+    if (clear_totals(fx, Np, N, Np, nc)) return;
     if (i < N) {
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
@@ -122,8 +125,8 @@ __global__ void __launch_bounds__(128) wsym_pack_kernel(double *pos,
     warp_max(mx + kMaxX, ax);
 }
 
-// The totals of every particle: read and zeroed, x G, stored, with an optional
-// closing kick; NEXT: also the next step's opening kick, drift and pack (its
+// The totals of every particle: read, x G, stored, with an optional
+// closing kick; NEXT: zeroed, also the next step's opening kick, drift and pack (its
 // masses are already packed), and no store of the acceleration, which the
 // next step's fold replaces before anything reads it.
 template <bool NEXT>
@@ -153,7 +156,7 @@ __global__ void __launch_bounds__(128) wsym_fold_kernel(const Params p, double G
     bool ok = true;
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-        a[c] = G * take_fixed(p, c, i, F);
+        a[c] = G * take_fixed<NEXT>(p, c, i, F);
         ok = ok && isfinite(a[c]);
         if (!NEXT) acc[3 * i + c] = a[c];
         if (vel) {
@@ -170,7 +173,7 @@ __global__ void __launch_bounds__(128) wsym_fold_kernel(const Params p, double G
         }
     }
     if (!NEXT && pot) {
-        const double gp = -G * take_fixed(p, 3, i, p.fxe[1]);
+        const double gp = -G * take_fixed<false>(p, 3, i, p.fxe[1]);
         pot[i] = gp;
         ok = ok && isfinite(gp);
     }
@@ -178,7 +181,7 @@ __global__ void __launch_bounds__(128) wsym_fold_kernel(const Params p, double G
 }
 
 unsigned *maxima(const ForceJob &j) {
-    return reinterpret_cast<unsigned *>(j.ws + j.L.wsym_head + 128);
+    return reinterpret_cast<unsigned *>(j.ws + j.L.status + kHeadMaxima);
 }
 
 Params params_of(const ForceJob &j) {
@@ -190,7 +193,7 @@ Params params_of(const ForceJob &j) {
     p.eps2 = ef * ef;
     p.keep = j.precision != NB_PREC_FP32;
     p.fx = reinterpret_cast<unsigned long long *>(j.ws + j.L.wsym_fx);
-    p.fxe = reinterpret_cast<int *>(j.ws + j.L.wsym_head + 64);
+    p.fxe = reinterpret_cast<int *>(j.ws + j.L.status + kHeadExponents);
     p.mx = maxima(j);
     p.status = reinterpret_cast<uint32_t *>(j.ws + j.L.status);
     // every partial and total: N max|m| times the largest |d| (|d|^2 +
@@ -226,9 +229,11 @@ int launch_pair_kernel(Params &p, bool split, bool pot, cudaStream_t st) {
 }
 
 int launch_wsym_pack(const ForceJob &j, double *vel, double kick, double drift) {
-    return launch_pdl(wsym_pack_kernel, (unsigned)(j.L.Np / 128), 128, 0, j.stream,
+    const int nc = j.pot ? 4 : 3;
+    return launch_pdl(wsym_pack_kernel, pack_blocks(j.L.Np, j.N), 128, 0, j.stream,
                       const_cast<double *>(j.pos), vel, j.acc, j.mass, j.N, j.L.Np, kick, drift,
-                      reinterpret_cast<float *>(j.ws + j.L.packA), maxima(j));
+                      reinterpret_cast<float *>(j.ws + j.L.packA), maxima(j),
+                      reinterpret_cast<unsigned long long *>(j.ws + j.L.wsym_fx), nc);
 }
 
 int launch_wsym_fold(const ForceJob &j, const Params &p, double *pot, bool next, double *vel,
