@@ -353,23 +353,22 @@ struct JerkPh {
             float2 dw = mul2(dx, wx);
             dw = fma2(dy, wy, dw);
             dw = fma2(dz, wz, dw);
-            const float2 r = f2(rsqrt_approx(r2.x), rsqrt_approx(r2.y));
+            float2 r = f2(rsqrt_approx(r2.x), rsqrt_approx(r2.y));
+            if (SELF) r = mask_self<IPAIR>(r, k, self_h);
             const float2 rr = mul2(r, r);
             const float2 r3 = mul2(rr, r);
             const float2 q = mul2(mul2(rr, f2(-3.f, -3.f)), dw);
             const float2 ex = fma2(q, dx, wx);
             const float2 ey = fma2(q, dy, wy);
             const float2 ez = fma2(q, dz, wz);
-            float2 mj = J[3];
-            if (SELF) mj = mask_self<IPAIR>(mj, k, self_h);
-            const float2 sj = mul2(mj, r3);
+            const float2 sj = mul2(J[3], r3);
             s.a[k][0] = fma2(sj, dx, s.a[k][0]);
             s.a[k][1] = fma2(sj, dy, s.a[k][1]);
             s.a[k][2] = fma2(sj, dz, s.a[k][2]);
             s.a[k][3] = fma2(sj, ex, s.a[k][3]);
             s.a[k][4] = fma2(sj, ey, s.a[k][4]);
             s.a[k][5] = fma2(sj, ez, s.a[k][5]);
-            if constexpr (POT) s.a[k][6] = fma2(mj, r, s.a[k][6]);
+            if constexpr (POT) s.a[k][6] = fma2(J[3], r, s.a[k][6]);
             if (SYM) {
                 const float2 si = mul2(s.m[k], r3);
                 T[0] = k ? fma2(si, dx, T[0]) : mul2(si, dx);
@@ -414,6 +413,8 @@ __global__ void __launch_bounds__(128) wsym_predict_pack_kernel(
         const double md = mass[i];
         m = __double2float_rn(md);
         am = fabsf(m);
+    } else {
+        hi[0] = kPadX;
     }
     store_packed(soa, Np, i, hi, lo, m);
 #pragma unroll
@@ -468,7 +469,7 @@ int launch_jerk_wsym(const JerkJob &j, JerkParams q) {
     p.soa = q.soa;
     p.Np = j.L.Np;
     p.N = j.N;
-    p.eps2 = q.eps2;
+    p.eps = (float)j.eps;
     p.keep = j.precision != NB_PREC_FP32;
     p.fx = reinterpret_cast<unsigned long long *>(j.ws + j.L.wsym_fx);
     p.fxe = reinterpret_cast<int *>(j.ws + j.L.status + kHeadExponents);

@@ -708,6 +708,8 @@ __global__ void __launch_bounds__(128) wsym_vjp_pack_kernel(
         }
         m = __double2float_rn(mass[i]);
         if (!step_form && pbar) pb = __double2float_rn(coef * pbar[i]);
+    } else {
+        hi[0] = kPadX;
     }
     store_packed(soa, Np, i, hi, lo, m);
 #pragma unroll
@@ -765,8 +767,7 @@ int launch_vjp_wsym(const VjpJob &j, bool pb, bool fused) {
     p.csoa = csoa;
     p.Np = j.L.Np;
     p.N = j.N;
-    const float ef = (float)j.eps;
-    p.eps2 = ef * ef;
+    p.eps = (float)j.eps;
     p.keep = true;
     p.fx = reinterpret_cast<unsigned long long *>(j.ws + j.L.wsym_fx);
     p.fxe = reinterpret_cast<int *>(j.ws + j.L.status + kHeadExponents);

@@ -67,15 +67,14 @@ struct ForcePh {
             float2 r2 = fma2(dx, dx, e2);
             r2 = fma2(dy, dy, r2);
             r2 = fma2(dz, dz, r2);
-            const float2 r = f2(rsqrt_approx(r2.x), rsqrt_approx(r2.y));
+            float2 r = f2(rsqrt_approx(r2.x), rsqrt_approx(r2.y));
+            if (SELF) r = mask_self<IPAIR>(r, k, self_h);
             const float2 r3 = mul2(mul2(r, r), r);
-            float2 mj = J[3];
-            if (SELF) mj = mask_self<IPAIR>(mj, k, self_h);
-            const float2 sj = mul2(mj, r3);
+            const float2 sj = mul2(J[3], r3);
             s.a[k][0] = fma2(sj, dx, s.a[k][0]);
             s.a[k][1] = fma2(sj, dy, s.a[k][1]);
             s.a[k][2] = fma2(sj, dz, s.a[k][2]);
-            if constexpr (POT) s.a[k][3] = fma2(mj, r, s.a[k][3]);
+            if constexpr (POT) s.a[k][3] = fma2(J[3], r, s.a[k][3]);
             if (SYM) {
                 const float2 si = mul2(s.m[k], r3);
                 T[0] = k ? fma2(si, dx, T[0]) : mul2(si, dx);
@@ -119,6 +118,8 @@ __global__ void __launch_bounds__(128) wsym_pack_kernel(double *pos,
         m = __double2float_rn(md);
         am = __double2float_ru(fabs(md));
         ax = fmaxf(fabsf(hi[0]), fmaxf(fabsf(hi[1]), fabsf(hi[2])));
+    } else {
+        hi[0] = kPadX;
     }
     store_packed(soa, Np, i, hi, lo, m);
     warp_max(mx + kMaxM, am);
@@ -189,8 +190,7 @@ Params params_of(const ForceJob &j) {
     p.soa = reinterpret_cast<const float *>(j.ws + j.L.packA);
     p.Np = j.L.Np;
     p.N = j.N;
-    const float ef = (float)j.eps;
-    p.eps2 = ef * ef;
+    p.eps = (float)j.eps;
     p.keep = j.precision != NB_PREC_FP32;
     p.fx = reinterpret_cast<unsigned long long *>(j.ws + j.L.wsym_fx);
     p.fxe = reinterpret_cast<int *>(j.ws + j.L.status + kHeadExponents);

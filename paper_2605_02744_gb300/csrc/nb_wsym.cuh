@@ -78,7 +78,7 @@ struct Params {
     int64_t N;
     int64_t nb;          // blocks
     int64_t per_warp, extra;  // scheduling units per warp; the first `extra` warps take one more
-    float eps2;
+    float eps;
     bool keep;           // compensated i-side sums (every policy but FP32)
     unsigned long long *fx;  // [components][4 limbs][Np] fixed-point totals
     int *fxe;                // [kMaxGroups] the call's exponents (written here)
@@ -101,6 +101,29 @@ enum MaxWord { kMaxM = 0, kMaxV = 1, kMaxX = 2, kMaxC = 3, kMaxP = 4 };
 struct Scales {
     int x, m, c;
 };
+// The exponent of the unit of length, from those of max|x| and eps (v < 2^e):
+// max|x| itself, unless eps is so much smaller that eps^-3 would leave FP32
+// (one escaper at 10^6 with eps = 1e-8: the unit follows eps, whose inverse
+// cube stays below 2^111, with room for a jerk's velocity) or larger (x^-3 is
+// then eps^-3, and the accelerations, d / eps^3, must not underflow).  At most
+// 2^6 below max|x| all the same: the smallest pair terms, of the system's
+// size, stay 2^29 above the grid (a VJP's or jerk's, which fall with its cube;
+// kMaxBound), and an eps 2^42 below max|x| is beyond the 48 bits of the
+// positions anyway.
+constexpr int kSmallEps = 36, kUnitBelow = 6;
+__host__ __device__ constexpr int length_exponent(int ex, int ee) {
+    int z = ex < ee + kSmallEps ? ex : ee + kSmallEps;
+    z = z > ex - kUnitBelow ? z : ex - kUnitBelow;
+    z = z > ee ? z : ee;
+    return z < -60 ? -60 : (z > 60 ? 60 : z);
+}
+// Exponent of the scaled bounds at most: no finite FP32 partial is larger, and
+// 2^19 of them fit the limbs.
+constexpr int kMaxBound = 127;
+// Where the packs put padding slots along x: their pairs must be finite (at the
+// origin, zero mass times r^-3 at a particle on the same spot was a NaN), which
+// they are between 2^-4 and 2^116 units of length.
+constexpr float kPadX = 72057594037927936.f;  // 2^56
 // Exponents of the maxima (v < 2^e; fx::kNoBound: not finite), for the bounds:
 // integers, because a few dependent FP64 operations at the start of every
 // kernel cost microseconds on this part.
@@ -114,6 +137,10 @@ enum Factor { kFx = 0, kFm = 1, kFc = 2, kFp = 3, kFone = 4 };  // 2^-x 2^-m 2^-
 __device__ __forceinline__ int exponent_of(unsigned bits) {
     const int f = (int)(bits >> 23);
     return f == 0 || f == 0xff ? 0 : min(max(f - 126, -60), 60);
+}
+__device__ __forceinline__ int exponent_or(unsigned bits, int other) {
+    const int f = (int)(bits >> 23);
+    return f == 0 || f == 0xff ? other : f - 126;
 }
 __device__ __forceinline__ int bound_exponent(unsigned bits) {
     const int f = (int)(bits >> 23);
@@ -173,7 +200,8 @@ struct Geo {
 };
 
 // Zeroes the halves of v that pair a particle with itself: rotation step 0 of
-// the diagonal block's j-set h.
+// the diagonal block's j-set h.  What is zeroed is r^-1, so that nothing
+// infinite meets a zero.
 template <bool IPAIR>
 __device__ __forceinline__ float2 mask_self(float2 v, int k, int h) {
     v.x = (IPAIR ? h == 2 * k : k == 2 * h) ? 0.f : v.x;
@@ -284,14 +312,16 @@ __global__ void __launch_bounds__(Geo<PH>::NTHR, 1) wsym_kernel(const Params p) 
                        bv = __ldcg(p.mx + kMaxV), bc = __ldcg(p.mx + kMaxC),
                        bp = __ldcg(p.mx + kMaxP);
         Scales z;
-        z.x = exponent_of(bx);
+        const int ee = exponent_or(__float_as_uint(p.eps), 60);
+        z.x = length_exponent(exponent_or(bx, ee), ee);
         z.m = exponent_of(bm);
         z.c = min(max(exponent_of(bc), exponent_of(bp) + z.x), 60);
         const Maxima mm = {bound_exponent(bm), bound_exponent(bv), bound_exponent(bc),
                            bound_exponent(bp)};
         if (l < PH::GROUPS) {
             const int up = PH::shift(z, l);
-            const int Fg = fx::limb_exponent(PH::bound(p, mm, l) - up);
+            const int b = PH::bound(p, mm, l) - up;
+            const int Fg = fx::limb_exponent(b >= fx::kNoBound / 2 ? b : min(b, kMaxBound));
             sF[l] = Fg;
             // value = 2^up (scaled value)
             if (blockIdx.x == 0) p.fxe[l] = Fg == fx::kNoGrid ? Fg : Fg - up;
@@ -305,7 +335,7 @@ __global__ void __launch_bounds__(Geo<PH>::NTHR, 1) wsym_kernel(const Params p) 
     }
     __syncthreads();
     // eps^2 in scaled lengths (at least the smallest normal float)
-    const float es = fmaxf(p.eps2 * sFac[kFx] * sFac[kFx], 1.17549435e-38f);
+    const float eu = p.eps * sFac[kFx], es = fmaxf(eu * eu, 1.17549435e-38f);
     const float2 e2 = f2(es, es);
     int F[PH::GROUPS];
 #pragma unroll
