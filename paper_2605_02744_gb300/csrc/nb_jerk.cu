@@ -424,7 +424,7 @@ __global__ void __launch_bounds__(128) wsym_predict_pack_kernel(
     warp_max(mx + kMaxX, ax);
 }
 
-// The totals of every particle: read, x G, then stored (h = 0) or
+// The totals of every particle: read and zeroed, x G, then stored (h = 0) or
 // taken through the Hermite corrector, as jerk_kernel's epilogue.
 template <bool POT>
 __global__ void __launch_bounds__(128) wsym_jerk_fold_kernel(const Params p, const JerkParams q,
@@ -439,8 +439,8 @@ __global__ void __launch_bounds__(128) wsym_jerk_fold_kernel(const Params p, con
     bool ok = true;
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-        const double a1 = q.G * take_fixed<false>(p, c, i, Fa);
-        const double j1 = q.G * take_fixed<false>(p, 3 + c, i, Fj);
+        const double a1 = q.G * take_fixed(p, c, i, Fa);
+        const double j1 = q.G * take_fixed(p, 3 + c, i, Fj);
         if (h != 0.0) {
             const double x0 = q.pos[3 * i + c], v0 = q.vel[3 * i + c];
             const double a0 = q.acc[3 * i + c], j0 = q.jerk[3 * i + c];
@@ -452,7 +452,7 @@ __global__ void __launch_bounds__(128) wsym_jerk_fold_kernel(const Params p, con
         q.jerk[3 * i + c] = j1;
         ok = ok && isfinite(a1) && isfinite(j1);
     }
-    if (POT) q.pot[i] = -q.G * take_fixed<false>(p, 6, i, p.fxe[2]);
+    if (POT) q.pot[i] = -q.G * take_fixed(p, 6, i, p.fxe[2]);
     if (!ok) dev::set_status(p.status, kStatusNonFinite);
 }
 
@@ -485,7 +485,7 @@ int launch_jerk_wsym(const JerkJob &j, JerkParams q) {
     const int nc = q.pot ? 7 : 6;
     for (int64_t n = 0; n < (j.nsteps > 0 ? j.nsteps : 1); ++n) {
         q.h = j.nsteps > 0 ? j.h : 0.0;
-        int rc = launch_pdl(wsym_predict_pack_kernel, pack_blocks(j.L.Np, j.N), 128, 0, j.stream,
+        int rc = launch_pdl(wsym_predict_pack_kernel, pack_blocks(j.L.Np, j.N, nc), 128, 0, j.stream,
                             j.pos, j.vel, j.acc, j.jerk, j.mass, j.N, j.L.Np, q.h,
                             reinterpret_cast<float *>(j.ws + j.L.packA), mx, p.fx,
                             nc);

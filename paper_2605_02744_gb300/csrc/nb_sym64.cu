@@ -262,7 +262,7 @@ __global__ void __launch_bounds__(128) sym64_fold_kernel(const Params64 p, doubl
     bool ok = true;
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-        const double a = G * take_fixed<NEXT>(t, c, i, F);
+        const double a = G * take_fixed(t, c, i, F);
         ok = ok && isfinite(a);
         if (!NEXT) acc[3 * i + c] = a;
         if (vel) {
@@ -275,7 +275,7 @@ __global__ void __launch_bounds__(128) sym64_fold_kernel(const Params64 p, doubl
         }
     }
     if (!NEXT && pot) {
-        const double gp = -G * take_fixed<false>(t, 3, i, F);
+        const double gp = -G * take_fixed(t, 3, i, F);
         pot[i] = gp;
         ok = ok && isfinite(gp);
     }
@@ -304,7 +304,7 @@ struct Run64 {
     }
     int open(double *vel, double kick, double drift) {
         const int nc = j.pot ? 4 : 3;
-        return launch_pdl(sym64_open_kernel, pack_blocks(j.N, j.N), 128, 0, j.stream,
+        return launch_pdl(sym64_open_kernel, pack_blocks(j.N, j.N, nc), 128, 0, j.stream,
                           const_cast<double *>(j.pos), vel, j.acc, j.mass, j.N, kick, drift, mx, p.fx,
                           p.Np, nc);
     }

@@ -721,7 +721,7 @@ __global__ void __launch_bounds__(128) wsym_vjp_pack_kernel(
     warp_max(mx + kMaxP, fabsf(pb));
 }
 
-// The totals of every particle: read, x G, stored or added;
+// The totals of every particle: read and zeroed, x G, stored or added;
 // FUSED: the acceleration and the rewind, as vjp_epilogue.
 template <bool FUSED>
 __global__ void __launch_bounds__(128) wsym_vjp_fold_kernel(const Params p, const VjpParams q,
@@ -735,18 +735,18 @@ __global__ void __launch_bounds__(128) wsym_vjp_fold_kernel(const Params p, cons
     bool ok = true;
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-        const double g = q.G * take_fixed<false>(p, c, i, Fx);
+        const double g = q.G * take_fixed(p, c, i, Fx);
         q.pos_bar[3 * i + c] = q.accumulate ? q.pos_bar[3 * i + c] + g : g;
         ok = ok && isfinite(g);
     }
-    const double gm = -q.G * take_fixed<false>(p, 3, i, Fm);
+    const double gm = -q.G * take_fixed(p, 3, i, Fm);
     q.mass_bar[i] = q.accumulate ? q.mass_bar[i] + gm : gm;
     ok = ok && isfinite(gm);
     if (FUSED) {
         const int Fa = p.fxe[2];
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
-            const double a = q.G * take_fixed<false>(p, 4 + c, i, Fa);
+            const double a = q.G * take_fixed(p, 4 + c, i, Fa);
             q.acc_out[3 * i + c] = a;
             const double vh = q.vhalf[3 * i + c] - q.rewind_kick * a;
             q.vhalf[3 * i + c] = vh;
@@ -783,7 +783,7 @@ int launch_vjp_wsym(const VjpJob &j, bool pb, bool fused) {
     p.set_scale(3, n * e1);
     p.set_scale(4, n * e2);
     const int nc = fused ? 7 : 4;
-    int rc = launch_pdl(wsym_vjp_pack_kernel, pack_blocks(j.L.Np, j.N), 128, 0, j.stream, j.pos,
+    int rc = launch_pdl(wsym_vjp_pack_kernel, pack_blocks(j.L.Np, j.N, nc), 128, 0, j.stream, j.pos,
                         j.mass, j.acc_bar, j.pot_bar, j.vel_bar, j.pos_bar, j.drift_dt,
                         j.kick_coef, j.step_form ? 1 : 0, j.N, j.L.Np, soa, csoa, mx, p.fx,
                         nc);

@@ -126,8 +126,8 @@ __global__ void __launch_bounds__(128) wsym_pack_kernel(double *pos,
     warp_max(mx + kMaxX, ax);
 }
 
-// The totals of every particle: read, x G, stored, with an optional
-// closing kick; NEXT: zeroed, also the next step's opening kick, drift and pack (its
+// The totals of every particle: read and zeroed, x G, stored, with an optional
+// closing kick; NEXT: also the next step's opening kick, drift and pack (its
 // masses are already packed), and no store of the acceleration, which the
 // next step's fold replaces before anything reads it.
 template <bool NEXT>
@@ -157,7 +157,7 @@ __global__ void __launch_bounds__(128) wsym_fold_kernel(const Params p, double G
     bool ok = true;
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-        a[c] = G * take_fixed<NEXT>(p, c, i, F);
+        a[c] = G * take_fixed(p, c, i, F);
         ok = ok && isfinite(a[c]);
         if (!NEXT) acc[3 * i + c] = a[c];
         if (vel) {
@@ -174,7 +174,7 @@ __global__ void __launch_bounds__(128) wsym_fold_kernel(const Params p, double G
         }
     }
     if (!NEXT && pot) {
-        const double gp = -G * take_fixed<false>(p, 3, i, p.fxe[1]);
+        const double gp = -G * take_fixed(p, 3, i, p.fxe[1]);
         pot[i] = gp;
         ok = ok && isfinite(gp);
     }
@@ -230,7 +230,7 @@ int launch_pair_kernel(Params &p, bool split, bool pot, cudaStream_t st) {
 
 int launch_wsym_pack(const ForceJob &j, double *vel, double kick, double drift) {
     const int nc = j.pot ? 4 : 3;
-    return launch_pdl(wsym_pack_kernel, pack_blocks(j.L.Np, j.N), 128, 0, j.stream,
+    return launch_pdl(wsym_pack_kernel, pack_blocks(j.L.Np, j.N, nc), 128, 0, j.stream,
                       const_cast<double *>(j.pos), vel, j.acc, j.mass, j.N, j.L.Np, kick, drift,
                       reinterpret_cast<float *>(j.ws + j.L.packA), maxima(j),
                       reinterpret_cast<unsigned long long *>(j.ws + j.L.wsym_fx), nc);

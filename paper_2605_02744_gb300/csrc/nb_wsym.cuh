@@ -467,41 +467,44 @@ __global__ void __launch_bounds__(Geo<PH>::NTHR, 1) wsym_kernel(const Params p) 
     if (bad) dev::set_status(p.status, kStatusNonFinite);
 }
 
-// The pack of every call clears its totals (the workspace may have served
-// another size), with blocks of 128 threads beyond the ones that pack the slots,
-// two slots a thread (acceleration + jerk of 1024 particles: 18.8 us on totals
-// known to be zero, 19.8 us so, 20.4 us with the 24 words of a particle stored
-// by the thread that packs it).
-inline unsigned pack_blocks(int64_t slots, int64_t N) {
-    return (unsigned)(cdiv(slots, 128) + cdiv(N, 256));
+// The fold leaves the totals that it reads at zero, but the workspace may have
+// served another size or kernel since: the pack of every call makes sure, with
+// blocks of 128 threads beyond the ones that pack the slots, a component of two
+// slots per thread.  They read first: stores that have to be out before the
+// pair kernel cost more than the loads, which the pack's own hide (acceleration
+// + jerk of 1024 particles: 18.8 us with totals known to be zero and so, 20.4
+// us when the packing threads stored the 24 words of a particle).
+inline unsigned pack_blocks(int64_t slots, int64_t N, int nc) {
+    return (unsigned)(cdiv(slots, 128) + nc * cdiv(N, 256));
 }
-// True for the clearing blocks, after their stores.
+// True for the clearing blocks, after their work.
 __device__ __forceinline__ bool clear_totals(unsigned long long *fx, int64_t slots, int64_t N,
                                              int64_t Np, int nc) {
-    const int64_t b = (int64_t)blockIdx.x - (slots + 127) / 128;
+    const int b = (int)(blockIdx.x - (unsigned)((slots + 127) / 128));
     if (b < 0) return false;
-    const int64_t s = 2 * (b * 128 + threadIdx.x);  // Np is even
+    const int64_t s = 2 * ((int64_t)(b / nc) * 128 + threadIdx.x);  // Np is even
     if (s < N) {
-#pragma unroll 4
-        for (int w = 0; w < fx::kLimbs * nc; ++w)
-            *reinterpret_cast<ulonglong2 *>(fx + w * Np + s) = make_ulonglong2(0ull, 0ull);
+        unsigned long long *q = fx + (int64_t)(b % nc) * fx::kLimbs * Np + s;
+        ulonglong2 v[fx::kLimbs];
+#pragma unroll
+        for (int k = 0; k < fx::kLimbs; ++k) v[k] = *reinterpret_cast<const ulonglong2 *>(q + k * Np);
+#pragma unroll
+        for (int k = 0; k < fx::kLimbs; ++k)
+            if (v[k].x | v[k].y)
+                *reinterpret_cast<ulonglong2 *>(q + k * Np) = make_ulonglong2(0ull, 0ull);
     }
     return true;
 }
 
-// The value of component e of slot s; CLEAR: zeroes it for the loop's next
-// evaluation.
-template <bool CLEAR>
+// Reads and zeroes component e of slot s; its value.
 __device__ __forceinline__ double take_fixed(const Params &p, int e, int64_t s, int F) {
     unsigned long long *wd = p.fx + (int64_t)(fx::kLimbs * e) * p.Np + s;
     long long w[fx::kLimbs];
 #pragma unroll
     for (int q = 0; q < fx::kLimbs; ++q) w[q] = (long long)__ldcs(wd + q * p.Np);
-    if (CLEAR) {
 #pragma unroll
-        for (int q = 0; q < fx::kLimbs; ++q)
-            if (w[q]) wd[q * p.Np] = 0ull;
-    }
+    for (int q = 0; q < fx::kLimbs; ++q)
+        if (w[q]) wd[q * p.Np] = 0ull;
     return fx::limb_value(w, F);
 }
 
