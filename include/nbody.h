@@ -103,17 +103,24 @@ typedef enum {
  * N max|m| max(0.385 / eps^2, 1 / eps) on every acceleration component and
  * potential; it is finer than FP64 rounding unless that bound exceeds the
  * smallest |a_i| by more than ~10^14.  DEFAULT takes, for eps > 0, SYMMETRIC
- * for 24576 <= N <= 2^24 (FP32 and FP64 pairs) and, FP32 pairs only, from
+ * for 24576 <= N <= 2^24 with FP32 pairs (below eps = 1e-8 without
+ * ADAPTIVE positions, for the grid's sake) and, FP32 pairs only, from
  * N = 4800 unless a launch shape (nb_tune), NB_POS_ADAPTIVE or the
  * test_unissued_stage hook asks for the direct kernel; below that, under the
  * same conditions, a small-system kernel that evaluates every ordered pair;
+ * for FP64 pairs, SYMMETRIC for 64 <= N <= 2^24 and eps >= 1e-14;
  * DIRECT otherwise.  nb_forces_vjp, the step adjoints and nb_forces_jerk /
- * nb_hermite4 take symmetric pairs (same combining, same bounds times the
- * largest cotangent or velocity) for 256 <= N <= 2^24, eps > 0 and FP32
+ * nb_hermite4 take symmetric pairs (same combining)
+ * for 256 <= N <= 2^24, eps > 0 and FP32
  * pairs unless pairs is DIRECT or a launch shape or the hook is set.  Where
  * every pair takes the same displacement form (the VJP, the jerk, forces
  * below 32768 / 65536 particles), the totals have 174 instead of 100 bits:
- * 224 B per particle of every single-system workspace up to 2^24.
+ * 224 B per particle of every single-system workspace up to 2^24.  Their
+ * bounds are N max|m| times 0.385 / eps^2 (accelerations), 1 / eps
+ * (potential) or 4 max|c or v| / eps^3 (VJP, jerk, from the cotangents or
+ * velocities), N max|c| 0.67 / eps^2 for mass_bar; with FP32 pairs the grid
+ * is also at most 2^-32 of max|m| (max|c or v|) / max|x|^2 (^3), however
+ * small eps is.
  * For batches (B > 1, nb_forces_batched and
  * nb_step with offsets) DEFAULT and SYMMETRIC take the symmetric batched
  * path (warp-granular work items; workspace about 250 B per particle plus

@@ -304,10 +304,11 @@ bool positions_split(const nb_opts *o) {
 constexpr int64_t kAdaptiveMinN = 1 << 16;
 constexpr int64_t kAdaptiveMinNStepping = 1 << 15;
 
-bool positions_adaptive(const nb_opts *o, int64_t N, bool stepping) {
+bool positions_adaptive(const nb_opts *o, int64_t N, double eps, bool stepping) {
     if (o->precision == NB_PREC_FP64) return false;
     if (o->positions == NB_POS_ADAPTIVE) return true;
     if (o->positions != NB_POS_DEFAULT) return false;
+    if (eps > 0.0 && eps < kSymMinEps && sym_wanted(o, N, 1)) return false;
     return o->precision != NB_PREC_FP32 &&
            N >= (stepping ? kAdaptiveMinNStepping : kAdaptiveMinN);
 }
@@ -379,7 +380,7 @@ static int make_force_job(ForceJob *j, const double *pos, const double *mass, in
     j->kick = 0.0;
     j->precision = o->precision;
     j->split = positions_split(o);
-    j->adaptive = positions_adaptive(o, N);
+    j->adaptive = positions_adaptive(o, N, eps);
     j->reuse_order = false;
     j->gamma = o->near_gamma > 0.f ? o->near_gamma : kNearFarGamma;
     j->packed_ready = false;
@@ -387,7 +388,10 @@ static int make_force_job(ForceJob *j, const double *pos, const double *mass, in
     // an explicit NB_PAIRS_SYMMETRIC with eps = 0 is refused by the launcher
     j->sym = sym_wanted(o, N, 1) && (eps > 0.0 || o->pairs == NB_PAIRS_SYMMETRIC);
     if (o->precision == NB_PREC_FP64 && o->pairs == NB_PAIRS_DEFAULT)
-        j->sym = eps > 0.0 && N >= kSym64MinN && N <= kSymMaxN;
+        j->sym = eps >= kSym64MinEps && N >= kSym64MinN && N <= kSymMaxN;
+    // asked for by name, the adaptive displacement stays, with direct pairs
+    if (o->positions == NB_POS_ADAPTIVE && o->pairs == NB_PAIRS_DEFAULT && eps < kSymMinEps)
+        j->sym = false;
     j->row = !j->sym && eps > 0.0 && o->precision != NB_PREC_FP64 &&
              o->pairs == NB_PAIRS_DEFAULT && !shape_asked(o) &&
              o->positions != NB_POS_ADAPTIVE && o->test_unissued_stage == 0 && row_fits(N);
@@ -769,7 +773,7 @@ static int step_batched_direct(nb_state *s, double dt, int64_t nsteps, const nb_
 static int step_single_direct(nb_state *s, double dt, int64_t nsteps, const nb_opts *o) {
     ForceJob j;
     NB_TRY(make_force_job(&j, s->pos, s->mass, s->N, s->eps, s->acc, s->pot, s->ws, s->ws_bytes, o));
-    j.adaptive = positions_adaptive(o, s->N, nsteps > 0);
+    j.adaptive = positions_adaptive(o, s->N, s->eps, nsteps > 0);
     if (takes_sym64(j)) {
         if (nsteps == 0 && s->acc_valid) return NB_OK;
         return launch_step_sym64(j, s->vel, dt, nsteps, s->acc_valid != 0);

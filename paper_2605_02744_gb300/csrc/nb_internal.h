@@ -171,8 +171,9 @@ bool positions_split(const nb_opts *opts);
 // true when the split displacement is applied only to near tile pairs of a
 // Hilbert-sorted pack (explicit NB_POS_ADAPTIVE, or the default for the
 // KAHAN and F64ACC policies from N >= 2^16 for one evaluation and from
-// N >= 2^15 for a step loop; 1/64 is the default near_gamma).
-bool positions_adaptive(const nb_opts *opts, int64_t N, bool stepping = false);
+// N >= 2^15 for a step loop, unless pairs are symmetric and eps is below
+// kSymMinEps; 1/64 is the default near_gamma).
+bool positions_adaptive(const nb_opts *opts, int64_t N, double eps, bool stepping = false);
 // Steps of one nb_step call between full re-sorts of the adaptive path.
 constexpr int64_t kResortEvery = 16;
 
@@ -258,6 +259,18 @@ constexpr int64_t kWsymJerkMinN = 256;
 // 36 at 1024).
 constexpr int64_t kSym64MinN = 64;
 constexpr int kWsymComponents = 7;  // sums per particle at most
+// Smallest softenings by default of the symmetric paths whose totals' grid is a
+// fixed share of a bound that grows with eps^-2, where the direct kernels keep
+// 2^-24 (FP64 2^-53) of any term; in terms of max|m| / max|x|^2, for max|x| = 1:
+//  - the adaptive path, 2^-100 of the bound: 2^-24 at 1e-8 and 2^24 particles
+//    (of each particle's sum of as many terms still 2^-48), but 2^29 at 1e-16.
+//    Below it the hi/lo displacement for every pair, i.e. the warp-granular
+//    path, whose grid does not follow eps beyond what FP32 resolves
+//    (wsym::length_exponent);
+//  - FP64 pairs, 2^-174 of it: 2^-68 at 1e-14 and 16384 particles (2^24:
+//    2^-58), but 2^-48 at 1e-17.  Below it direct pairs.
+constexpr double kSymMinEps = 1e-8;
+constexpr double kSym64MinEps = 1e-14;
 // Largest system of the warp-granular path (its accumulators take 2^19 adds,
 // one per block of 128 slots and range end); an explicit request for
 // symmetric pairs without the adaptive displacement goes direct above it.

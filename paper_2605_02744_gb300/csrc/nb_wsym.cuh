@@ -106,11 +106,11 @@ struct Scales {
 // (one escaper at 10^6 with eps = 1e-8: the unit follows eps, whose inverse
 // cube stays below 2^111, with room for a jerk's velocity) or larger (x^-3 is
 // then eps^-3, and the accelerations, d / eps^3, must not underflow).  At most
-// 2^6 below max|x| all the same: the smallest pair terms, of the system's
-// size, stay 2^29 above the grid (a VJP's or jerk's, which fall with its cube;
-// kMaxBound), and an eps 2^42 below max|x| is beyond the 48 bits of the
-// positions anyway.
-constexpr int kSmallEps = 36, kUnitBelow = 6;
+// 2^5 below max|x| all the same: the smallest pair terms, of the system's
+// size, stay 2^32 above the grid (a VJP's or jerk's, which fall with its cube;
+// kMaxBound), and an eps 2^47 below max|x|, where eps^-3 is infinite again, is
+// at the 48 bits of the positions.
+constexpr int kSmallEps = 36, kUnitBelow = 5;
 __host__ __device__ constexpr int length_exponent(int ex, int ee) {
     int z = ex < ee + kSmallEps ? ex : ee + kSmallEps;
     z = z > ex - kUnitBelow ? z : ex - kUnitBelow;

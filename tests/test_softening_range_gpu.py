@@ -83,3 +83,66 @@ def test_two_particles_on_one_spot(n):
 def test_units_of_length(n, size, eps):
     s = ics.plummer_lognormal(n, seed=n)
     check(size * s.pos, s.vel, s.mass, eps)
+
+
+@pytest.mark.parametrize("n", [300, 5001, 12001])
+@pytest.mark.parametrize("eps", [1e-8, 0.999e-8, 1e-12, 1e-16, 1.2e-19])
+def test_tiny_softening(n, eps):
+    """The totals' bounds grow with eps^-2 and eps^-3; their grid must not."""
+    s = ics.plummer_lognormal(n, seed=n)
+    check(s.pos, s.vel, s.mass, eps)
+
+
+@pytest.mark.parametrize("n", [300, 5001])
+@pytest.mark.parametrize("eps", [1e-8, 0.999e-8, 1e-14, 0.999e-14, 1e-16, 1.2e-19])
+def test_fp64_pairs_at_tiny_softening(n, eps):
+    """Symmetric from 1e-14, direct below."""
+    s = ics.plummer_lognormal(n, seed=n)
+    ra, rp = oracle.forces(s.pos, s.mass, eps, 1.0)
+    o = binding.make_opts("fp64")
+    ws = binding.workspace(n, 1, o)
+    x, m = dev(s.pos), dev(s.mass)
+    acc, pot = torch.empty_like(x), torch.empty_like(m)
+    binding.nb_forces(x, m, eps, acc, pot, ws, o)
+    assert binding.nb_poll_status(ws, o) == binding.NB_OK
+    assert rel_vec_err(host(acc), ra).max() <= 1e-12 and rel_err(host(pot), rp).max() <= 1e-12
+
+
+def test_fp64_symmetric_pair_terms_over_magnitudes():
+    """test_sym64_gpu's pair terms on the symmetric kernel, asked for by name:
+    the reciprocal root over 69 decades."""
+    n, eps = 200, 1e-10
+    d = np.concatenate([[0.0], np.logspace(-9, 60, n - 1) * np.linspace(1.0, 1.9, n - 1)])
+    pos = np.zeros((n, 3))
+    pos[:, 0] = d
+    mass = np.full(n, 1e-300)
+    mass[0] = 1.0
+    o = binding.make_opts("fp64", pairs="symmetric")
+    ws = binding.workspace(n, 1, o)
+    x, m = dev(pos), dev(mass)
+    acc, pot = torch.empty_like(x), torch.empty_like(m)
+    binding.nb_forces(x, m, eps, acc, pot, ws, o)
+    dl = d[1:].astype(np.longdouble)
+    r2 = dl * dl + np.longdouble(eps) ** 2
+    ref = -dl / (r2 * np.sqrt(r2))
+    big = np.abs(ref) > 2.0 ** -120 * 1.02 * n * 0.385 / eps ** 2
+    assert np.abs(host(acc)[1:, 0][big] / ref[big] - 1).max() <= 2e-15
+    assert np.abs(host(pot)[1:] * np.sqrt(r2) + 1)[big].max() <= 2e-15
+
+
+@pytest.mark.parametrize("prec", ["kahan", "fp32"])
+def test_large_system_at_tiny_softening(prec):
+    """Above 24576 particles, where the adaptive path's grid has 100 bits."""
+    n, eps = 66000, 1e-12
+    s = ics.plummer_lognormal(n, seed=2)
+    rows = np.arange(0, n, 331)
+    ra, rp = oracle.forces_rows(s.pos, s.mass, eps, rows)
+    o = binding.make_opts(prec)
+    ws = binding.workspace(n, 1, o)
+    x, m = dev(s.pos), dev(s.mass)
+    acc, pot = torch.empty_like(x), torch.empty_like(m)
+    binding.nb_forces(x, m, eps, acc, pot, ws, o)
+    assert binding.nb_poll_status(ws, o) == binding.NB_OK
+    gate = 1e-5 if prec == "kahan" else 1e-4
+    assert rel_vec_err(host(acc)[rows], ra).max() <= gate
+    assert rel_err(host(pot)[rows], rp).max() <= gate
