@@ -62,8 +62,13 @@ extern "C" {
 /* ---- pair-loop precision policies ------------------------------------ */
 typedef enum {
     NB_PREC_FP32 = 0,   /* FP32 pairs, FP32 running sums                      */
-    NB_PREC_KAHAN = 1,  /* FP32 pairs, per-tile FP32 sums Kahan-added         */
-    NB_PREC_F64ACC = 2, /* FP32 pairs, per-tile FP32 sums added in FP64       */
+    NB_PREC_KAHAN = 1,  /* FP32 pairs, per-tile FP32 sums added to a
+                           compensated FP32 sum (a pair of floats)            */
+    NB_PREC_F64ACC = 2, /* FP32 pairs, per-tile FP32 sums added in FP64, or
+                           in three floats that keep more than its 53 bits.
+                           The VJP keeps this grade under every FP32-pair
+                           policy; on its symmetric path the row's own mass
+                           and cotangent enter as FP32, like its partners'    */
     NB_PREC_FP64 = 3    /* FP64 pairs and sums                                */
 } nb_precision;
 

@@ -463,6 +463,15 @@ __global__ void __launch_bounds__(128) wsym_jerk_fold_kernel(const Params p, con
 // fill less evenly (27 / 24 us at 2047).
 constexpr int64_t kJerkWideMinN = 12288;
 
+template <bool F64>
+int launch_jerk_pairs(Params &p, bool pot, cudaStream_t st) {
+    if (p.N >= kJerkWideMinN)
+        return pot ? launch_pairs<JerkPh<true, true>, F64>(p, st)
+                   : launch_pairs<JerkPh<true, false>, F64>(p, st);
+    return pot ? launch_pairs<JerkPh<false, true>, F64>(p, st)
+               : launch_pairs<JerkPh<false, false>, F64>(p, st);
+}
+
 int launch_jerk_wsym(const JerkJob &j, JerkParams q) {
     unsigned *mx = reinterpret_cast<unsigned *>(j.ws + j.L.status + kHeadMaxima);
     Params p{};
@@ -490,12 +499,8 @@ int launch_jerk_wsym(const JerkJob &j, JerkParams q) {
                             reinterpret_cast<float *>(j.ws + j.L.packA), mx, p.fx,
                             nc);
         if (rc) return rc;
-        if (j.N >= kJerkWideMinN)
-            rc = q.pot ? launch_pairs<JerkPh<true, true>>(p, j.stream)
-                       : launch_pairs<JerkPh<true, false>>(p, j.stream);
-        else
-            rc = q.pot ? launch_pairs<JerkPh<false, true>>(p, j.stream)
-                       : launch_pairs<JerkPh<false, false>>(p, j.stream);
+        rc = j.precision == NB_PREC_F64ACC ? launch_jerk_pairs<true>(p, q.pot != nullptr, j.stream)
+                                           : launch_jerk_pairs<false>(p, q.pot != nullptr, j.stream);
         if (rc) return rc;
         auto fold = q.pot ? wsym_jerk_fold_kernel<true> : wsym_jerk_fold_kernel<false>;
         rc = launch_pdl(fold, (unsigned)cdiv(j.N, 128), 128, 0, j.stream, p, q, mx);

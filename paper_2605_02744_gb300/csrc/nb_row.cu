@@ -18,9 +18,9 @@
 // broadcast in registers (dev::pair2: 18 packed FP32 operations per two hi/lo
 // pairs, 19 with the potential).  The lanes' sums of four rows are combined
 // with a reduce-scatter over the warp (16 shuffles for 16 values), the warps'
-// sums in shared memory as compensated float pairs in warp order.  So a sum
-// of plain FP32 adds covers N / 256 terms per lane and the tree over 64 of
-// them, and the rest keeps every rounding error.
+// sums in shared memory in FP64 (F64ACC) or as compensated float pairs.  So a
+// sum of plain FP32 adds covers N / 256 terms per lane and the tree over 64 of
+// them, and the rest is of the policy's own kind.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -143,7 +143,9 @@ __device__ __forceinline__ void row_group(const RowParams &p, int r0, int nr, in
     if (l % LPV == 0 && 4 * g + l / LPV < 4 * nr) part[4 * g + l / LPV] = sum;
 }
 
-template <bool SPLIT, bool POT, bool NEXT>
+// F64: the warps' sums are added in FP64 (F64ACC), else as a compensated float
+// pair.
+template <bool SPLIT, bool POT, bool NEXT, bool F64>
 __global__ void __launch_bounds__(NT, CPS) row_kernel(const RowParams p) {
     __shared__ float rows[6][kMaxRows];
     __shared__ float part[NW][kMaxRows * 4];  // [warp][row][component]
@@ -169,10 +171,18 @@ __global__ void __launch_bounds__(NT, CPS) row_kernel(const RowParams p) {
         const int c = v & 3;
         if (c == 3 && !POT) continue;
         const int64_t i = r0 + (v >> 2);
-        float2 t = f2(0.f, 0.f);
+        double sum;
+        if (F64) {
+            static_assert(NW == 4, "a tree over the warps");
+            sum = (fpconv::f2d(part[0][v]) + fpconv::f2d(part[1][v])) +
+                  (fpconv::f2d(part[2][v]) + fpconv::f2d(part[3][v]));
+        } else {
+            float2 t = f2(0.f, 0.f);
 #pragma unroll
-        for (int w2 = 0; w2 < NW; ++w2) two_add(t, part[w2][v]);
-        const double a = p.G * (fpconv::f2d(t.x) + fpconv::f2d(t.y));
+            for (int w2 = 0; w2 < NW; ++w2) two_add(t, part[w2][v]);
+            sum = fpconv::f2d(t.x) + fpconv::f2d(t.y);
+        }
+        const double a = p.G * sum;
         if (!fpconv::finite_d(a)) dev::set_status(p.status, kStatusNonFinite);
         if (c == 3) {
             p.pot[i] = -a;
@@ -194,11 +204,12 @@ __global__ void __launch_bounds__(NT, CPS) row_kernel(const RowParams p) {
     }
 }
 
-template <bool SPLIT>
+template <bool SPLIT, bool F64>
 int launch_row(const RowParams &p, bool next, cudaStream_t st) {
     const int64_t ctas = std::min<int64_t>(CPS * device_sm_count(), (p.N + 1) / 2);
-    auto k = next ? row_kernel<SPLIT, false, true>
-                  : (p.pot ? row_kernel<SPLIT, true, false> : row_kernel<SPLIT, false, false>);
+    auto k = next ? row_kernel<SPLIT, false, true, F64>
+                  : (p.pot ? row_kernel<SPLIT, true, false, F64>
+                           : row_kernel<SPLIT, false, false, F64>);
     return launch_pdl(k, (unsigned)ctas, NT, 0, st, p);
 }
 
@@ -263,8 +274,12 @@ RowParams params_of(const ForceJob &j) {
     return p;
 }
 
-int launch_split(const RowParams &p, bool split, bool next, cudaStream_t st) {
-    return split ? launch_row<true>(p, next, st) : launch_row<false>(p, next, st);
+int launch_rows(const ForceJob &j, const RowParams &p, bool next) {
+    if (j.precision == NB_PREC_F64ACC)
+        return j.split ? launch_row<true, true>(p, next, j.stream)
+                       : launch_row<false, true>(p, next, j.stream);
+    return j.split ? launch_row<true, false>(p, next, j.stream)
+                   : launch_row<false, false>(p, next, j.stream);
 }
 
 }  // namespace
@@ -276,7 +291,7 @@ int launch_force_row(const ForceJob &j) {
     p.vel = j.vel;
     p.kick = j.kick;
     const int rc = pack_rows(j, nullptr, 0.0, 0.0, false);
-    return rc ? rc : launch_split(p, j.split, false, j.stream);
+    return rc ? rc : launch_rows(j, p, false);
 }
 
 int launch_step_row(const ForceJob &j, double *vel, double dt, int64_t nsteps, bool acc_valid) {
@@ -297,7 +312,7 @@ int launch_step_row(const ForceJob &j, double *vel, double dt, int64_t nsteps, b
         p.pot = next ? nullptr : j.pot;
         p.vel = nsteps ? vel : nullptr;
         p.kick = e ? half : 0.0;
-        if ((rc = launch_split(p, j.split, next, j.stream))) return rc;
+        if ((rc = launch_rows(j, p, next))) return rc;
     }
     return NB_OK;
 }

@@ -789,14 +789,14 @@ int launch_vjp_wsym(const VjpJob &j, bool pb, bool fused) {
                         nc);
     if (rc) return rc;
     if (fused)
-        rc = j.split ? launch_pairs<VjpPh<false, true, true>>(p, j.stream)
-                     : launch_pairs<VjpPh<false, true, false>>(p, j.stream);
+        rc = j.split ? launch_pairs<VjpPh<false, true, true>, true>(p, j.stream)
+                     : launch_pairs<VjpPh<false, true, false>, true>(p, j.stream);
     else if (pb)
-        rc = j.split ? launch_pairs<VjpPh<true, false, true>>(p, j.stream)
-                     : launch_pairs<VjpPh<true, false, false>>(p, j.stream);
+        rc = j.split ? launch_pairs<VjpPh<true, false, true>, true>(p, j.stream)
+                     : launch_pairs<VjpPh<true, false, false>, true>(p, j.stream);
     else
-        rc = j.split ? launch_pairs<VjpPh<false, false, true>>(p, j.stream)
-                     : launch_pairs<VjpPh<false, false, false>>(p, j.stream);
+        rc = j.split ? launch_pairs<VjpPh<false, false, true>, true>(p, j.stream)
+                     : launch_pairs<VjpPh<false, false, false>, true>(p, j.stream);
     if (rc) return rc;
     VjpParams q{};
     q.G = j.G;

@@ -213,18 +213,21 @@ Params params_of(const ForceJob &j) {
 // size: 111.0 / 102.8 us at 16384, 1366 / 1295 us at 65536.
 constexpr int64_t kWideBlockMinN = 12288;
 
-template <bool POT>
+template <bool POT, bool F64>
 int launch_pair_shape(Params &p, bool split, cudaStream_t st) {
-    if (!split) return launch_pairs<ForcePh<false, 4, 16, false, POT>>(p, st);
-    return p.N >= kWideBlockMinN ? launch_pairs<ForcePh<false, 8, 8, true, POT>>(p, st)
-                                 : launch_pairs<ForcePh<false, 4, 12, true, POT>>(p, st);
+    if (!split) return launch_pairs<ForcePh<false, 4, 16, false, POT>, F64>(p, st);
+    return p.N >= kWideBlockMinN ? launch_pairs<ForcePh<false, 8, 8, true, POT>, F64>(p, st)
+                                 : launch_pairs<ForcePh<false, 4, 12, true, POT>, F64>(p, st);
 }
 
-int launch_pair_kernel(Params &p, bool split, bool pot, cudaStream_t st) {
-    kernel_timer_begin(st);
-    const int rc = pot ? launch_pair_shape<true>(p, split, st)
-                       : launch_pair_shape<false>(p, split, st);
-    kernel_timer_end(st);
+int launch_pair_kernel(const ForceJob &j, Params &p, bool pot) {
+    const bool f64 = j.precision == NB_PREC_F64ACC;
+    kernel_timer_begin(j.stream);
+    const int rc = pot ? (f64 ? launch_pair_shape<true, true>(p, j.split, j.stream)
+                              : launch_pair_shape<true, false>(p, j.split, j.stream))
+                       : (f64 ? launch_pair_shape<false, true>(p, j.split, j.stream)
+                              : launch_pair_shape<false, false>(p, j.split, j.stream));
+    kernel_timer_end(j.stream);
     return rc;
 }
 
@@ -251,7 +254,7 @@ int launch_force_wsym(const ForceJob &j) {
     Params p = params_of(j);
     int rc = launch_wsym_pack(j, nullptr, 0.0, 0.0);
     if (rc) return rc;
-    if ((rc = launch_pair_kernel(p, j.split, j.pot != nullptr, j.stream))) return rc;
+    if ((rc = launch_pair_kernel(j, p, j.pot != nullptr))) return rc;
     return launch_wsym_fold(j, p, j.pot, false, j.vel, j.kick, 0.0, 0.0);
 }
 
@@ -264,7 +267,7 @@ int launch_step_wsym(const ForceJob &j, double *vel, double dt, int64_t nsteps, 
     for (int64_t e = acc_valid ? 1 : 0; e <= nsteps; ++e) {
         const bool next = e < nsteps;
         double *pot = next ? nullptr : j.pot;
-        if ((rc = launch_pair_kernel(p, j.split, pot != nullptr, j.stream))) return rc;
+        if ((rc = launch_pair_kernel(j, p, pot != nullptr))) return rc;
         if ((rc = launch_wsym_fold(j, p, pot, next, nsteps ? vel : nullptr, e ? half : 0.0, half,
                                    dt)))
             return rc;

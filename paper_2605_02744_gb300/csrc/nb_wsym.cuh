@@ -28,13 +28,12 @@
 // sums (at most 256 terms) go into the particle's fixed-point totals
 // (nb_fixed.cuh, four limbs: integer atomics, exact, so results do not depend on the
 // order in which warps arrive).  The i-side register sums are folded every 4
-// j-sets (128 terms per stream) into a compensated float pair (TwoSum; the
-// FP32 policy drops the compensation) in shared memory, and at the end of the
+// j-sets (128 terms per stream) into a total of the policy's own kind (Total
+// below) in shared memory, and at the end of the
 // warp's segment of a row into the same totals.  The warps of a CTA own
 // consecutive ranges, so their last segments mostly belong to one row: these
-// are added up in the same compensated form across the CTA, in warp order,
-// before the atomics.  KAHAN and F64ACC share this arithmetic: it keeps what
-// either asks a running sum to keep.
+// are added up in the same form across the CTA, in warp order,
+// before the atomics.
 //
 // What bounds it: the register file.  A packed FMA with three distinct
 // operands reads six registers and issues at 64 % of the FP32 peak (two
@@ -175,14 +174,63 @@ __device__ __forceinline__ void poison(unsigned long long *top_limb) {
     atomicMax(reinterpret_cast<long long *>(top_limb), fx::kPoison);
 }
 
-// TwoSum (Knuth): s + c + x kept as an unevaluated pair; without `keep` (the
-// FP32 policy's plain running sums) the rounding error of the add is dropped.
-__device__ __forceinline__ float2 two_add(float2 t, float x, bool keep = true) {
-    const float s = __fadd_rn(t.x, x);
-    const float z = __fsub_rn(s, t.x);
-    const float e = __fadd_rn(__fsub_rn(t.x, __fsub_rn(s, z)), __fsub_rn(x, z));
-    return f2(s, keep ? __fadd_rn(t.y, e) : 0.f);
+// TwoSum (Knuth): a + b as a float and its exact rounding error.
+__device__ __forceinline__ float2 two_sum(float a, float b) {
+    const float s = __fadd_rn(a, b);
+    const float z = __fsub_rn(s, a);
+    return f2(s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, z)), __fsub_rn(b, z)));
 }
+// t + x as an unevaluated pair; without `keep` (the FP32 policy's plain running
+// sums) the rounding error of the add is dropped.
+__device__ __forceinline__ float2 two_add(float2 t, float x, bool keep = true) {
+    const float2 u = two_sum(t.x, x);
+    return f2(u.x, keep ? __fadd_rn(t.y, u.y) : 0.f);
+}
+
+// A row's running total of a component over a warp's segment and the warps of
+// a CTA.  KAHAN: a compensated float pair; FP32: a plain float (keep = false).
+template <bool F64>
+struct Total {
+    float2 v;
+    __device__ __forceinline__ void zero() { v = f2(0.f, 0.f); }
+    __device__ __forceinline__ void add(float x, bool keep) { v = two_add(v, x, keep); }
+    __device__ __forceinline__ void merge(const Total &o) { v = two_add(two_add(v, o.v.x), o.v.y); }
+    // the floats to add up; the low ones are zero for the first flushes of a row
+    template <class F>
+    __device__ __forceinline__ void parts(const F &f) const {
+        f(v.x);
+        if (v.y != 0.f) f(v.y);
+    }
+};
+// F64ACC and the VJP: three floats, s and c by TwoSum, so that only additions
+// into d round, 2^-48 below the total: more than the 53 bits of the FP64 sums
+// that they stand for, in 13 FP32 operations.  An FP64 add holds the pipe of
+// this part for as long as 64 of them.  Against a float pair for F64ACC too:
+// 433 us a step at 32768 with the pair, 444 in FP64, 434 so; acceleration +
+// jerk 779 / 863 / 779 us; VJP of 16384 195.0 / 200.2 / 198.4 us.
+template <>
+struct Total<true> {
+    float s, c, d;
+    __device__ __forceinline__ void zero() { s = c = d = 0.f; }
+    __device__ __forceinline__ void add(float x, bool = true) {
+        const float2 t = two_sum(s, x), u = two_sum(c, t.y);
+        s = t.x;
+        c = u.x;
+        d = __fadd_rn(d, u.y);
+    }
+    __device__ __forceinline__ void merge(const Total &o) {
+        const float2 t = two_sum(s, o.s), u = two_sum(c, o.c), v = two_sum(u.x, t.y);
+        s = t.x;
+        c = v.x;
+        d = __fadd_rn(d, __fadd_rn(o.d, __fadd_rn(u.y, v.y)));
+    }
+    template <class F>
+    __device__ __forceinline__ void parts(const F &f) const {
+        f(s);
+        if (c != 0.f) f(c);
+        if (d != 0.f) f(d);
+    }
+};
 
 // Geometry of a physics: K register groups per lane.  With IPAIR a group's .x
 // and .y are two i-slots and the lane has one j-particle, broadcast as (x, x);
@@ -281,13 +329,14 @@ __device__ __forceinline__ void load_j(const Params &p, int slot,
     }
 }
 
-template <class PH>
+template <class PH, bool F64>
 __global__ void __launch_bounds__(Geo<PH>::NTHR, 1) wsym_kernel(const Params p) {
     using GE = Geo<PH>;
     constexpr int NWARP = PH::WARPS, NTHR = GE::NTHR, NC = PH::NC, NV = GE::NV;
     constexpr int BW = GE::BW, JSET = GE::JSET, UPJ = GE::UPJ, UPI = GE::UPI;
     extern __shared__ __align__(16) unsigned char wsym_smem[];
-    float2 *tot = reinterpret_cast<float2 *>(wsym_smem);  // [NV][NTHR]
+    using Tot = Total<F64>;
+    Tot *tot = reinterpret_cast<Tot *>(wsym_smem);  // [NV][NTHR]
     __shared__ int sF[kMaxGroups];
     __shared__ int stag[NWARP];
     __shared__ float sFac[4];
@@ -350,12 +399,11 @@ __global__ void __launch_bounds__(Geo<PH>::NTHR, 1) wsym_kernel(const Params p) 
 #pragma unroll
             for (int e = 0; e < NC; ++e) {
                 if constexpr (PH::IPAIR) {
-                    float2 *t = tot + (2 * k * NC + e) * NTHR + tid, *t1 = t + NC * NTHR;
-                    *t = two_add(*t, S.a[k][e].x, p.keep);
-                    *t1 = two_add(*t1, S.a[k][e].y, p.keep);
+                    Tot *t = tot + (2 * k * NC + e) * NTHR + tid;
+                    t->add(S.a[k][e].x, p.keep);
+                    t[NC * NTHR].add(S.a[k][e].y, p.keep);
                 } else {
-                    float2 *t = tot + (k * NC + e) * NTHR + tid;
-                    *t = two_add(*t, S.a[k][e].x + S.a[k][e].y, p.keep);
+                    tot[(k * NC + e) * NTHR + tid].add(S.a[k][e].x + S.a[k][e].y, p.keep);
                 }
                 S.a[k][e] = f2(0.f, 0.f);
             }
@@ -374,9 +422,8 @@ __global__ void __launch_bounds__(Geo<PH>::NTHR, 1) wsym_kernel(const Params p) 
         if (lo) atomicAdd(wd, (unsigned long long)lo);
         if (hi) atomicAdd(wd + p.Np, (unsigned long long)hi);
     };
-    auto add_row = [&](int e, int slot, float2 t) {
-        add(e, slot, t.x, sF[PH::group(e)]);
-        add(e, slot, t.y, sF[PH::group(e)]);
+    auto add_row = [&](int e, int slot, const Tot &t) {
+        t.parts([&](float v) { add(e, slot, v, sF[PH::group(e)]); });
     };
     while (u < u_end) {
         const int r0 = (int)u & (UPJ - 1), s0 = r0 * GR;
@@ -397,7 +444,7 @@ __global__ void __launch_bounds__(Geo<PH>::NTHR, 1) wsym_kernel(const Params p) 
                 for (int e = 0; e < NC; ++e) S.a[k][e] = f2(0.f, 0.f);
             }
 #pragma unroll
-            for (int v = 0; v < NV; ++v) tot[v * NTHR + tid] = f2(0.f, 0.f);
+            for (int v = 0; v < NV; ++v) tot[v * NTHR + tid].zero();
             load_j<PH>(p, jb + ((l + s0) & 31), jn);
             open = true;
         }
@@ -448,20 +495,18 @@ __global__ void __launch_bounds__(Geo<PH>::NTHR, 1) wsym_kernel(const Params p) 
 #pragma unroll 1
     for (int v = tid; v < NV * 32; v += NTHR) {
         const int vk = v >> 5, lane = v & 31, e = vk % NC, k = vk / NC;
-        float2 t = f2(0.f, 0.f);
+        Tot t;
+        t.zero();
         int row = -1;
 #pragma unroll 1
         for (int w2 = 0; w2 <= NWARP; ++w2) {
             const int r = w2 < NWARP ? stag[w2] : -1;
             if (r != row) {
                 if (row >= 0) add_row(e, row * BW + 32 * k + lane, t);
-                t = f2(0.f, 0.f);
+                t.zero();
                 row = r;
             }
-            if (r >= 0) {
-                const float2 q = tot[vk * NTHR + 32 * w2 + lane];
-                t = two_add(two_add(t, q.x), q.y);
-            }
+            if (r >= 0) t.merge(tot[vk * NTHR + 32 * w2 + lane]);
         }
     }
     if (bad) dev::set_status(p.status, kStatusNonFinite);
@@ -509,11 +554,11 @@ __device__ __forceinline__ double take_fixed(const Params &p, int e, int64_t s, 
 }
 
 // One CTA per SM, every warp the same number of steps.
-template <class PH>
+template <class PH, bool F64>
 int launch_pairs(Params &p, cudaStream_t st) {
-    auto kern = wsym_kernel<PH>;
+    auto kern = wsym_kernel<PH, F64>;
     using GE = Geo<PH>;
-    constexpr size_t smem = (size_t)GE::NV * GE::NTHR * sizeof(float2);
+    constexpr size_t smem = (size_t)GE::NV * GE::NTHR * sizeof(Total<F64>);
     const int rc = smem_optin(reinterpret_cast<const void *>(kern), smem);
     if (rc != NB_OK) return rc;
     p.nb = cdiv(p.N, GE::BW);
