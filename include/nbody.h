@@ -119,7 +119,8 @@ typedef enum {
  * for 256 <= N <= 2^24, eps > 0 and FP32
  * pairs unless pairs is DIRECT or a launch shape or the hook is set.  Where
  * every pair takes the same displacement form (the VJP, the jerk, forces
- * below 32768 / 65536 particles), the totals have 174 instead of 100 bits:
+ * below 38912 particles without ADAPTIVE positions, and above where eps is
+ * below 1e-8 or above 1), the totals have 174 instead of 100 bits:
  * 224 B per particle of every single-system workspace up to 2^24.  Their
  * bounds are N max|m| times 0.385 / eps^2 (accelerations), 1 / eps
  * (potential) or 4 max|c or v| / eps^3 (VJP, jerk, from the cotangents or

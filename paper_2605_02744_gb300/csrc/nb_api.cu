@@ -782,7 +782,7 @@ static int step_single_direct(nb_state *s, double dt, int64_t nsteps, const nb_o
         if (nsteps == 0 && s->acc_valid) return NB_OK;
         return launch_step_wsym(j, s->vel, dt, nsteps, s->acc_valid != 0);
     }
-    if (j.sym && j.adaptive && j.precision != NB_PREC_FP64 && nsteps > 0)
+    if (j.sym && j.precision != NB_PREC_FP64 && s->eps > 0.0 && nsteps > 0)
         return launch_step_sym(j, s->vel, dt, nsteps, s->acc_valid != 0);
     if (j.row) {
         if (nsteps == 0 && s->acc_valid) return NB_OK;

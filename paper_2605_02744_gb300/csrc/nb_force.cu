@@ -523,7 +523,7 @@ int launch_force(const ForceJob &j) {
     if (j.sym && guard) return fail(NB_ERR_UNSUPPORTED, "symmetric pairs need eps > 0");
     if (takes_wsym(j)) return launch_force_wsym(j);
     if (j.row) return launch_force_row(j);
-    if (j.sym && adaptive) return launch_force_sym(j);
+    if (j.sym) return launch_force_sym(j);
     if (adaptive) {
         // boxes per 64 j-slots and per warp of i-slots (32 IR slots)
         const int tile_unit = 64;

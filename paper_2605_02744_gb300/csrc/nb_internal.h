@@ -271,9 +271,16 @@ constexpr int kWsymComponents = 7;  // sums per particle at most
 //    2^-58), but 2^-48 at 1e-17.  Below it direct pairs.
 constexpr double kSymMinEps = 1e-8;
 constexpr double kSym64MinEps = 1e-14;
-// Largest system of the warp-granular path (its accumulators take 2^19 adds,
-// one per block of 128 slots and range end); an explicit request for
-// symmetric pairs without the adaptive displacement goes direct above it.
+// Forces with one displacement form for every pair: from this size on the
+// adaptive path's kernel with 2048-slot blocks, below it the warp-granular one
+// (2048-slot blocks / warp-granular, us a step: FP32 420 / 413 at 36000, 513 /
+// 528 at 40960, 1288 / 1346 at 65536; F64ACC hi/lo 535 / 525, 654 / 674, 1624 /
+// 1704).
+constexpr int64_t kSymPlainMinN = 38912;
+// A softening above it, in whatever unit, stays with the warp-granular path,
+// which scales lengths: unscaled, r^-3 underflows FP32 beyond 4e12.
+constexpr double kSymPlainMaxEps = 1.0;
+// Largest system of FP64 pairs on the symmetric path.
 constexpr int64_t kWsymMaxN = 1 << 26;
 struct SymSizes {
     int64_t nb, T, U, ctas;  // row blocks, items, stream-K units, CTAs
@@ -302,7 +309,9 @@ int launch_step_sym(const ForceJob &job, double *vel, double dt, int64_t nsteps,
 // The warp-granular symmetric path (nb_wsym.cu; no adaptive displacement):
 // one evaluation, and an nb_step loop's evaluations with its O(N) work fused.
 inline bool takes_wsym(const ForceJob &j) {
-    return j.sym && !j.adaptive && j.eps > 0.0 && j.precision != NB_PREC_FP64 && j.N <= kWsymMaxN;
+    return j.sym && !j.adaptive && j.eps > 0.0 && j.precision != NB_PREC_FP64 &&
+           (j.N < kSymPlainMinN ||
+            ((j.eps < kSymMinEps || j.eps > kSymPlainMaxEps) && j.N <= kSymMaxN));
 }
 int launch_force_wsym(const ForceJob &job);
 int launch_step_wsym(const ForceJob &job, double *vel, double dt, int64_t nsteps, bool acc_valid);

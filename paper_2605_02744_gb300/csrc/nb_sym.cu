@@ -67,7 +67,13 @@
 // (x_j.hi - x_i.hi) + (x_j.lo - x_i.lo) only when the bounding boxes are
 // closer than gamma * max|x| (a 32-bit mask per warp and item, from the
 // Hilbert-sorted pack's boxes of 256 i- and 64 j-slots), single floats
-// elsewhere.  Systems with one form for every pair go to nb_wsym.cu.
+// elsewhere.  Systems with one form for every pair (single floats: MODE 0,
+// hi/lo: MODE 1) are not sorted; below kSymPlainMinN they go to nb_wsym.cu,
+// whose j-side sums are added to the totals per block of 128 or 256 slots
+// instead of 2048 -- finer ranges, but 8 to 16 times the atomics, which no
+// longer fit beside the arithmetic once the totals outgrow the L2 (MODE 0
+// here / there: 1288 / 1346 us a step at 65536, 5.21 / 5.74 ms at 131072,
+// 328 / 365 ms at 2^20).
 #include <cuda_runtime.h>
 
 #include <stdlib.h>
@@ -125,7 +131,8 @@ struct SymParams {
     int64_t U;          // stream-K units T * US (KBP j-sets of one item each)
     int64_t ctas;       // grid size of the pair kernel
     float eps2;
-    float gamma;        // adaptive threshold; the mode decides whether it is used
+    int mode;           // displacement: 0 single floats, 1 hi/lo, 2 adaptive
+    float gamma;        // adaptive threshold
     const float *jbox;  // per 64 slots: lo[3], hi[3], max|x|, pad
     const float *wbox;  // per 256 slots
     unsigned long long *acc_fx;  // [4 components][2 words][Np] fixed-point totals
@@ -154,11 +161,13 @@ __device__ __forceinline__ void load_jp(const SymParams &p, int64_t s, float (&j
 }
 
 // POT: the potential sums too (the caller wants phi).  The i-slots' lo parts
-// come from shared memory: only near j-sets use them, and 245 of 255
-// registers are taken.
-template <int POL, bool POT>
+// stay in registers for MODE 1 (every j-set is near) and come from shared
+// memory for MODE 2 (only near j-sets use them, and 245 of 255 registers are
+// taken).
+template <int POL, int MODE, bool POT>
 __global__ void __launch_bounds__(NT, CPS) force_sym_kernel(const SymParams p) {
     constexpr int NWJ = NW, IRJ = IRP, SNTJ = NT;
+    constexpr bool LOSM = MODE == 2;
     constexpr int HW = IRJ / 2;  // j-sets per warp i-set
     constexpr size_t kRedBytesJ = kRedBytes;
     extern __shared__ __align__(16) unsigned char smemj[];
@@ -166,7 +175,7 @@ __global__ void __launch_bounds__(NT, CPS) force_sym_kernel(const SymParams p) {
     Acc<POL> *tot = reinterpret_cast<Acc<POL> *>(smemj + kRedBytesJ);  // [IRJ * 4][SNTJ]
     constexpr bool MID = POL == NB_PREC_F64ACC;
     float *mid = reinterpret_cast<float *>(smemj + kRedBytesJ + 4 * IRJ * SNTJ * sizeof(Acc<POL>));
-    // (-x.lo, -x.lo) pairs [3][IRJ][SNTJ] after the F64ACC middle sums
+    // LOSM: (-x.lo, -x.lo) pairs [3][IRJ][SNTJ] after the F64ACC middle sums
     float2 *lo2 = reinterpret_cast<float2 *>(smemj + kRedBytesJ +
                                              4 * IRJ * SNTJ * sizeof(Acc<POL>) +
                                              (MID ? 4 * IRJ * SNTJ * sizeof(float) : 0)) +
@@ -203,9 +212,15 @@ __global__ void __launch_bounds__(NT, CPS) force_sym_kernel(const SymParams p) {
                 S.m[k] = f2(m, m);
                 const float xl = __ldg(p.soa + 4 * p.Np + sl), yl = __ldg(p.soa + 5 * p.Np + sl),
                             zl = __ldg(p.soa + 6 * p.Np + sl);
-                lo2[(0 * IRJ + k) * SNTJ] = f2(-xl, -xl);
-                lo2[(1 * IRJ + k) * SNTJ] = f2(-yl, -yl);
-                lo2[(2 * IRJ + k) * SNTJ] = f2(-zl, -zl);
+                if (LOSM) {
+                    lo2[(0 * IRJ + k) * SNTJ] = f2(-xl, -xl);
+                    lo2[(1 * IRJ + k) * SNTJ] = f2(-yl, -yl);
+                    lo2[(2 * IRJ + k) * SNTJ] = f2(-zl, -zl);
+                } else {
+                    S.nxl[k] = -xl;
+                    S.nyl[k] = -yl;
+                    S.nzl[k] = -zl;
+                }
                 S.ax[k] = S.ay[k] = S.az[k] = S.ph[k] = f2(0.f, 0.f);
             }
 #pragma unroll
@@ -217,13 +232,16 @@ __global__ void __launch_bounds__(NT, CPS) force_sym_kernel(const SymParams p) {
         }
         const bool sym = J != I;
         const int64_t jb = J * BI;
-        float wb[7], tb[7];
+        unsigned near = 0u;
+        if (MODE == 2) {
+            float wb[7], tb[7];
 #pragma unroll
-        for (int a = 0; a < 7; ++a) {
-            wb[a] = __ldg(p.wbox + (ib / (32 * IRJ)) * 8 + a);
-            tb[a] = __ldg(p.jbox + (jb / JSP + l) * 8 + a);
+            for (int a = 0; a < 7; ++a) {
+                wb[a] = __ldg(p.wbox + (ib / (32 * IRJ)) * 8 + a);
+                tb[a] = __ldg(p.jbox + (jb / JSP + l) * 8 + a);
+            }
+            near = __ballot_sync(0xffffffffu, boxes_near(wb, tb, p.gamma));
         }
-        const unsigned near = __ballot_sync(0xffffffffu, boxes_near(wb, tb, p.gamma));
         float jn[14];
         load_jp(p, jb + qa * JSP + l, jn);
         for (int q = qa; q < qb; ++q) {
@@ -234,13 +252,13 @@ __global__ void __launch_bounds__(NT, CPS) force_sym_kernel(const SymParams p) {
             const bool nq = (near >> q) & 1u;
             float4 b0, b1;
             if (sym) {
-                run_setj<IRJ, true, POT>(S, e2, jc, nq, b0, b1, -1, lo2, SNTJ);
+                run_setj<IRJ, MODE, true, POT, LOSM>(S, e2, jc, nq, b0, b1, -1, lo2, SNTJ);
                 float4 *r = red + (((half * KBP + (q % KBP)) * 2) * NWJ + w) * 32 + l;
                 r[0] = b0;
                 r[NWJ * 32] = b1;
             } else {
                 // the warp's own slots are j-sets HW w .. HW w + HW - 1 of the block
-                run_setj<IRJ, false, POT>(S, e2, jc, nq, b0, b1,
+                run_setj<IRJ, MODE, false, POT, LOSM>(S, e2, jc, nq, b0, b1,
                                           q / HW == w ? q % HW : -1, lo2, SNTJ);
             }
             if ((q + 1) % FLP == 0 || q + 1 == qb) {
@@ -367,9 +385,11 @@ __device__ __forceinline__ void store_box(float *out, const float (&lo)[3], cons
 // in place and the boxes of 64 and 256 slots (a block is 256 slots), as
 // sym_fold_kernel, kick_drift_pack_kernel, pack_sorted_kernel and two
 // slot_boxes_kernel launches do one after the other.  The acceleration is not
-// stored: the next fold replaces it before anything reads it.  At 65536
+// stored: the next fold replaces it before anything reads it.  Not SORTED
+// (MODE 0 and 1): particle order, no boxes.  At 65536
 // particles the ten launches of a step besides the pair kernel took 76 us
 // (ncu); now they are four, 28 us.
+template <bool SORTED>
 __global__ void __launch_bounds__(256) sym_fold_next_kernel(
     const SymParams p, int64_t N, const int *perm, double G, double *pos, double *vel, double kick,
     double next_kick, double drift, float *soa, float *jbox, float *wbox) {
@@ -388,7 +408,7 @@ __global__ void __launch_bounds__(256) sym_fold_next_kernel(
     int lo[3] = {ordered_f(3e38f), ordered_f(3e38f), ordered_f(3e38f)};
     int hi[3] = {ordered_f(-3e38f), ordered_f(-3e38f), ordered_f(-3e38f)};
     if (s < N) {
-        const int64_t i = perm[s];
+        const int64_t i = SORTED ? (int64_t)perm[s] : s;
         bool ok = true;
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
@@ -406,6 +426,7 @@ __global__ void __launch_bounds__(256) sym_fold_next_kernel(
         }
         if (!ok) dev::set_status(p.status, kStatusNonFinite);
     }
+    if (!SORTED) return;
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
         lo[c] = __reduce_min_sync(0xffffffffu, lo[c]);
@@ -509,7 +530,8 @@ __device__ __forceinline__ void item_of(int64_t t, int64_t nb, int64_t &I, int64
 
 // The near/far decisions the pair kernel will take on item t, by a warp: lane l
 // takes j-set l (unit l / 2); a unit's cost, on its even lane, is the maximum
-// over the warps of its two j-sets' sum.
+// over the warps of its two j-sets' sum (every one near or far unless the
+// mode is adaptive).
 __device__ __forceinline__ uint32_t unit_cost(const SymParams &p, int64_t t) {
     static_assert(NJSP == 32 && KBP == 2, "lane l: j-set l, unit l / 2");
     const int l = threadIdx.x & 31;
@@ -518,6 +540,7 @@ __device__ __forceinline__ uint32_t unit_cost(const SymParams &p, int64_t t) {
     const bool sym = I != J;
     const uint32_t cn = sym ? kCostSymNear : kCostDiagNear;
     const uint32_t cf = sym ? kCostSymFar : kCostDiagFar;
+    if (p.mode != 2) return (l & 1) ? 0u : 2 * (p.mode ? cn : cf) + kCostSymUnit;
     float tb[7];
 #pragma unroll
     for (int a = 0; a < 7; ++a) tb[a] = p.jbox[(J * NJSP + l) * 8 + a];
@@ -631,12 +654,12 @@ __global__ void __launch_bounds__(128) sym_ranges_kernel(const SymParams p,
     if (l == 0) lo[c] = a * US + off;
 }
 
-template <int POL, bool POT>
+template <int POL, int MODE, bool POT>
 int launch_pair(const SymParams &p, cudaStream_t st) {
-    auto kern = force_sym_kernel<POL, POT>;
+    auto kern = force_sym_kernel<POL, MODE, POT>;
     const size_t smem = kRedBytes + 4 * BI * sizeof(Acc<POL>) +
                         (POL == NB_PREC_F64ACC ? 4 * BI * sizeof(float) : 0) +
-                        3 * BI * sizeof(float2);
+                        (MODE == 2 ? 3 * BI * sizeof(float2) : 0);
     const int rc = smem_optin(reinterpret_cast<const void *>(kern), smem);
     if (rc != NB_OK) return rc;
     kernel_timer_begin(st);
@@ -674,16 +697,25 @@ int launch_fold(const SymParams &p, const ForceJob &j, const int *perm, double *
     return NB_OK;
 }
 
-template <int POL>
+template <int POL, int MODE>
 int launch_pair_pot(const SymParams &p, bool pot, cudaStream_t st) {
-    return pot ? launch_pair<POL, true>(p, st) : launch_pair<POL, false>(p, st);
+    return pot ? launch_pair<POL, MODE, true>(p, st) : launch_pair<POL, MODE, false>(p, st);
+}
+
+template <int POL>
+int launch_pair_mode(const SymParams &p, bool pot, cudaStream_t st) {
+    switch (p.mode) {
+        case 0: return launch_pair_pot<POL, 0>(p, pot, st);
+        case 1: return launch_pair_pot<POL, 1>(p, pot, st);
+        default: return launch_pair_pot<POL, 2>(p, pot, st);
+    }
 }
 
 int launch_pair_pol(const SymParams &p, int precision, bool pot, cudaStream_t st) {
     switch (precision) {
-        case NB_PREC_FP32: return launch_pair_pot<NB_PREC_FP32>(p, pot, st);
-        case NB_PREC_KAHAN: return launch_pair_pot<NB_PREC_KAHAN>(p, pot, st);
-        case NB_PREC_F64ACC: return launch_pair_pot<NB_PREC_F64ACC>(p, pot, st);
+        case NB_PREC_FP32: return launch_pair_mode<NB_PREC_FP32>(p, pot, st);
+        case NB_PREC_KAHAN: return launch_pair_mode<NB_PREC_KAHAN>(p, pot, st);
+        case NB_PREC_F64ACC: return launch_pair_mode<NB_PREC_F64ACC>(p, pot, st);
     }
     return fail(NB_ERR_INVALID, "unknown precision %d", precision);
 }
@@ -700,6 +732,7 @@ SymParams params_of(const ForceJob &j, const SymLayout &y) {
     p.ctas = z.ctas;
     const float ef = (float)j.eps;
     p.eps2 = ef * ef;
+    p.mode = j.adaptive ? 2 : (j.split ? 1 : 0);
     p.gamma = j.gamma;
     p.jbox = sort_tile_boxes(sb, j.L);
     p.wbox = sort_block_boxes(sb, j.L);
@@ -710,7 +743,12 @@ SymParams params_of(const ForceJob &j, const SymLayout &y) {
     return p;
 }
 
-int sorted_pack(const ForceJob &j, bool reuse_order) {
+// The pack of the current positions: in Hilbert order with its boxes, or (not
+// adaptive) in particle order.
+int pack_for(const SymParams &p, const ForceJob &j, bool reuse_order) {
+    if (p.mode != 2)
+        return launch_pack(j.pos, j.mass, j.N, j.L.Np,
+                           reinterpret_cast<float *>(j.ws + j.L.packA), nullptr, 0, j.stream);
     char *sb = j.ws + j.L.sortbuf;
     return launch_sorted_pack(j.pos, j.mass, j.N, j.L.Np, reinterpret_cast<float *>(j.ws + j.L.packA),
                               nullptr, 0, sort_perm(sb, j.L), sort_keys(sb), sort_box6(sb, j.L),
@@ -758,10 +796,11 @@ int launch_force_sym(const ForceJob &j) {
     NB_TRY_SYM(check_sym(j));
     const SymLayout y = sym_layout(j.ws, j.L);
     const SymParams p = params_of(j, y);
-    NB_TRY_SYM(sorted_pack(j, j.reuse_order));
+    NB_TRY_SYM(pack_for(p, j, j.reuse_order));
     NB_TRY_SYM(launch_split(p, j, y, true));
     NB_TRY_SYM(launch_pair_pol(p, j.precision, j.pot != nullptr, j.stream));
-    return launch_fold(p, j, sort_perm(j.ws + j.L.sortbuf, j.L), j.pot, j.vel, j.kick);
+    return launch_fold(p, j, p.mode == 2 ? sort_perm(j.ws + j.L.sortbuf, j.L) : nullptr, j.pot,
+                       j.vel, j.kick);
 }
 
 int launch_step_sym(const ForceJob &j, double *vel, double dt, int64_t nsteps, bool acc_valid) {
@@ -769,7 +808,8 @@ int launch_step_sym(const ForceJob &j, double *vel, double dt, int64_t nsteps, b
     const SymLayout y = sym_layout(j.ws, j.L);
     const SymParams p = params_of(j, y);
     char *sb = j.ws + j.L.sortbuf;
-    const int *perm = sort_perm(sb, j.L);
+    const bool sorted = p.mode == 2;
+    const int *perm = sorted ? sort_perm(sb, j.L) : nullptr;
     const double half = 0.5 * dt;
     const int64_t e0 = acc_valid ? 1 : 0;  // evaluation 0 primes a(x)
     int64_t sorted_at = -1;
@@ -781,17 +821,19 @@ int launch_step_sym(const ForceJob &j, double *vel, double dt, int64_t nsteps, b
         if (!packed) {
             const bool reuse = sorted_at >= 0 && e - sorted_at < kResortEvery;
             if (!reuse) sorted_at = e;
-            NB_TRY_SYM(sorted_pack(j, reuse));
+            NB_TRY_SYM(pack_for(p, j, reuse));
         }
         const bool last = e == nsteps;
         double *pot = last ? j.pot : nullptr;
-        NB_TRY_SYM(launch_split(p, j, y, e == e0));
+        // the ranges follow the boxes; without them they are the same all along
+        if (sorted || e == e0) NB_TRY_SYM(launch_split(p, j, y, e == e0));
         NB_TRY_SYM(launch_pair_pol(p, j.precision, pot != nullptr, j.stream));
         // the next evaluation keeps the order: its kick, drift and pack in the fold
-        packed = !last && e + 1 - sorted_at < kResortEvery;
+        packed = !last && (!sorted || e + 1 - sorted_at < kResortEvery);
         opened = packed;
+        auto next = sorted ? sym_fold_next_kernel<true> : sym_fold_next_kernel<false>;
         if (packed)
-            NB_TRY_SYM(launch_pdl(sym_fold_next_kernel, (unsigned)(p.Np / 256), 256, 0, j.stream, p,
+            NB_TRY_SYM(launch_pdl(next, (unsigned)(p.Np / 256), 256, 0, j.stream, p,
                                   j.N, perm, j.G, const_cast<double *>(j.pos), vel,
                                   e ? half : 0.0, half, dt,
                                   reinterpret_cast<float *>(j.ws + j.L.packA),

@@ -28,6 +28,7 @@ using dev::rsqrt_approx;
 template <int IRJ>
 struct ISetJ {
     float2 nx[IRJ], ny[IRJ], nz[IRJ];     // (-x_i.hi, -x_i.hi)
+    float nxl[IRJ], nyl[IRJ], nzl[IRJ];   // -x_i.lo
     float2 m[IRJ];                        // (m_i, m_i)
     float2 ax[IRJ], ay[IRJ], az[IRJ], ph[IRJ];  // per j-stream running sums
 };
@@ -47,9 +48,9 @@ __device__ __forceinline__ float2 lds_pair(const float2 *q) {
     return v;
 }
 
-// The i-slots' -x.lo values come as broadcast pairs from shared memory
-// (lo2[(c IRJ + k) stride]).
-template <int IRJ, bool NEAR, bool SYM, bool POT, bool SELF>
+// LOSM: the i-slots' -x.lo values come as broadcast pairs from shared
+// memory (lo2[(c IRJ + k) stride]) instead of registers.
+template <int IRJ, bool NEAR, bool SYM, bool POT, bool SELF, bool LOSM>
 __device__ __forceinline__ void stepj(ISetJ<IRJ> &S, const float2 e2, const float2 JX, const float2 JY,
                                       const float2 JZ, const float2 JM, const float2 JXL,
                                       const float2 JYL, const float2 JZL, float2 &BX, float2 &BY,
@@ -62,9 +63,15 @@ __device__ __forceinline__ void stepj(ISetJ<IRJ> &S, const float2 e2, const floa
         float2 dy = add2(JY, S.ny[k]);
         float2 dz = add2(JZ, S.nz[k]);
         if (NEAR) {
-            dx = add2(dx, add2(JXL, lds_pair(lo2 + (0 * IRJ + k) * stride)));
-            dy = add2(dy, add2(JYL, lds_pair(lo2 + (1 * IRJ + k) * stride)));
-            dz = add2(dz, add2(JZL, lds_pair(lo2 + (2 * IRJ + k) * stride)));
+            if (LOSM) {
+                dx = add2(dx, add2(JXL, lds_pair(lo2 + (0 * IRJ + k) * stride)));
+                dy = add2(dy, add2(JYL, lds_pair(lo2 + (1 * IRJ + k) * stride)));
+                dz = add2(dz, add2(JZL, lds_pair(lo2 + (2 * IRJ + k) * stride)));
+            } else {
+                dx = add2(dx, add2(JXL, f2(S.nxl[k], S.nxl[k])));
+                dy = add2(dy, add2(JYL, f2(S.nyl[k], S.nyl[k])));
+                dz = add2(dz, add2(JZL, f2(S.nzl[k], S.nzl[k])));
+            }
         }
         float2 r2 = fma2(dx, dx, e2);
         r2 = fma2(dy, dy, r2);
@@ -112,7 +119,7 @@ __device__ __forceinline__ float2 shfl2(float2 v, int src) {
 // 32 steps over one 64-slot j-set (j[0..6]: slot l, j[7..13]: slot 32 + l);
 // b0 / b1: the j-side sums (-a, phi order as BX, BY, BZ, BP) of the two
 // j-particles, home again on their lane.
-template <int IRJ, bool NEAR, bool SYM, bool POT>
+template <int IRJ, bool NEAR, bool SYM, bool POT, bool LOSM>
 __device__ __forceinline__ void rotate_setj(ISetJ<IRJ> &S, const float2 e2, const float (&j)[14],
                                             float4 &b0, float4 &b1, int self_h, const float2 *lo2,
                                             int stride) {
@@ -139,14 +146,14 @@ __device__ __forceinline__ void rotate_setj(ISetJ<IRJ> &S, const float2 e2, cons
     };
     int s0 = 0;
     if (self_h >= 0) {
-        stepj<IRJ, NEAR, SYM, POT, true>(S, e2, JX, JY, JZ, JM, JXL, JYL, JZL, BX, BY, BZ, BP,
+        stepj<IRJ, NEAR, SYM, POT, true, LOSM>(S, e2, JX, JY, JZ, JM, JXL, JYL, JZL, BX, BY, BZ, BP,
                                                self_h, lo2, stride);
         rotate();
         s0 = 1;
     }
 #pragma unroll 2
     for (int st = s0; st < 32; ++st) {
-        stepj<IRJ, NEAR, SYM, POT, false>(S, e2, JX, JY, JZ, JM, JXL, JYL, JZL, BX, BY, BZ, BP,
+        stepj<IRJ, NEAR, SYM, POT, false, LOSM>(S, e2, JX, JY, JZ, JM, JXL, JYL, JZL, BX, BY, BZ, BP,
                                                 -1, lo2, stride);
         rotate();
     }
@@ -154,14 +161,14 @@ __device__ __forceinline__ void rotate_setj(ISetJ<IRJ> &S, const float2 e2, cons
     b1 = make_float4(BX.y, BY.y, BZ.y, BP.y);
 }
 
-template <int IRJ, bool SYM, bool POT>
+template <int IRJ, int MODE, bool SYM, bool POT, bool LOSM>
 __device__ __forceinline__ void run_setj(ISetJ<IRJ> &S, const float2 e2, const float (&j)[14],
                                          bool near, float4 &b0, float4 &b1, int self_h,
                                          const float2 *lo2, int stride) {
-    if (near)
-        rotate_setj<IRJ, true, SYM, POT>(S, e2, j, b0, b1, self_h, lo2, stride);
+    if (MODE == 1 || (MODE == 2 && near))
+        rotate_setj<IRJ, true, SYM, POT, LOSM>(S, e2, j, b0, b1, self_h, lo2, stride);
     else
-        rotate_setj<IRJ, false, SYM, POT>(S, e2, j, b0, b1, self_h, lo2, stride);
+        rotate_setj<IRJ, false, SYM, POT, LOSM>(S, e2, j, b0, b1, self_h, lo2, stride);
 }
 
 // j-slots s (.x, j[0..6]) and s + 32 (.y, j[7..13]) of a packed SoA
