@@ -113,7 +113,8 @@ typedef enum {
  * N = 4800 unless a launch shape (nb_tune), NB_POS_ADAPTIVE or the
  * test_unissued_stage hook asks for the direct kernel; below that, under the
  * same conditions, a small-system kernel that evaluates every ordered pair;
- * for FP64 pairs, SYMMETRIC for 64 <= N <= 2^24 and eps >= 1e-14;
+ * for FP64 pairs, SYMMETRIC for 64 <= N <= 2^24 and eps >= 1e-14 (above
+ * 2^24 also when asked for they go DIRECT);
  * DIRECT otherwise.  nb_forces_vjp, the step adjoints and nb_forces_jerk /
  * nb_hermite4 take symmetric pairs (same combining)
  * for 256 <= N <= 2^24, eps > 0 and FP32

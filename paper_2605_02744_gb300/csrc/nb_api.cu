@@ -219,8 +219,7 @@ WsLayout ws_layout(int64_t N, int32_t B, const nb_opts *opts) {
     off = align256(off + 2 * (size_t)L.max_grid * (size_t)L.record_bytes_per_i);
     L.scratch = off;
     off = align256(off + kScratchBase + batched_scratch_bytes(B));
-    if (B == 1 && (N <= kSymMaxN ||
-                   (N <= kWsymMaxN && opts && opts->pairs == NB_PAIRS_SYMMETRIC))) {
+    if (B == 1 && N <= kSymMaxN) {
         L.wsym_fx = off;
         off = align256(off + 8 * fx::kLimbs * kWsymComponents * (size_t)L.Np);
     }

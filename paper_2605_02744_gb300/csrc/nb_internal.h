@@ -280,8 +280,11 @@ constexpr int64_t kSymPlainMinN = 38912;
 // A softening above it, in whatever unit, stays with the warp-granular path,
 // which scales lengths: unscaled, r^-3 underflows FP32 beyond 4e12.
 constexpr double kSymPlainMaxEps = 1.0;
-// Largest system of FP64 pairs on the symmetric path.
-constexpr int64_t kWsymMaxN = 1 << 26;
+// The warp-granular and the FP64 totals take 2^19 adds; they serve up to
+// kSymMaxN in blocks of at least 64 slots, i.e. 2^18 j-side adds and one to
+// three per warp that shares the row.
+constexpr int kMinBlockSlots = 64;
+static_assert(kSymMaxN / kMinBlockSlots <= 1 << 18, "adds per fixed-point total");
 struct SymSizes {
     int64_t nb, T, U, ctas;  // row blocks, items, stream-K units, CTAs
     size_t fx_bytes, cost_bytes;
@@ -319,7 +322,7 @@ int launch_step_wsym(const ForceJob &job, double *vel, double dt, int64_t nsteps
 // FP64 pairs, each unordered pair once (nb_sym64.cu): one evaluation, and an
 // nb_step loop's.
 inline bool takes_sym64(const ForceJob &j) {
-    return j.sym && j.eps > 0.0 && j.precision == NB_PREC_FP64 && j.N <= kWsymMaxN;
+    return j.sym && j.eps > 0.0 && j.precision == NB_PREC_FP64 && j.N <= kSymMaxN;
 }
 int launch_force_sym64(const ForceJob &job);
 int launch_step_sym64(const ForceJob &job, double *vel, double dt, int64_t nsteps, bool acc_valid);

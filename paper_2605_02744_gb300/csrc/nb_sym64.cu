@@ -31,6 +31,7 @@ using namespace wsym;
 
 constexpr int K = 2;                 // i-slots per lane
 constexpr int BW = 32 * K;           // slots per block
+static_assert(BW >= kMinBlockSlots, "adds per total");
 constexpr int WARPS = 8, NTHR = 32 * WARPS;
 constexpr int JPB = K;               // j-sets of 32 per block
 

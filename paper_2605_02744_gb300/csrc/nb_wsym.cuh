@@ -244,7 +244,7 @@ struct Geo {
     static constexpr int JPB = BW / JSET;                     // j-sets per block
     static constexpr int UPJ = 32 / GR, UPI = JPB * UPJ;      // scheduling units
     static constexpr int NV = SL * PH::NC, NTHR = 32 * PH::WARPS;
-    static_assert(2048 % BW == 0, "blocks tile the padded pack");
+    static_assert(2048 % BW == 0 && BW >= kMinBlockSlots, "blocks tile the padded pack");
 };
 
 // Zeroes the halves of v that pair a particle with itself: rotation step 0 of
