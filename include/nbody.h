@@ -122,7 +122,8 @@ typedef enum {
  * every pair takes the same displacement form (the VJP, the jerk, forces
  * below 38912 particles without ADAPTIVE positions, and above where eps is
  * below 1e-8 or above 1), the totals have 174 instead of 100 bits:
- * 224 B per particle of every single-system workspace up to 2^24.  Their
+ * 224 B per particle (up to 2^24 particles), which share their part of the
+ * workspace with the other paths' scratch.  Their
  * bounds are N max|m| times 0.385 / eps^2 (accelerations), 1 / eps
  * (potential) or 4 max|c or v| / eps^3 (VJP, jerk, from the cotangents or
  * velocities), N max|c| 0.67 / eps^2 for mass_bar; with FP32 pairs the grid

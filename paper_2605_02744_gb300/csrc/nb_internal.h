@@ -92,13 +92,15 @@ struct WsLayout {
     size_t counters;  // uint32 arrival counters, one per i-block (cleared by each call's pack)
     size_t packA;     // float SoA [7][Np]: x.hi y.hi z.hi m x.lo y.lo z.lo
     size_t packB;     // float SoA [4][Np]: VJP cotangents (cx, cy, cz, pbar/3)
+    size_t scratch;   // O(N) reduction scratch (energy partials, batched queue)
+    // one region: the four-limb totals, or the FP64 cotangents, the sort, the
+    // records and the two-word totals
+    size_t wsym_fx;   // warp-granular path: fixed-point totals, 7 components x 4 limbs per slot
     size_t cot64;     // double SoA [4][Np]: the same cotangents in FP64
     size_t sortbuf;   // Hilbert keys, permutation, tile/block boxes (adaptive path)
     size_t records;   // stream-K partial records
-    size_t scratch;   // O(N) reduction scratch (energy partials, batched queue)
     size_t sym_fx;    // symmetric-pair path: fixed-point totals, 64 B per slot
     size_t sym_cost;  // symmetric-pair path: item costs, their prefix, CTA ranges
-    size_t wsym_fx;   // warp-granular path: fixed-point totals, 7 components x 4 limbs per slot
     size_t bsym, bsym_bytes;  // batched symmetric-pair path (0 bytes: not provisioned)
     size_t sym_fx_bytes;      // 0 when the symmetric path is not provisioned
     size_t total;

@@ -29,3 +29,11 @@ def test_four_limb_totals_end_at_their_headroom(size, prec):
     kw = dict(precision=getattr(B, prec), pairs=B.NB_PAIRS_SYMMETRIC)
     n = 1 << 24
     assert size(n + 2048, **kw) < size(n, **kw)
+
+
+@pytest.mark.parametrize("n,mb", [(1024, 34.0), (16384, 57.0), (24576, 58.0), (65536, 64.0),
+                                  (1 << 20, 340.0), (1 << 24, 4600.0)])
+def test_totals_share_the_other_paths_scratch(size, n, mb):
+    """The 224 B a particle of the four-limb totals come out of what the sort, the
+    records and the two-word totals need anyway, as far as that goes."""
+    assert size(n) <= mb * 1e6
