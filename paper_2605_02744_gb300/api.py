@@ -23,6 +23,10 @@ def _resolve_tune(tune, kind, precision, n, autotune):
     return hit if hit is not None else autotune()
 
 
+def _force_kind(pairs) -> str:
+    return "force-direct" if pairs == "direct" else "force"
+
+
 def forces(pos, mass, eps: float, precision="f64acc", G: float = 1.0, with_pot: bool = True,
            tune=None, ws=None, stream=None, positions="default", pairs="default"):
     """(acc, pot) for one system; pos [N,3], mass [N] CUDA float64 tensors.
@@ -33,8 +37,8 @@ def forces(pos, mass, eps: float, precision="f64acc", G: float = 1.0, with_pot: 
     """
     if tune == "auto":
         from . import tune as T
-        tune = _resolve_tune(tune, "force", precision, mass.shape[0],
-                             lambda: T.autotune_forces(pos, mass, eps, precision))
+        tune = _resolve_tune(tune, _force_kind(pairs), precision, mass.shape[0],
+                             lambda: T.autotune_forces(pos, mass, eps, precision, pairs=pairs))
     opts = B.make_opts(precision, G, stream, tune=tune, positions=positions, pairs=pairs)
     n = mass.shape[0]
     acc = torch.empty((n, 3), dtype=torch.float64, device=pos.device)
@@ -97,9 +101,9 @@ class System:
         if tune == "auto":
             from . import tune as T
             if offsets is None:
-                tune = _resolve_tune(tune, "force", precision, n,
+                tune = _resolve_tune(tune, _force_kind(pairs), precision, n,
                                      lambda: T.autotune_forces(self.pos, self.mass, eps,
-                                                               precision))
+                                                               precision, pairs=pairs))
             else:
                 kind = "batched-" + T.batched_pairs(precision, pairs)
                 tune = _resolve_tune(tune, kind, precision, n,

@@ -1,7 +1,9 @@
 """Launch-shape autotuner with a JSON cache.
 
 For the single-system kernels a candidate is an nb_tune (threads, i-particles
-per thread, j-tile, bulk-copy stages, persistent CTAs per SM); for batches it
+per thread, j-tile, bulk-copy stages, persistent CTAs per SM), which names a
+shape of the direct kernel, or the empty one, which leaves the kernel to the
+library; for batches it
 is the work-item width in j-blocks (symmetric pairs, the default) or the
 thread-block-cluster size (direct pairs).  Every candidate this
 build compiled (``nb_tune_valid``) is timed on the caller's inputs with CUDA
@@ -52,7 +54,10 @@ def _bucket(n: int) -> int:
 
 def _key(kind: str, precision: str, n: int, device=None) -> str:
     props = torch.cuda.get_device_properties(device or torch.cuda.current_device())
-    return f"{props.name}|sm{props.major}{props.minor}|{kind}|{precision}|N{_bucket(n)}"
+    # "+": chosen with the untuned kernel among the candidates (entries without it
+    # force a direct shape on sizes that have a faster kernel, and are not read)
+    mark = "+" if kind.startswith("force") else ""
+    return f"{props.name}|sm{props.major}{props.minor}|{kind}{mark}|{precision}|N{_bucket(n)}"
 
 
 def _load() -> dict:
@@ -76,7 +81,8 @@ def _store(key: str, value: dict) -> None:
 
 
 def lookup(kind: str, precision: str, n: int):
-    """The cached tune for this device/kind/precision/size bucket, or None."""
+    """The cached tune for this device/kind/precision/size bucket, or None (an
+    empty dict is a choice: the library's own kernel)."""
     hit = _load().get(_key(kind, precision, n))
     return None if hit is None else hit["tune"]
 
@@ -109,20 +115,23 @@ def batched_pairs(precision: str, pairs: str = "default") -> str:
 
 
 def autotune_forces(pos, mass, eps: float, precision="kahan", reps: int = 5, warmup: int = 2,
-                    candidates=None, store: bool = True) -> dict:
+                    candidates=None, store: bool = True, pairs: str = "default") -> dict:
     """Time nb_forces for every compiled candidate; returns the best nb_tune dict.
 
-    The candidates are shapes of the direct (every ordered pair) kernel, which
-    is what is timed; the symmetric-pair path has one fixed shape.
+    The shapes are those of the direct (every ordered pair) kernel and are timed
+    on it; unless direct pairs are asked for, the empty tune is timed too, with
+    the kernel that the library takes by itself.  The result is cached under the
+    kind "force", or "force-direct" for direct pairs.
     """
+    direct = pairs == "direct"
     n = mass.shape[0]
     acc = torch.empty((n, 3), dtype=torch.float64, device=pos.device)
     pot = torch.empty(n, dtype=torch.float64, device=pos.device)
     results = []
-    for cand in candidates or FORCE_CANDIDATES:
+    for cand in candidates or ([] if direct else [{}]) + FORCE_CANDIDATES:
         if not B.nb_tune_valid(cand):
             continue
-        opts = B.make_opts(precision, tune=cand, pairs="direct")
+        opts = B.make_opts(precision, tune=cand, pairs="direct" if cand else pairs)
         ws = B.workspace(n, 1, opts, pos.device)
         run = lambda: B.nb_forces(pos, mass, eps, acc, pot, ws, opts)
         for _ in range(warmup):
@@ -132,7 +141,7 @@ def autotune_forces(pos, mass, eps: float, precision="kahan", reps: int = 5, war
     results.sort(key=lambda r: (r[0], r[1]))
     best = results[0]
     if store:
-        _store(_key("force", precision, n),
+        _store(_key("force-direct" if direct else "force", precision, n),
                {"tune": best[2], "ms": best[0],
                 "all": [{"tune": c, "ms": t} for t, _, c in results]})
     return best[2]
