@@ -458,10 +458,11 @@ __global__ void __launch_bounds__(128) wsym_jerk_fold_kernel(const Params p, con
 
 // From this size on a lane holds eight i-slots as four (x_a, x_b) pairs against
 // one j-particle instead of four broadcast i-slots against two j: half the
-// shuffles and half the adds to the totals per pair (802 / 862 us at 32768,
-// 12.3 / 13.4 ms at 131072), in blocks twice as wide, which smaller systems
-// fill less evenly (27 / 24 us at 2047).
-constexpr int64_t kJerkWideMinN = 12288;
+// shuffles and half the adds to the totals per pair, in blocks twice as wide,
+// which smaller systems fill less evenly (wide / narrow, KAHAN: 24.3 / 21.0 us
+// at 2047, 79.5 / 75.2 at 8192, 97.9 / 102.6 at 10000, 168.5 / 187.7 at 14336,
+// 779 / 876 at 32768; F64ACC the same within 2 %).
+constexpr int64_t kJerkWideMinN = 9216;
 
 template <bool F64>
 int launch_jerk_pairs(Params &p, bool pot, cudaStream_t st) {

@@ -14,9 +14,9 @@
 //
 // The reciprocal square root is the hardware's seed (rsqrt.approx.ftz.f64)
 // improved by one third-order Householder step, five FP64 operations, where
-// the library call took about eight.  GB300, 16384 particles: 10.75 ms (direct
-// pairs), 6.1 ms (earlier symmetric form), 5.0 ms now;
-// 2048: 1.35 ms -> 95 us; 20001: 25.1 -> 7.5 ms.
+// the library call took about eight.  GB300, one evaluation with potentials:
+// 16384 particles 10.78 ms (direct pairs) -> 5.42 ms, 2047: 1349 -> 99 us,
+// 24577: 16.16 (earlier symmetric form) -> 12.26 ms.
 #include <cuda_runtime.h>
 
 #include <algorithm>

@@ -205,12 +205,13 @@ Params params_of(const ForceJob &j) {
 }
 
 // Slots per lane and warps per SM.  With the hi/lo displacement eight slots a
-// lane (8 warps, 244 registers) amortise the shuffles best once there are
+// lane (8 warps, 240 registers) amortise the shuffles best once there are
 // enough steps for every warp; below, the smaller blocks of four slots (12
-// warps) start and finish faster: F64ACC evaluation 53.7 / 51.1 us at 8192,
-// 125.6 / 131.3 us at 16384 (eight / four).  Single-float displacements need
+// warps) start and finish faster (F64ACC evaluation, eight / four: 56.4 / 52.3
+// us at 8192, 67.5 / 64.6 at 10000, 89.3 / 90.9 at 12288, 109.2 / 116.0 at
+// 14336, 485 / 515 at 32768).  Single-float displacements need
 // fewer registers, and 16 warps of four slots hide more latency at every
-// size: 111.0 / 102.8 us at 16384, 1366 / 1295 us at 65536.
+// size: 111.0 / 102.8 us at 16384.
 constexpr int64_t kWideBlockMinN = 12288;
 
 template <bool POT, bool F64>

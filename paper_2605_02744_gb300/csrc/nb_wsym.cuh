@@ -35,15 +35,19 @@
 // are added up in the same form across the CTA, in warp order,
 // before the atomics.
 //
-// What bounds it: the register file.  A packed FMA with three distinct
+// What bounds it: in part the register file.  A packed FMA with three distinct
 // operands reads six registers and issues at 64 % of the FP32 peak (two
 // distinct: 95 %; measured on chains of independent operations), and 6 of a
-// force pair's 16, 17 of a jerk pair's 39 operations are of that kind: about
-// 80 % of the peak is the ceiling, and the pipe is busy 70 % of the time (ncu,
-// 16384 and 32768 particles), whatever the number of warps, the order of the
-// operations in the source or the unrolling.  GB300, 16384 particles, one
-// evaluation with its pack and fold: F64ACC forces 195 -> 123 us, acceleration
-// + jerk 945 -> 252 us, VJP 333 -> 200 us against the direct kernels.
+// force pair's 16, 17 of a jerk pair's 39 operations are of that kind, so that
+// 80 to 83 % of the peak is the ceiling of the mix: 88 us for the pairs of 16384
+// particles (hi/lo), which take 114.  Of the rest the ends are a part (pack, fold
+// and launches 6 us a step, each warp's first loads, a row's end); the pipe is
+// busy 70 % of the time within the kernel (ncu, 16384 and 32768 particles)
+// whatever the number of warps, the order of the operations in the source or
+// the unrolling, and what else keeps it from 80 % is not known.  GB300, 16384
+// particles, one evaluation with its pack and fold: F64ACC forces 194 -> 141
+// us, acceleration + jerk 945 -> 232 us, VJP 332 -> 198 us against the direct
+// kernels.
 #pragma once
 
 #include <cuda_runtime.h>
