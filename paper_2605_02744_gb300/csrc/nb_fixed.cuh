@@ -176,8 +176,9 @@ __host__ __device__ inline double value(unsigned long long word_hi, unsigned lon
 // The same with four signed limbs of 44 bits, X = sum L_q 2^(44 q), for the
 // warp-granular kernels: their VJP and jerk bounds grow with eps^-3, and 100
 // bits below them would be coarser than the FP32 pair terms once eps is below
-// ~1e-6 of the system size; 174 bits are not before ~1e-13 of it, where FP32
-// displacements have long run out.  A 24-bit significand touches one limb, or
+// ~1e-6 of the system size; 174 bits are not before ~1e-11 of it, and from there
+// the grid of the FP32-pair kernels no longer follows eps
+// (wsym::length_exponent).  A 24-bit significand touches one limb, or
 // two where it straddles a boundary, whatever its sign.  19 bits of headroom:
 // 2^19 adds per accumulator.
 constexpr int kLimbs = 4, kLimbBits = 44;

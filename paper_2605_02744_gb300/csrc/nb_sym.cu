@@ -60,7 +60,7 @@
 // N max|m| max(0.385 / eps^2, 1 / eps) on every partial and total (the
 // largest value of |d| (|d|^2 + eps^2)^-3/2 is 0.385 / eps^2 at
 // |d| = eps / sqrt 2).  The fold kernel reads each particle's accumulators
-// once (and zeroes them for the next call), applies G, scatters through the
+// once (and zeroes them for a loop's next evaluation), applies G, scatters through the
 // Hilbert permutation and optionally kicks the velocity.
 //
 // Displacements are adaptive: per (warp i-set, j-set) the hi/lo form

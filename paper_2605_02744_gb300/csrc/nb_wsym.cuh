@@ -40,9 +40,9 @@
 // distinct: 95 %; measured on chains of independent operations), and 6 of a
 // force pair's 16, 17 of a jerk pair's 39 operations are of that kind, so that
 // 80 to 83 % of the peak is the ceiling of the mix: 88 us for the pairs of 16384
-// particles (hi/lo), which take 114.  Of the rest the ends are a part (pack, fold
-// and launches 6 us a step, each warp's first loads, a row's end); the pipe is
-// busy 70 % of the time within the kernel (ncu, 16384 and 32768 particles)
+// particles (hi/lo), which take about 117.  Of the rest the ends are a part (each
+// warp's first loads, a row's end, the launch); the pipe is
+// busy 69 % of the time within the kernel (ncu, 16384 particles)
 // whatever the number of warps, the order of the operations in the source or
 // the unrolling, and what else keeps it from 80 % is not known.  GB300, 16384
 // particles, one evaluation with its pack and fold: F64ACC forces 194 -> 141
