@@ -217,11 +217,12 @@ WsLayout ws_layout(int64_t N, int32_t B, const nb_opts *opts) {
     off = align256(off + 16 * (size_t)L.Np);
     L.cot64 = off;
     off = align256(off + 32 * (size_t)L.Np);
-    // No call uses the four-limb totals together with the sort, the records,
-    // the two-word totals or the direct VJP's cotangents, and every call clears
-    // its own: they share one region (not the row kernel's second pack, which
-    // lies with the cotangents below kWsymMinN: a gradient's forward and
-    // backward steps would leave each other something to clear).
+    // No call uses the four-limb totals together with the sort, the records or
+    // the direct VJP's cotangents, and every call clears its own: they share one
+    // region (not the row kernel's second pack, which lies with the cotangents
+    // below kWsymMinN: a gradient's forward and backward steps would leave each
+    // other something to clear; and not the two-word totals, which are what an
+    // option that rules symmetric pairs out does without).
     L.wsym_fx = N >= kWsymMinN ? L.cot64 : off;
     const size_t wsym_end =
         B == 1 && N <= kSymMaxN
@@ -230,6 +231,7 @@ WsLayout ws_layout(int64_t N, int32_t B, const nb_opts *opts) {
     off = align256(off + sortbuf_bytes(L.Np));
     L.records = off;
     off = align256(off + 2 * (size_t)L.max_grid * (size_t)L.record_bytes_per_i);
+    off = std::max(off, wsym_end);
     if (sym_provisioned(opts, N, B)) {
         const SymSizes z = sym_sizes(L.Np);
         L.sym_fx = off;
@@ -238,7 +240,6 @@ WsLayout ws_layout(int64_t N, int32_t B, const nb_opts *opts) {
         L.sym_cost = off;
         off = align256(off + z.cost_bytes);
     }
-    off = std::max(off, wsym_end);
     if (bsym_wanted(opts, N, B)) {
         L.bsym = off;
         L.bsym_bytes = bsym_layout(N, B, bsym_item_blocks(opts)).bytes;

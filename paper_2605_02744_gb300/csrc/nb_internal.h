@@ -93,8 +93,8 @@ struct WsLayout {
     size_t packA;     // float SoA [7][Np]: x.hi y.hi z.hi m x.lo y.lo z.lo
     size_t packB;     // float SoA [4][Np]: VJP cotangents (cx, cy, cz, pbar/3)
     size_t scratch;   // O(N) reduction scratch (energy partials, batched queue)
-    // one region: the four-limb totals, or the FP64 cotangents, the sort, the
-    // records and the two-word totals
+    // one region: the four-limb totals, or the FP64 cotangents (from 4800
+    // particles), the sort and the records
     size_t wsym_fx;   // warp-granular path: fixed-point totals, 7 components x 4 limbs per slot
     size_t cot64;     // double SoA [4][Np]: the same cotangents in FP64
     size_t sortbuf;   // Hilbert keys, permutation, tile/block boxes (adaptive path)

@@ -32,8 +32,8 @@ def test_four_limb_totals_end_at_their_headroom(size, prec):
 
 
 @pytest.mark.parametrize("n,mb", [(1024, 34.0), (16384, 57.0), (24576, 58.0), (65536, 64.0),
-                                  (1 << 20, 340.0), (1 << 24, 4600.0)])
+                                  (1 << 20, 364.0), (1 << 24, 6000.0)])
 def test_totals_share_the_other_paths_scratch(size, n, mb):
-    """The 224 B a particle of the four-limb totals come out of what the sort, the
-    records and the two-word totals need anyway, as far as that goes."""
+    """The 224 B a particle of the four-limb totals come out of what the FP64
+    cotangents, the sort and the records need anyway, as far as that goes."""
     assert size(n) <= mb * 1e6
