@@ -214,7 +214,8 @@ inline size_t sortbuf_bytes(int64_t Np) {
 // redone from the current positions.
 // counters: ncounters arrival counters to clear (0: none).
 int launch_sorted_pack(const double *pos, const double *mass, int64_t N, int64_t Np, float *soa,
-                       uint32_t *counters, int64_t ncounters, int *perm, unsigned long long *keys, long long *box6, float *tile_boxes,
+                       uint32_t *counters, int64_t ncounters, int *perm,
+                       unsigned long long *keys, long long *box6, float *tile_boxes,
                        int tile_unit, float *block_boxes, int block_unit, bool reuse_order,
                        cudaStream_t st);
 

@@ -768,7 +768,6 @@ int launch_vjp_wsym(const VjpJob &j, bool pb, bool fused) {
     p.Np = j.L.Np;
     p.N = j.N;
     p.eps = (float)j.eps;
-    p.keep = true;
     p.fx = reinterpret_cast<unsigned long long *>(j.ws + j.L.wsym_fx);
     p.fxe = reinterpret_cast<int *>(j.ws + j.L.status + kHeadExponents);
     p.mx = mx;

@@ -82,7 +82,7 @@ struct Params {
     int64_t nb;          // blocks
     int64_t per_warp, extra;  // scheduling units per warp; the first `extra` warps take one more
     float eps;
-    bool keep;           // compensated i-side sums (every policy but FP32)
+    bool keep;           // KAHAN: compensated i-side sums; FP32: plain ones
     unsigned long long *fx;  // [components][4 limbs][Np] fixed-point totals
     int *fxe;                // [kMaxGroups] the call's exponents (written here)
     const unsigned *mx;      // maxima of the inputs (float bits), see MaxWord
